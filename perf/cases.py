@@ -90,7 +90,7 @@ def _draw_spin(rng, n_lo, n_hi, do, **more):
         ly = rng.choice([1, 1, 2, 3, 4, 5])
         lx = int(round(rng.randint(n_lo, n_hi) / ly))
         n = lx * ly
-        if lx < 2 or not n_lo <= n <= n_hi or n - (lx // 2) * ly > 16:
+        if lx < 2 or not n_lo <= n <= n_hi:
             continue
         j2 = rng.choice([0.0, 0.25, 0.5, 0.3, 0.41])
         return _spin(None, lx, ly, j2, max(1, n // 2 - rng.choice([0, 0, 0, 1, 2, 3])), do, **more)
@@ -113,7 +113,9 @@ def _draw_hub(rng, n_lo, n_hi, do, **more):
 
 def _model(case, seed=0):
     if case["model"] == "spin":
-        m = wl.j1j2_torus(case["lx"], case["ly"], 1.0, case["j2"], case["n_up"])
+        # side A: the first half of the sites (the cut of the repository's configurations)
+        half = (1 << (case["lx"] * case["ly"] // 2)) - 1
+        m = wl.j1j2_torus(case["lx"], case["ly"], 1.0, case["j2"], case["n_up"], cut_mask=half)
         if case["kind"] == "ground":
             # a point of an anisotropy scan: the energy is another one for another seed
             m.jz = m.jz * (1.0 + (37 * int(seed) % 32) / 64.0)
