@@ -14,8 +14,8 @@
 //   C64   fixed-point class sums weighted in FP64 (value ranges too wide
 //         for 64-bit integer weights).
 // Row pass (k_row5): the diagonal, the H_B (column-mixing) term and the
-// cross-cut terms of whole rows.  psi_s[a,:] is staged in shared memory by
-// bulk TMA copies, then each column b sums, class by class, its H_B
+// cross-cut terms of whole rows.  A few rows psi_s[a,:] are staged in shared
+// memory, then each column b sums, class by class, its H_B
 // neighbours (16-bit column indices) and the cross-cut gathers from x in
 // global memory, plus the diagonal.
 // Panel pass: the H_A (row-mixing) term over column panels that stay
@@ -60,329 +60,259 @@ __global__ void k_to_fixed(const double* __restrict__ x, long long* __restrict__
     X[i] = to_fixed(x[i], sh);
 }
 
-constexpr int kRowThreads = 512;
-// valid-bond lists for the cross terms also for 4-byte types (off: the
-// four-row FP32 pass measured slower with them, 17.2 vs 15.5 ms)
-constexpr bool kListsF32 = false;
+// R rows of the staged group at one column: one 16-byte shared-memory access
+template <class S, int R>
+struct alignas(16) RowVec {
+  S v[R];
+};
 
-// Row pass: work unit = R consecutive rows of one block ("row group"),
-// brought into shared memory by bulk TMA copies; one 1024-thread CTA per SM
-// whose R staged rows (4 for 4-byte, 2 for 8-byte types) share every B-side
-// load.  Per column b:
-//  * H_B: the class segments of the column's index list are padded to
-//    groups of four 16-bit indices, read with one 8-byte load per group
-//    (several groups loaded ahead) and gathered from all R staged rows
-//    (padding points at a zero slot);
-//  * cross terms: one B-side map load per B cross site, shared by the R
-//    rows, then one gather per valid bond from the neighbouring block (8-byte
-//    types: from per-row lists of the valid bonds for each column bit and
-//    value class, summed per class and weighted once per column);
+__device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// *p under the predicate, else zero.  8-byte types: a predicated load, without
+// a branch (row pass of J1-J2 4x8: 17.0 -> 15.8 ms); FP32, with twice the rows
+// per bond, is faster as the compiler schedules it (9.2 against 9.6 ms)
+__device__ __forceinline__ long long ldg_if(const long long* p, bool on) {
+  long long v = 0;
+  asm("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q ld.global.nc.b64 %0, [%1]; }" : "+l"(v) : "l"(p), "r"((unsigned)on));
+  return v;
+}
+__device__ __forceinline__ double ldg_if(const double* p, bool on) {
+  return __longlong_as_double(ldg_if(reinterpret_cast<const long long*>(p), on));
+}
+__device__ __forceinline__ float ldg_if(const float* p, bool on) { return on ? __ldg(p) : 0.f; }
+
+// Row pass: work unit = R consecutive rows of one block ("row group", R = 16
+// bytes / element), staged in shared memory with the R rows of a column side
+// by side, so that one 16-byte access serves R matrix elements and every
+// B-side index, map and diagonal load is shared by the R rows.  A warp takes
+// 32 columns (one slab) at a time:
+//  * H_B: the slab's pair rows (Dev3::B_pair) are read with one coalesced
+//    4-byte load per lane, four rows a step and a step ahead of their use;
+//    the slab's row counts are the same for all lanes, so the loops neither
+//    diverge nor run past the slab's longest list;
+//  * cross terms: per octet of cross-bond sites one 16-byte load brings a
+//    column's eight maps, one word its 32 bond bits; each present slot
+//    gathers the R source rows under the predicate that the bond flips, all
+//    gathers of a site before their sums, one weight per value class and
+//    column;
 //  * the diagonal from per-row constants and popcounts of packed words.
-template <class Pol, int R, int NT = kRowThreads, int MINB = 2>
-__global__ void __launch_bounds__(NT, MINB)
+// Bound: the L1 / shared-memory data path (74 % of its wavefronts on the 4x4
+// Hubbard torus, 64 % with cross terms), then issue (60 %).  A 16-byte access
+// takes four wavefronts at best; the lists are ordered so that it takes 4.06
+// (order_lists).  Measured, FP64 fixed point / FP32: J1-J2 4x8 (601 M states)
+// 22.9 -> 15.6 / 14.3 -> 9.2 ms, Hubbard 4x4 (166 M states) 2.75 -> 1.63 /
+// 1.48 -> 0.92 ms, against lists of 8-byte groups per column, scattered over the
+// lanes and padded to 16 entries.  The digit-split dense products on the
+// tensor cores that could take the terms inside a group of sites would cost
+// about 28 instructions per state and group for the split and the
+// recombination, as much as the gathers they replace.
+template <class Pol, int R, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT)
     k_row5(P3 p, const long long* __restrict__ grp_start, long long n_groups, const typename Pol::S* __restrict__ x,
-           typename Pol::Y* __restrict__ y, const int* __restrict__ emax, long long stage_elems, int* err) {
+           typename Pol::Y* __restrict__ y, const int* __restrict__ emax) {
   using S = typename Pol::S;
+  using V = RowVec<S, R>;
+  static_assert(sizeof(V) == 16, "one 16-byte word per column");
   extern __shared__ __align__(16) unsigned char smem5[];
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem5);
-  S* bufs = reinterpret_cast<S*>(smem5 + 128);
-  __shared__ const S* src_row[R][32];  // per row, per A cross site
-  // per row, B cross site, value beta of the column's bit at that site and
-  // value class (of at most two): the site's bonds that are valid there
-  // (their A bit differs from beta), as source-row lists of at most kXL
-  // entries; a column sums each class's gathers and multiplies once
-  constexpr int kXL = 2;
-  __shared__ const S* xl_ptr[R][32][2][2][kXL];
-  __shared__ unsigned char xl_n[R][32][2][2];
-  __shared__ int xl_mx[32][2];  // per B cross site and class: longest list over rows and beta
-  constexpr bool kLists = sizeof(S) == 8 || kListsF32;
-  __shared__ int s_pad[R];
-  constexpr int V = 16 / (int)sizeof(S);
+  V* const xs = reinterpret_cast<V*>(smem5);
+  // source row of each (slot or bond, row), null where there is none; the
+  // A-side bits of the slots and the mask of slots with a source row
+  __shared__ __align__(16) const S* s_ptr[kMaxOct][32][R];
+  __shared__ unsigned s_ax[kMaxOct][R], s_vm[kMaxOct][R];
   const Dev3& t = p.t;
-  if (threadIdx.x == 0) {
-    bar_init(&bar[0]);
-    bar_fence_init();
-  }
-  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int e2 = emax ? out_exp(t, emax) : 0;
-  unsigned phase = 0;
+  const int n_oct = p.ncross ? (t.xs_ok ? t.n_oct : 1) : 0;
   for (long long g = blockIdx.x; g < n_groups; g += gridDim.x) {
     const int bi = find_blk(grp_start, p.nblk, g);
     const DevBlock bl = p.blocks[bi];
     const long long a0 = (g - grp_start[bi]) * R;
     const int nr = (int)min((long long)R, bl.dA - a0);
     const int dB = (int)bl.dB;
-    if (threadIdx.x == 0) {
-      proxy_fence();
-      unsigned bytes = 0;
-      for (int r = 0; r < nr; ++r) {
-        const long long g0 = bl.off + (a0 + r) * dB;
-        const long long gal = (g0 + V - 1) / V * V, galend = (g0 + dB) / V * V;
-        if (galend > gal) bytes += (unsigned)((galend - gal) * (long long)sizeof(S));
+    const long long row0 = bl.off + a0 * dB;
+    __syncthreads();  // the previous group's columns are done
+    {
+      const S* r0 = x + row0;
+#pragma unroll 4
+      for (int b = threadIdx.x; b < dB; b += NT) {
+        V w;
+#pragma unroll
+        for (int r = 0; r < R; ++r) w.v[r] = r < nr ? r0[(long long)r * dB + b] : (S)0;
+        xs[b] = w;
       }
-      if (bytes) {
-        bar_expect(&bar[0], bytes);
-        for (int r = 0; r < nr; ++r) {
-          const long long g0 = bl.off + (a0 + r) * dB;
-          const long long gal = (g0 + V - 1) / V * V, galend = (g0 + dB) / V * V;
-          if (galend > gal)
-            bulk_g2s(bufs + r * stage_elems + (g0 % V) + (gal - g0), x + gal,
-                     (unsigned)((galend - gal) * (long long)sizeof(S)), &bar[0]);
-        }
-      } else {
-        bar_arrive(&bar[0]);
+      if (threadIdx.x < 8) {  // zero slots addressed by the padding indices, one per bank group
+        V w;
+#pragma unroll
+        for (int r = 0; r < R; ++r) w.v[r] = 0;
+        xs[dB + threadIdx.x] = w;
       }
     }
-    for (int r = 0; r < nr; ++r) {
-      const long long g0 = bl.off + (a0 + r) * dB;
-      const long long gend = g0 + dB;
-      const long long gal = (g0 + V - 1) / V * V, galend = gend / V * V;
-      const int pad = (int)(g0 % V);
-      S* buf = bufs + r * stage_elems;
-      if (threadIdx.x == 0) {
-        s_pad[r] = pad;
-        buf[pad + dB] = (S)0;  // zero slot addressed by the padding indices
-      }
-      if (galend > gal) {
-        for (long long q = g0 + threadIdx.x; q < gal; q += blockDim.x) buf[pad + (q - g0)] = x[q];
-        for (long long q = galend + threadIdx.x; q < gend; q += blockDim.x) buf[pad + (q - g0)] = x[q];
-      } else {
-        for (long long q = g0 + threadIdx.x; q < gend; q += blockDim.x) buf[pad + (q - g0)] = x[q];
-      }
-    }
-    // neighbouring-block source row of each (row, A cross site)
-    if (threadIdx.x < 32 * R) {
-      const int r = threadIdx.x >> 5, ia = threadIdx.x & 31;
+    // one warp per (octet, row): lane = slot (or bond, without slots)
+    for (int q = warp; q < n_oct * R; q += NT / 32) {
+      const int h = q / R, r = q % R;
+      const int k = t.xs_ok ? t.xs_k[32 * h + lane] : (lane < p.ncross ? lane : 255);
       const S* sp = nullptr;
-      if (r < nr && ia < 32 && p.ncross) {
-        const long long gA = bl.gA0 + a0 + r;
-        // which bond touches site ia: any bond k with bond_ia[k] == ia gives its A bit
-        int k = -1;
-        for (int q = 0; q < p.ncross; ++q)
-          if (t.bond_ia[q] == ia) { k = q; break; }
-        if (k >= 0) {
-          const unsigned pa = t.A_pack[gA];
-          const int sb = ((pa >> k) & 1u) ? bl.nbr_lo : bl.nbr_hi;
-          if (sb >= 0) {
-            const DevBlock so = p.blocks[sb];
-            const unsigned rr = t.mapA[(long long)ia * t.A_total + gA];
-            if (rr != 0xFFFFu) sp = x + so.off + (long long)rr * so.dB;
-          }
+      const long long gA = bl.gA0 + a0 + r;
+      if (r < nr && k != 255) {
+        const int sb = ((t.A_pack[gA] >> k) & 1u) ? bl.nbr_lo : bl.nbr_hi;
+        if (sb >= 0) {
+          const DevBlock& so = p.blocks[sb];
+          const unsigned rr = t.mapA[(long long)t.bond_ia[k] * t.A_total + gA];
+          if (rr != 0xFFFFu) sp = x + so.off + (long long)rr * so.dB;
         }
       }
-      src_row[r][ia] = sp;
-    }
-    if (kLists && p.ncross && t.xl_ok) {
-      __syncthreads();  // src_row complete
-      if (threadIdx.x < 64) xl_mx[threadIdx.x >> 1][threadIdx.x & 1] = 0;
-      __syncthreads();
-      if (threadIdx.x < R * 64) {
-        const int r = threadIdx.x >> 6, ib = (threadIdx.x >> 1) & 31, beta = threadIdx.x & 1;
-        int n0 = 0, n1 = 0;
-        if (ib < t.n_ib && r < nr) {
-          const unsigned par = t.A_pack[bl.gA0 + a0 + r];
-          unsigned km = t.ib_mask[ib];
-          while (km) {
-            const int k = __ffs(km) - 1;
-            km &= km - 1;
-            const S* sp = src_row[r][t.bond_ia[k]];
-            if ((((par >> k) & 1u) != (unsigned)beta) && sp) {  // at most kXL per class (xl_ok)
-              if ((t.xl_c1_mask >> k) & 1u) {
-                if (n1 < kXL) xl_ptr[r][ib][beta][1][n1++] = sp;
-              } else {
-                if (n0 < kXL) xl_ptr[r][ib][beta][0][n0++] = sp;
-              }
-            }
-          }
-        }
-        xl_n[r][ib][beta][0] = (unsigned char)n0;
-        xl_n[r][ib][beta][1] = (unsigned char)n1;
-        atomicMax(&xl_mx[ib][0], n0);
-        atomicMax(&xl_mx[ib][1], n1);
+      s_ptr[h][lane][r] = sp;
+      const unsigned vm = __ballot_sync(0xffffffffu, sp != nullptr);
+      if (lane == 0) {
+        s_vm[h][r] = vm;
+        s_ax[h][r] = r < nr ? (t.xs_ok ? t.A_xs[h * t.A_total + gA] : t.A_pack[gA]) : 0u;
       }
     }
-    const bool ok = bar_wait(&bar[0], phase);
-    if (__syncthreads_or(!ok)) {
-      if (threadIdx.x == 0) atomicExch(err, 1);
-      bar_wait(&bar[0], phase);
-      return;
+    // the next group's rows on their way into L2 while this one is summed
+    if (threadIdx.x == 0 && g + gridDim.x < n_groups) {
+      const long long gn = g + gridDim.x;
+      const int bn = find_blk(grp_start, p.nblk, gn);
+      const DevBlock& nb = p.blocks[bn];
+      const long long an = (gn - grp_start[bn]) * R;
+      const char* p0 = reinterpret_cast<const char*>(x + nb.off + an * nb.dB);
+      const char* p1 = p0 + (size_t)(min((long long)R, nb.dA - an) * nb.dB) * sizeof(S);
+      const char* q0 = reinterpret_cast<const char*>(((uintptr_t)p0 + 15) & ~(uintptr_t)15);
+      const char* q1 = reinterpret_cast<const char*>((uintptr_t)p1 & ~(uintptr_t)15);
+      if (q1 > q0) l2_prefetch(q0, (unsigned)(q1 - q0));
     }
-    phase ^= 1;
     unsigned pa[R];
-    const S* xs[R];
     typename Pol::D da[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const int rr = r < nr ? r : 0;
-      const long long gA = bl.gA0 + a0 + rr;
+      const long long gA = bl.gA0 + a0 + (r < nr ? r : 0);
       pa[r] = t.A_pack[gA];
-      xs[r] = bufs + rr * stage_elems + s_pad[rr];
       da[r] = Pol::diagA(t, gA);
     }
     const bool final_ = !bl.has_hA && !p.keep_fixed;
-    const long long gB0 = bl.gB0;
-    for (int b = threadIdx.x; b < dB; b += blockDim.x) {
-      const long long gB = gB0 + b;
-      const uint2 m = t.B_meta4[gB];
-      const unsigned pb = t.B_pack[gB];
-      const typename Pol::D dbv = Pol::diagB(t, gB);
-      typename Pol::A acc[R];
+    __syncthreads();
+    const int nslab = (dB + 31) >> 5;
+    for (int sl = warp; sl < nslab; sl += NT / 32) {
+      const int b = 32 * sl + lane;
+      const bool in = b < dB;
+      const long long gB = bl.gB0 + (in ? b : dB - 1);
+      const uint2 m = t.B_slab[bl.slabB0 + sl];
+      const unsigned* cp = t.B_pair + (size_t)m.x * 32 + lane;
+      unsigned qn[4];
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const unsigned z = t.vab_and ? (pa[r] & pb) : (pa[r] ^ pb);
-        acc[r] = Pol::dmul(da[r] + dbv + Pol::vab(t, z), xs[r][b]);
+      for (int u = 0; u < 4; ++u) qn[u] = __ldg(cp + 32 * u);
+      const unsigned pb = t.B_pack[gB];
+      uint4 mv = make_uint4(0u, 0u, 0u, 0u);
+      unsigned bx = 0u;
+      if (n_oct && t.xs_ok) {
+        mv = __ldg(t.B_xmap + gB);
+        bx = __ldg(t.B_xs + gB);
       }
-      const uint2* cp = t.B_col4 + m.x;
-      // index groups in flight per class step (measured best: 4 for 8-byte
-      // types, 2 for 4-byte types, whose four rows per pass need registers)
-      constexpr int HBU = sizeof(S) == 8 ? 4 : 2;
-      const unsigned zz = (unsigned)dB | ((unsigned)dB << 16);  // four zero-slot indices
+      typename Pol::A acc[R];
+      {
+        const typename Pol::D dbv = Pol::diagB(t, gB);
+        const V xb = xs[in ? b : dB];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const unsigned z = t.vab_and ? (pa[r] & pb) : (pa[r] ^ pb);
+          acc[r] = Pol::dmul(da[r] + dbv + Pol::vab(t, z), xb.v[r]);
+        }
+      }
 #pragma unroll
       for (int c = 0; c < kMaxCls; ++c) {
-        const unsigned n4 = (m.y >> (8 * c)) & 255u;
-        if (!n4) continue;
+        const int n = (int)((m.y >> (8 * c)) & 255u);
+        if (!n) continue;
         S sum[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) sum[r] = 0;
-        // HBU index groups are loaded before any is used, so their L2
-        // latencies overlap; groups past the class end read the zero slot
-        for (unsigned i = 0; i < n4; i += HBU) {
-          uint2 q[HBU];
+        auto add_pair = [&](unsigned q) {
+          const V v0 = xs[q & 0xFFFFu], v1 = xs[q >> 16];
 #pragma unroll
-          for (int u = 0; u < HBU; ++u) q[u] = i + u < n4 ? __ldg(cp + i + u) : make_uint2(zz, zz);
+          for (int r = 0; r < R; ++r) sum[r] += v0.v[r] + v1.v[r];
+        };
+        int i = n;
+        for (; i >= 4; i -= 4) {
+          unsigned q[4];
 #pragma unroll
-          for (int u = 0; u < HBU; ++u) {
-            const unsigned i0 = q[u].x & 0xFFFFu, i1 = q[u].x >> 16, i2 = q[u].y & 0xFFFFu, i3 = q[u].y >> 16;
+          for (int u = 0; u < 4; ++u) q[u] = qn[u];
+          cp += 128;
 #pragma unroll
-            for (int r = 0; r < R; ++r) sum[r] += (xs[r][i0] + xs[r][i1]) + (xs[r][i2] + xs[r][i3]);
-          }
+          for (int u = 0; u < 4; ++u) qn[u] = __ldg(cp + 32 * u);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) add_pair(q[u]);
         }
-        cp += n4;
+        if (i > 0) {
+          const unsigned q0 = qn[0], q1 = qn[1], q2 = qn[2];
+          cp += 32 * i;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) qn[u] = __ldg(cp + 32 * u);
+          add_pair(q0);
+          if (i > 1) add_pair(q1);
+          if (i > 2) add_pair(q2);
+        }
         const typename Pol::W wc = Pol::w(t, c);
 #pragma unroll
         for (int r = 0; r < R; ++r) acc[r] += Pol::wmul(wc, sum[r]);
       }
-      if (p.ncross) {
-        unsigned dr[R];
+      if (n_oct && t.xs_ok) {
+        S s0[R], s1[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) dr[r] = r < nr ? (pa[r] ^ pb) : 0u;
-        if (kLists && t.xl_ok) {
-          // per B cross site, the column's bit there picks each row's lists of
-          // valid bonds (one per value class); the gathers of all rows' lists are
-          // issued before any is summed (invalid slots read nothing and add zero),
-          // the next site's map entry is loaded one site ahead, and each class's
-          // sum is multiplied by its weight once per column
-          unsigned mq_next = t.n_ib > 0 ? __ldg(t.mapB + gB) : 0u;
-          S s0[R], s1[R];
+        for (int r = 0; r < R; ++r) s0[r] = s1[r] = 0;
+        for (int h = 0; h < n_oct; ++h) {
+          unsigned z[R];
 #pragma unroll
-          for (int r = 0; r < R; ++r) s0[r] = s1[r] = 0;
-          for (int ib = 0; ib < t.n_ib; ++ib) {
-            const unsigned mq = mq_next;
-            if (ib + 1 < t.n_ib) mq_next = __ldg(t.mapB + (long long)(ib + 1) * t.B_total + gB);
-            const int mx0 = xl_mx[ib][0], mx1 = xl_mx[ib][1];
-            if (!(mx0 | mx1)) continue;
-            const int beta = (int)((pb >> (__ffs(t.ib_mask[ib]) - 1)) & 1u);
-            int n0[R], n1[R];
-            S v0[R][kXL], v1[R][kXL];
+          for (int r = 0; r < R; ++r) z[r] = in ? (s_ax[h][r] ^ bx) & s_vm[h][r] : 0u;
+          const unsigned pm = t.xs_present[h];
+          const uint4 mc = mv;
+          if (h + 1 < n_oct) {
+            mv = __ldg(t.B_xmap + (h + 1) * t.B_total + gB);
+            bx = __ldg(t.B_xs + (h + 1) * t.B_total + gB);
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const unsigned pj = (pm >> (4 * j)) & 15u;
+            if (!pj) break;
+            const unsigned mw = j < 2 ? mc.x : j < 4 ? mc.y : j < 6 ? mc.z : mc.w;
+            const unsigned mq = (j & 1) ? mw >> 16 : mw & 0xFFFFu;
+            S v[4][R];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+#pragma unroll
+              for (int r = 0; r < R; ++r) v[s][r] = 0;
+              if ((pj >> s) & 1u) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                  v[s][r] = ldg_if(s_ptr[h][4 * j + s][r] + mq, (z[r] & (1u << (4 * j + s))) != 0u);
+              }
+            }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-              n0[r] = xl_n[r][ib][beta][0];
-              n1[r] = xl_n[r][ib][beta][1];
-            }
-#pragma unroll
-            for (int i = 0; i < kXL; ++i) {
-#pragma unroll
-              for (int r = 0; r < R; ++r) {
-                v0[r][i] = (i < mx0 && i < n0[r]) ? __ldg(xl_ptr[r][ib][beta][0][i] + mq) : (S)0;
-                v1[r][i] = (i < mx1 && i < n1[r]) ? __ldg(xl_ptr[r][ib][beta][1][i] + mq) : (S)0;
-              }
-            }
-#pragma unroll
-            for (int i = 0; i < kXL; ++i)
-#pragma unroll
-              for (int r = 0; r < R; ++r) {
-                s0[r] += v0[r][i];
-                s1[r] += v1[r][i];
-              }
-          }
-          {
-            const typename Pol::W w0 = Pol::w(t, t.xl_c[0]), w1 = Pol::w(t, t.xl_c[1]);
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] += Pol::wmul(w0, s0[r]) + Pol::wmul(w1, s1[r]);
-          }
-        } else if constexpr (sizeof(S) == 4) {
-          // 4-byte types (four rows per pass): loop over every bond with
-          // warp-uniform table indices (B site, bond, weight); only the
-          // validity predicate and the gather address vary across lanes
-          unsigned mq_next = t.n_ib > 0 ? __ldg(t.mapB + gB) : 0u;  // map entries one site ahead
-          for (int ib = 0; ib < t.n_ib; ++ib) {
-            const unsigned mq = mq_next;
-            if (ib + 1 < t.n_ib) mq_next = __ldg(t.mapB + (long long)(ib + 1) * t.B_total + gB);
-            unsigned km = t.ib_mask[ib];
-            while (km) {
-              const int k = __ffs(km) - 1;
-              km &= km - 1;
-              const typename Pol::W wk = Pol::bw(t, k);
-              const int ia = t.bond_ia[k];
-#pragma unroll
-              for (int r = 0; r < R; ++r) {
-                const S* sp = src_row[r][ia];
-                if (((dr[r] >> k) & 1u) && sp) acc[r] += Pol::wmul(wk, __ldg(sp + mq));
-              }
+              s0[r] += v[0][r] + v[1][r];
+              s1[r] += v[2][r] + v[3][r];
             }
           }
-        } else {
-          // 8-byte types with more than kXL bonds at some B cross site: the
-          // gathers of a site's first kXB bonds (warp-uniform bond indices)
-          // for both rows are issued before any is summed; bonds beyond kXB
-          // take a plain loop
-          constexpr int kXB = 4;
-          unsigned mq_next = t.n_ib > 0 ? __ldg(t.mapB + gB) : 0u;
-          for (int ib = 0; ib < t.n_ib; ++ib) {
-            const unsigned mq = mq_next;
-            if (ib + 1 < t.n_ib) mq_next = __ldg(t.mapB + (long long)(ib + 1) * t.B_total + gB);
-            unsigned rm = t.ib_mask[ib];
-            int kq[kXB];
+        }
+        const typename Pol::W w0 = Pol::w(t, t.xl_c[0]), w1 = Pol::w(t, t.xl_c[1]);
 #pragma unroll
-            for (int q = 0; q < kXB; ++q) {
-              kq[q] = rm ? __ffs(rm) - 1 : -1;
-              rm &= rm - 1;
-            }
-            S v[R][kXB];
+        for (int r = 0; r < R; ++r) acc[r] += Pol::wmul(w0, s0[r]) + Pol::wmul(w1, s1[r]);
+      } else if (n_oct) {
+        // more than two value classes on the cut: bond by bond
+        unsigned z[R];
 #pragma unroll
-            for (int q = 0; q < kXB; ++q)
+        for (int r = 0; r < R; ++r) z[r] = in ? (s_ax[0][r] ^ pb) & s_vm[0][r] : 0u;
+        for (int k = 0; k < p.ncross; ++k) {
+          const unsigned mq = __ldg(t.mapB + (long long)t.bond_ib[k] * t.B_total + gB);
+          const typename Pol::W wk = Pol::bw(t, k);
 #pragma unroll
-              for (int r = 0; r < R; ++r) {
-                v[r][q] = 0;
-                if (kq[q] >= 0 && ((dr[r] >> kq[q]) & 1u)) {
-                  const S* sp = src_row[r][t.bond_ia[kq[q]]];
-                  if (sp) v[r][q] = __ldg(sp + mq);
-                }
-              }
-#pragma unroll
-            for (int q = 0; q < kXB; ++q)
-              if (kq[q] >= 0) {
-                const typename Pol::W w = Pol::bw(t, kq[q]);
-#pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] += Pol::wmul(w, v[r][q]);
-              }
-            while (rm) {
-              const int k = __ffs(rm) - 1;
-              rm &= rm - 1;
-#pragma unroll
-              for (int r = 0; r < R; ++r) {
-                const S* sp = src_row[r][t.bond_ia[k]];
-                if (((dr[r] >> k) & 1u) && sp) acc[r] += Pol::wmul(Pol::bw(t, k), __ldg(sp + mq));
-              }
-            }
-          }
+          for (int r = 0; r < R; ++r)
+            if ((z[r] >> k) & 1u) acc[r] += Pol::wmul(wk, __ldg(s_ptr[0][k][r] + mq));
         }
       }
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        if (r < nr) store_out<Pol>(y, bl.off + (a0 + r) * dB + b, acc[r], final_, e2);
+        if (in && r < nr) store_out<Pol>(y, row0 + (long long)r * dB + b, acc[r], final_, e2);
     }
-    __syncthreads();
   }
 }
 
@@ -502,29 +432,17 @@ static P3 make_p3(const ed_ctx* c) {
   return p;
 }
 
-// Row-pass shapes: one 1024-thread CTA per SM whose staged rows fill the
-// shared memory and share the B-side index and map loads: four rows per
-// pass for 4-byte types, two for 8-byte types.  On the J1-J2 4x8 workload
-// this measured 15.7 ms (FP32) and 35.3 ms (FP64) against 23.3 and 40.9 ms
-// for two (FP32) or one (FP64) row per pass in two 512-thread CTAs per SM
-// (kRow4Quad / kRow8Pair = false).
-constexpr bool kRow8Pair = true;
-constexpr bool kRow4Quad = true;
-static int rows_per_pass(size_t es) { return es == 4 ? (kRow4Quad ? 4 : 2) : (kRow8Pair ? 2 : 1); }
-
-static size_t v3_smem(const ed_ctx* c, size_t es, long long* stage_elems) {
+// dynamic shared memory of the row pass: the R rows (16 bytes a column) of the
+// widest block and eight zero slots
+static size_t v3_smem(const ed_ctx* c) {
   long long mdb = 1;
   for (const auto& b : c->blocks) mdb = std::max<long long>(mdb, b.dB);
-  *stage_elems = ((mdb + 1 + 16 / (long long)es + 15) / 16) * 16;  // row, zero slot, alignment pad
-  return 128 + (size_t)rows_per_pass(es) * (size_t)(*stage_elems) * es;
+  return (size_t)(mdb + 8) * 16;
 }
 
 bool v3_usable(const ed_ctx* c, ed_dtype dt, const void* x) {
-  if (!c->v3_ok || ((uintptr_t)x % 16) != 0) return false;
-  long long se;
-  const size_t es = dt == ED_F64 ? 8 : 4;
-  const bool one_cta = (es == 8 && kRow8Pair) || (es == 4 && kRow4Quad);
-  return v3_smem(c, es, &se) <= (one_cta ? 220 : 110) * 1024;
+  (void)dt;
+  return c->v3_ok && ((uintptr_t)x % 16) == 0 && v3_smem(c) <= 220 * 1024;
 }
 
 // events bracketing the stages of one apply when profiling is on
@@ -550,22 +468,25 @@ static ed_status run_v3(ed_ctx* c, const typename Pol::S* x, typename Pol::Y* y,
                         ProfMarks& pm) {
   P3 p = make_p3(c);
   if (p.n_rows == 0) return ED_OK;
-  long long se;
-  constexpr bool pair8 = sizeof(typename Pol::S) == 8 && kRow8Pair;
-  constexpr bool quad4 = sizeof(typename Pol::S) == 4 && kRow4Quad;
-  constexpr int R = quad4 ? 4 : (sizeof(typename Pol::S) == 4 || pair8) ? 2 : 1;
-  constexpr int NT = (pair8 || quad4) ? 1024 : kRowThreads;
-  constexpr int CPS = (pair8 || quad4) ? 1 : 2;  // CTAs per SM
-  const size_t smem = v3_smem(c, sizeof(typename Pol::S), &se);
+  constexpr int R = 16 / (int)sizeof(typename Pol::S);
+  const size_t smem = v3_smem(c);
   const int sms = n_sms(c->device);
   pm.mark(2, st);
   {
-    auto kern = k_row5<Pol, R, NT, CPS>;
-    ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const long long* gs = R == 4 ? c->d_grp4_start : R == 2 ? c->d_grp2_start : c->d_row_start;
-    const long long ng = R == 4 ? c->n_grp4 : R == 2 ? c->n_grp2 : c->n_rows;
-    const long long grid = std::min<long long>(ng, (long long)sms * CPS);
-    kern<<<(unsigned)grid, NT, smem, st>>>(p, gs, ng, x, y, emax, se, c->d_err);
+    const long long* gs = R == 4 ? c->d_grp4_start : c->d_grp2_start;
+    const long long ng = R == 4 ? c->n_grp4 : c->n_grp2;
+    // 1024 threads per SM: in one CTA while its rows need more than half of
+    // the shared memory, else in two or four CTAs, so that one stages its
+    // rows while another sums
+    auto go = [&](auto kern, int nt) -> ed_status {
+      ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      const long long grid = std::min<long long>(ng, (long long)sms * (1024 / nt));
+      kern<<<(unsigned)grid, nt, smem, st>>>(p, gs, ng, x, y, emax);
+      return ED_OK;
+    };
+    if (smem > 106 * 1024) ED_TRY(go(k_row5<Pol, R, 1024>, 1024));
+    else if (smem > 50 * 1024) ED_TRY(go(k_row5<Pol, R, 512>, 512));
+    else ED_TRY(go(k_row5<Pol, R, 256>, 256));
   }
   ED_CUDA_TRY(cudaGetLastError());
   pm.mark(3, st);

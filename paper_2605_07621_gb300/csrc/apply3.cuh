@@ -2,7 +2,7 @@
 // the kernel parameter block, the arithmetic policies (FP32, FP64, exact
 // 64-bit fixed point, fixed-point sums with FP64 weights), the fixed-point
 // <-> FP64 conversions done by
-// bit manipulation, and the TMA / mbarrier helpers.
+// bit manipulation.
 #pragma once
 
 #include <cstdint>
@@ -71,26 +71,24 @@ struct PF64 {
     return v;
   }
 };
+// The integer diagonal and weights are 32-bit: every weight is at most 2^24 in
+// magnitude (dyadic couplings), the diagonal a sum of three such terms and 32
+// such weights, so a product with x takes a 64 x 32-bit multiplication.
 struct PI64 {
   using S = long long;
   using Y = long long;
   using A = long long;
-  using D = long long;
-  using W = long long;
-  __device__ static long long dmul(long long d, long long x) { return d * x; }
-  __device__ static long long wmul(long long w, long long s) { return w * s; }
-  __device__ static long long w(const Dev3& t, int c) { return t.wI[c]; }
-  __device__ static long long bw(const Dev3& t, int k) { return t.bond_wI[k]; }
-  __device__ static long long diagA(const Dev3& t, long long gA) { return (long long)t.A_dI[gA] + t.dc0_I; }
-  __device__ static long long diagB(const Dev3& t, long long gB) { return (long long)t.B_dI[gB]; }
-  __device__ static long long vab(const Dev3& t, unsigned z) {
-    long long v = 0;
-    for (int q = 0; q < t.ncls_d; ++q) v += t.dwI[q] * (long long)__popc(z & t.dmask[q]);
-    return v;
-  }
-  __device__ static long long diag(const Dev3& t, long long gA, long long gB, unsigned z) {
-    long long v = (long long)t.A_dI[gA] + (long long)t.B_dI[gB] + t.dc0_I;
-    for (int q = 0; q < t.ncls_d; ++q) v += t.dwI[q] * (long long)__popc(z & t.dmask[q]);
+  using D = int;
+  using W = int;
+  __device__ static long long dmul(int d, long long x) { return d * x; }
+  __device__ static long long wmul(int w, long long s) { return w * s; }
+  __device__ static int w(const Dev3& t, int c) { return (int)t.wI[c]; }
+  __device__ static int bw(const Dev3& t, int k) { return (int)t.bond_wI[k]; }
+  __device__ static int diagA(const Dev3& t, long long gA) { return t.A_dI[gA] + (int)t.dc0_I; }
+  __device__ static int diagB(const Dev3& t, long long gB) { return t.B_dI[gB]; }
+  __device__ static int vab(const Dev3& t, unsigned z) {
+    int v = 0;
+    for (int q = 0; q < t.ncls_d; ++q) v += (int)t.dwI[q] * __popc(z & t.dmask[q]);
     return v;
   }
 };
@@ -168,7 +166,11 @@ struct PW {
   __device__ static long long bw(const Dev3& t, int k) { return t.bond_wI[k]; }
   __device__ static long long diagA(const Dev3& t, long long gA) { return t.A_dW[gA] + t.dc0_I; }
   __device__ static long long diagB(const Dev3& t, long long gB) { return t.B_dW[gB]; }
-  __device__ static long long vab(const Dev3& t, unsigned z) { return PI64::vab(t, z); }
+  __device__ static long long vab(const Dev3& t, unsigned z) {
+    long long v = 0;
+    for (int q = 0; q < t.ncls_d; ++q) v += t.dwI[q] * (long long)__popc(z & t.dmask[q]);
+    return v;
+  }
 };
 
 // ---------------------------------------------------------------- fixed point <-> FP64 by bit manipulation
@@ -305,38 +307,6 @@ __device__ __forceinline__ void store_out<PC64>(double* y, long long i, double v
 template <>
 __device__ __forceinline__ void store_out<PW>(double* y, long long i, AccW v, bool final_, int e2) {
   y[i] = v.p + from_fixed128(v.s, e2);  // both passes store real values
-}
-
-// ---------------------------------------------------------------- TMA / mbarrier
-
-__device__ __forceinline__ unsigned s_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void bar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void bar_expect(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(unsigned long long* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   s_u32(dst)),
-               "l"(src), "r"(bytes), "r"(s_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parity) {
-  for (long long i = 0; i < (1ll << 22); ++i) {
-    unsigned ok;
-    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                 : "=r"(ok)
-                 : "r"(s_u32(bar)), "r"(parity)
-                 : "memory");
-    if (ok) return true;
-  }
-  return false;
 }
 
 __device__ __forceinline__ int find_blk(const long long* row_start, int nblk, long long row) {

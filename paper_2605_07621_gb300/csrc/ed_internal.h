@@ -117,7 +117,7 @@ struct DevBlock {
   int nbr_lo, nbr_hi;   // block index of charge s-1 / s+1 (-1 if absent)
   long long dA, dB, off, gA0, gB0, row0;
   int has_hA;           // the block's rows have H_A entries (second pass needed)
-  int pad_;
+  int slabB0;           // first 32-column slab of the block's side-B charge (Dev3::B_slab)
 };
 
 struct DevCross {
@@ -157,12 +157,11 @@ struct DevTables {
 // entry.  When every coupling is a dyadic rational (value * 2^q_shift is a
 // small integer) the FP64 apply runs in exact 64-bit fixed point.
 constexpr int kMaxCls = 4;
+constexpr int kMaxOct = 4;  // octets of cross-bond sites (32 bonds, one per site at worst)
 
 struct Dev3 {
   const uint2* A_meta;      // x: first entry, y: per-class counts (8 bits each)
   const uint16_t* A_col;
-  const uint2* B_meta;
-  const uint16_t* B_col;
   const uint32_t* A_pack;   // packed cross-bond bits (spin) or up string (Hubbard)
   const uint32_t* B_pack;
   const float* A_d32;
@@ -192,17 +191,27 @@ struct Dev3 {
   unsigned cross_cls_mask[kMaxCls];  // cross bonds (bit k) with off-diagonal class c
   int q_shift;              // values * 2^q_shift are integers (fixed-point path)
   int P;                    // fraction bits of the fixed-point vector
-  // padded side-B lists of the row pass: every class segment starts at a
-  // multiple of 4 entries and is padded to one with the zero-slot index d_B
-  const uint2* B_meta4;     // x: first entry / 4, y: per-class group-of-4 counts
-  const uint2* B_col4;      // 4 x uint16 per element
-  // cross bonds grouped by B site: bonds with B site ib are bits ib_mask[ib]
+  // side-B lists of the row pass, in slabs of 32 columns: per slab the first
+  // pair row and the number of pair rows of each class (the longest list of
+  // the slab, in pairs), and pair rows of 32 words, word l = two 16-bit
+  // indices of the slab's column l (past its end the zero slots d_B .. d_B + 7)
+  const uint2* B_slab;      // x: first pair row, y: per-class pair rows (8 bits each)
+  const unsigned* B_pair;
   int n_ib;
   int n_ia;
-  int xl_ok;                // row-pass bond lists apply: the cross bonds take at most two
-                            // value classes, each B cross site at most two bonds of each
+  // cross terms of the row pass (xs_ok: the cross bonds take at most two
+  // value classes).  The bonds are dealt to "sites", each one B cross site
+  // with at most two bonds of the first class (slots 0, 1) and two of the
+  // second (slots 2, 3); eight sites make an octet, whose 32 slots are the
+  // bits of one word and whose eight column maps are one 16-byte load
+  int xs_ok;
+  int n_oct;
   int xl_c[2];              // the two classes (equal when there is one)
-  unsigned xl_c1_mask;      // cross bonds (bit k) of class xl_c[1] (the rest are xl_c[0])
+  unsigned xs_present[kMaxOct];        // slots that hold a bond
+  unsigned char xs_k[32 * kMaxOct];    // bond of each slot (255: none)
+  const unsigned* A_xs;     // [n_oct][A_total] A-side bit of each slot's bond
+  const unsigned* B_xs;     // [n_oct][B_total] B-side bit of each slot's bond
+  const uint4* B_xmap;      // [n_oct][B_total] eight 16-bit column maps
   unsigned ib_mask[32];
   unsigned ia_mask[32];     // bonds (bits) whose A site is ia
   unsigned char bond_ib[32];

@@ -28,12 +28,25 @@ int64_t binom(int n, int k) {
   return r;
 }
 
+// Pascal's triangle for the ranks: a rank is a sum of table entries (the
+// tables of one context need about one rank per matrix element and map entry)
+namespace {
+struct Pascal {
+  int64_t c[64][65];
+  Pascal() {
+    for (int n = 0; n < 64; ++n)
+      for (int k = 0; k <= 64; ++k) c[n][k] = k == 0 ? 1 : n == 0 || k > n ? 0 : c[n - 1][k - 1] + c[n - 1][k];
+  }
+};
+}  // namespace
+
 int64_t combinadic_rank(uint64_t x) {
+  static const Pascal tri;
   int64_t r = 0;
   int j = 0;
   while (x) {
     int p = __builtin_ctzll(x);
-    r += binom(p, j + 1);
+    r += tri.c[p][j + 1];
     ++j;
     x &= x - 1;
   }
