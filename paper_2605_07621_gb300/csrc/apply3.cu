@@ -316,50 +316,59 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
   }
 }
 
-// 32 x NC zeros read by k_panel4 in place of missing neighbour rows
-static __device__ __align__(16) long long g_zero_row[256];
+constexpr int kPanelCtas = 3;  // resident CTAs of the panel pass per SM
 
-// H_A panel pass with U neighbour rows in flight per class step: each warp
-// owns one output row of a 256-column panel, processed as sub-panels of
-// 32 * NC columns; the column indices of U consecutive H_A entries are read
-// first (warp-uniform), then all U x NC neighbour values are loaded before
-// any is summed, so U x NC independent loads per lane overlap their
-// latency instead of one neighbour row at a time.  Full sub-panels need no
-// per-column checks, and entries past a class's end read the zero row, so
-// their loads carry no predicates.
+// H_A panel pass: work item = a run of rows of one block times a panel of
+// 32 * NC columns.  A warp owns one output row of the panel at a time, a CTA
+// the item's rows in ascending order: side-A neighbours that differ in low
+// bits are a few rows away, so their panel segments (1 KB each) are found in
+// L1, the others in L2, where the whole column panel stays resident.  The
+// column indices of up to 32 entries are read by the 32 lanes at once and
+// their row offsets broadcast entry by entry; U neighbour rows (U x NC
+// independent loads per lane) are in flight before any is summed.  One CTA
+// per item, started in item order, keeps every SM on the same one or two
+// panels; a persistent grid drifts apart over many panels and loses the L2
+// residency (J1-J2 4x8: 17 ms).
+// Bound: latency of L2 (52 % of its throughput) and issue (57 %).  Measured,
+// FP64 fixed point / FP32: J1-J2 4x8 (601 M states) 9.8 -> 7.8 / 5.4 -> 4.1 ms,
+// Hubbard 4x4 (166 M states) 2.04 -> 1.65 / 1.16 -> 0.84 ms against one row and
+// 256 columns per warp with per-entry index loads and 64-bit offsets.  Runs of
+// 16 and 32 rows: 8.5 and 7.9 ms; two or four resident CTAs: 10.5 and 8.4 ms.
 template <class Pol, int NC, int U>
-__global__ void __launch_bounds__(256) k_panel4(P3 p, const int4* __restrict__ items, long long n_items,
+__global__ void __launch_bounds__(256, kPanelCtas) k_panel4(P3 p, const long long* __restrict__ item_start, int rows,
                                                 const typename Pol::S* __restrict__ x, typename Pol::Y* __restrict__ y,
                                                 const int* __restrict__ emax) {
   using S = typename Pol::S;
   constexpr int W = 32 * NC;
-  static_assert(256 % W == 0, "sub-panels must tile the 256-column panel");
   const Dev3& t = p.t;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e2 = emax ? out_exp(t, emax) : 0;
-  for (long long w = blockIdx.x; w < n_items; w += gridDim.x) {
-    const int4 it = items[w];
-    if (warp >= it.w) continue;
-    const DevBlock bl = p.blocks[it.x];
-    const long long a = it.z + warp;
-    const long long gA = bl.gA0 + a;
-    const long long dB = bl.dB;
-    const S* xb = x + bl.off;
-    typename Pol::Y* yrow = y + bl.off + a * dB;
-    const uint2 m = t.A_meta[gA];
-    for (int sp = 0; sp < 256; sp += W) {
-      const long long b0 = it.y + sp + lane;
-      if (it.y + sp >= dB) break;
-      const bool full = it.y + sp + W <= dB;
-      const S* xb0 = xb + b0;                                              // column b0 of row 0
-      const S* zr = reinterpret_cast<const S*>(g_zero_row) + lane;         // zeros at +32c
-      typename Pol::A acc[NC];
+  const long long w = blockIdx.x;
+  const int bi = find_blk(item_start, p.nblk, w);
+  const DevBlock& bl = p.blocks[bi];
+  const int nrun = (int)((bl.dA + rows - 1) / rows), q = (int)(w - item_start[bi]);
+  const int col0 = q / nrun * W, row0 = q % nrun * rows, row1 = min(row0 + rows, (int)bl.dA);
+  const unsigned dB = (unsigned)bl.dB;
+  const long long off = bl.off, gA0 = bl.gA0;
+  const unsigned b0 = col0 + lane;
+  const bool full = col0 + W <= (int)dB;
+  const S* xb0 = x + off + min(b0, dB - 1);
+  for (int a = row0 + warp; a < row1; a += 8) {
+    typename Pol::Y* yrow = y + off + (long long)a * dB + b0;
+    const uint2 m = t.A_meta[gA0 + a];
+    typename Pol::A acc[NC];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const long long b = b0 + 32 * c;
-        acc[c] = typename Pol::A(b < dB ? yrow[b] : (typename Pol::Y)0);
-      }
-      unsigned e = m.x;
+    for (int c = 0; c < NC; ++c)
+      acc[c] = typename Pol::A(full || b0 + 32 * c < dB ? yrow[32 * c] : (typename Pol::Y)0);
+    const uint16_t* ep = t.A_col + m.x;
+    const int tot = (int)((m.y & 255u) + ((m.y >> 8) & 255u) + ((m.y >> 16) & 255u) + (m.y >> 24));
+    int pos = 0, cb = 0;
+    unsigned ro = lane < tot ? (unsigned)ep[lane] * dB : 0u;  // row offset of entry cb + lane
+    auto run = [&](auto FULL) {
+      unsigned cc[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        cc[c] = decltype(FULL)::value ? 32u * c : (b0 + 32 * c < dB ? 32u * c : 0u);
 #pragma unroll
       for (int cl = 0; cl < kMaxCls; ++cl) {
         const int n = (int)((m.y >> (8 * cl)) & 255u);
@@ -367,57 +376,41 @@ __global__ void __launch_bounds__(256) k_panel4(P3 p, const int4* __restrict__ i
         S sum[NC];
 #pragma unroll
         for (int c = 0; c < NC; ++c) sum[c] = 0;
-        if (full) {
-          // full sub-panel: no per-column checks; entries past the class end
-          // read a zero row
-          for (int i0 = 0; i0 < n; i0 += U) {
-            const S* rp[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-              rp[u] = i0 + u < n ? xb0 + (long long)t.A_col[e + i0 + u] * dB : zr;
-            S v[U][NC];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-              for (int c = 0; c < NC; ++c) v[u][c] = __ldg(rp[u] + 32 * c);
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-              for (int c = 0; c < NC; ++c) sum[c] += v[u][c];
+        for (int i = 0; i < n; i += U) {
+          if (pos + U > cb + 32) {
+            cb = pos;
+            ro = cb + lane < tot ? (unsigned)ep[cb + lane] * dB : 0u;
           }
-        } else {
-        for (int i0 = 0; i0 < n; i0 += U) {
-          long long rowoff[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) rowoff[u] = i0 + u < n ? (long long)t.A_col[e + i0 + u] * dB : -1;
           S v[U][NC];
 #pragma unroll
-          for (int u = 0; u < U; ++u)
+          for (int u = 0; u < U; ++u) {
+            const S* rp = xb0 + __shfl_sync(0xffffffffu, ro, (pos - cb + u) & 31);
+            if (u == 0 || i + u < n) {
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-              const long long b = b0 + 32 * c;
-              v[u][c] = (rowoff[u] >= 0 && b < dB) ? __ldg(xb + rowoff[u] + b) : (S)0;
+              for (int c = 0; c < NC; ++c) v[u][c] = __ldg(rp + cc[c]);
+            } else {
+#pragma unroll
+              for (int c = 0; c < NC; ++c) v[u][c] = 0;
             }
+          }
 #pragma unroll
           for (int u = 0; u < U; ++u)
 #pragma unroll
             for (int c = 0; c < NC; ++c) sum[c] += v[u][c];
+          pos += min(U, n - i);
         }
-        }
-        e += n;
         const typename Pol::W wc = Pol::w(t, cl);
 #pragma unroll
         for (int c = 0; c < NC; ++c) acc[c] += Pol::wmul(wc, sum[c]);
       }
+    };
+    if (full) run(std::true_type{});
+    else run(std::false_type{});
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const long long b = b0 + 32 * c;
-        if (b < dB) store_out<Pol>(yrow, b, acc[c], true, e2);
-      }
-    }
+    for (int c = 0; c < NC; ++c)
+      if (full || b0 + 32 * c < dB) store_out<Pol>(yrow, 32 * c, acc[c], true, e2);
   }
 }
-
 
 static P3 make_p3(const ed_ctx* c) {
   P3 p;
@@ -490,16 +483,12 @@ static ed_status run_v3(ed_ctx* c, const typename Pol::S* x, typename Pol::Y* y,
   }
   ED_CUDA_TRY(cudaGetLastError());
   pm.mark(3, st);
-  if (c->n_panel_items > 0) {
-    const long long g2 = std::min<long long>(c->n_panel_items, (long long)sms * 8);
-    // measured on the 4x8 J1-J2 and 4x4 Hubbard workloads: 8-byte types
-    // gain from four neighbour rows in flight on 128-column sub-panels
-    // (one row at a time: 24.5 / 5.1 ms; four: 9.9 / 2.0 ms), FP32 from two
-    // rows in flight on full 256-column panels (6.2 -> 5.4 ms on J1-J2 4x8)
-    if constexpr (sizeof(typename Pol::S) == 4)
-      k_panel4<Pol, 8, 2><<<(unsigned)g2, 256, 0, st>>>(p, c->d_panel_items, c->n_panel_items, x, y, emax);
-    else
-      k_panel4<Pol, 4, 4><<<(unsigned)g2, 256, 0, st>>>(p, c->d_panel_items, c->n_panel_items, x, y, emax);
+  constexpr int q = sizeof(typename Pol::S) == 4 ? 1 : 0;
+  if (c->n_panel[q] > 0) {
+    // 1 KB of a row per panel: 128 columns of 8-byte types with four neighbour
+    // rows in flight, 256 of FP32 with two
+    const long long* is = c->d_panel_start + q * (c->blocks.size() + 1);
+    k_panel4<Pol, q ? 8 : 4, q ? 2 : 4><<<(unsigned)c->n_panel[q], 256, 0, st>>>(p, is, c->panel_rows[q], x, y, emax);
     ED_CUDA_TRY(cudaGetLastError());
   }
   return ED_OK;

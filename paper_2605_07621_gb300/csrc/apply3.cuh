@@ -221,32 +221,22 @@ __host__ __device__ __forceinline__ long long to_fixed(double v, int sh_base) {
   return s ? -X : X;
 }
 
-// Y * 2^e2 rounded to nearest (ties to even) FP64
+// Y * 2^e2 rounded to nearest (ties to even) FP64: the magnitude's leading one
+// moved to bit 63, its top 53 bits and the rounding increment added to the
+// exponent field (the implicit bit and a mantissa overflow carry into it).
+// Exponents outside the normal range give zero or infinity.
 __host__ __device__ __forceinline__ double from_fixed(long long Y, int e2) {
   if (Y == 0) return 0.0;
-  const unsigned long long s = Y < 0 ? 1ull : 0ull;
-  unsigned long long u = s ? (unsigned long long)(-Y) : (unsigned long long)Y;
-  int p = 63 - clz64(u);
-  unsigned long long mant;
-  if (p <= 52) {
-    mant = u << (52 - p);
-  } else {
-    const int sh = p - 52;
-    mant = u >> sh;
-    const unsigned long long rem = u & ((1ull << sh) - 1);
-    const unsigned long long half = 1ull << (sh - 1);
-    if (rem > half || (rem == half && (mant & 1ull))) {
-      ++mant;
-      if (mant >> 53) {
-        mant >>= 1;
-        ++p;
-      }
-    }
-  }
-  const int ex = p + e2 + 1023;
-  if (ex <= 0) return s ? -0.0 : 0.0;
-  if (ex >= 2047) return bits_f64((s << 63) | (0x7ffull << 52));
-  return bits_f64((s << 63) | ((unsigned long long)ex << 52) | (mant & 0xFFFFFFFFFFFFFull));
+  const unsigned long long s = Y < 0 ? 1ull << 63 : 0ull;
+  const unsigned long long u = s ? 0ull - (unsigned long long)Y : (unsigned long long)Y;
+  const int n = clz64(u);
+  const unsigned long long h = u << n;
+  unsigned long long m = h >> 11;
+  m += (((unsigned)h & 0x7FFu) + 0x3FFu + ((unsigned)m & 1u)) >> 11;
+  const int ex = 63 - n + e2 + 1023 + (int)(m >> 53);  // after rounding
+  if (ex <= 0) return bits_f64(s);
+  if (ex >= 2047) return bits_f64(s | (0x7ffull << 52));
+  return bits_f64(s | (((unsigned long long)(63 - n + e2 + 1022) << 52) + m));
 }
 
 // v * 2^e2 rounded to nearest (ties to even) FP64, v a 128-bit integer

@@ -272,6 +272,9 @@ struct ed_ctx {
   long long* d_grp4_start = nullptr; // per block: first four-row group (plus total)
   long long n_grp4 = 0;
   long long n_panel_items = 0;
+  long long* d_panel_start = nullptr;  // class-sorted H_A pass, [8-byte types, FP32][block]: first item (plus total)
+  long long n_panel[2] = {0, 0};
+  int panel_rows[2] = {8, 8};        // rows per item
   int* d_err = nullptr;              // set by kernels whose bounded waits ran out
   // class-sorted path
   bool v3_ok = false;                // tables below are valid

@@ -655,6 +655,30 @@ extern "C" ed_status ed_build_local_ops(ed_ctx* c, int flags) {
     c->n_panel_items = (long long)items.size();
     ED_TRY(upload(c, &c->d_panel_items, items));
   }
+  // items of the class-sorted H_A pass: panels of 1 KB of a row times runs of
+  // 64 rows (fewer while that leaves less than about four items per resident
+  // CTA, down to one row per warp)
+  {
+    std::vector<long long> ps;
+    for (int q = 0; q < 2; ++q) {
+      const int64_t cols = q ? 256 : 128;
+      for (int rows = 64;; rows /= 2) {
+        std::vector<long long> s1(1, 0);
+        for (size_t bi = 0; bi < c->blocks.size(); ++bi) {
+          const Block& b = c->blocks[bi];
+          const int64_t n = ((b.dA + rows - 1) / rows) * ((b.dB + cols - 1) / cols);
+          s1.push_back(s1.back() + (c->h_blocks[bi].has_hA ? n : 0));
+        }
+        if (s1.back() >= 1824 || rows <= 8) {
+          c->panel_rows[q] = rows;
+          c->n_panel[q] = s1.back();
+          ps.insert(ps.end(), s1.begin(), s1.end());
+          break;
+        }
+      }
+    }
+    ED_TRY(upload(c, &c->d_panel_start, ps));
+  }
   {
     std::vector<int> z(4, 0);
     ED_TRY(upload(c, &c->d_err, z));
