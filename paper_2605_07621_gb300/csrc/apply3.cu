@@ -42,22 +42,86 @@ void host_mul_wide(long long a, long long b, long long* hi, unsigned long long* 
   *lo = v.lo;
 }
 
-// largest biased exponent of x (atomic max into out[0]; out must start at 0)
-__global__ void k_exp_max(const double* __restrict__ x, long long n, int* out) {
-  int m = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    m = max(m, (int)(((unsigned long long)__double_as_longlong(x[i]) >> 52) & 0x7ffull));
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+// Programmatic dependent launch: the kernel is set up while the previous one
+// of the stream drains, and waits here until that one has finished and its
+// writes are visible.  Called before any access to global memory.  (H|psi> of
+// 12,870 / 853,776 states: 22.5 -> 16.3 / 32.8 -> 25.6 us.  Releasing the next
+// kernel earlier, by launch_dependents, costs the large sectors 7 %: its CTAs
+// take slots from the running kernel's last wave.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ int biased_exp(double v) {
+  return (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffull);
 }
 
-// |x| < 2^E with E = emax - 1022; X = round(x * 2^(P - E))
-__global__ void k_to_fixed(const double* __restrict__ x, long long* __restrict__ X, long long n,
-                           const int* __restrict__ emax, int P) {
-  const int E = emax[0] - 1022;
-  const int sh = P - E;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    X[i] = to_fixed(x[i], sh);
+// largest of the CTA's values, in every thread (blockDim a multiple of 32)
+__device__ __forceinline__ int block_max(int m) {
+  __shared__ int red[32];
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  const int w = threadIdx.x & 31;
+  return __reduce_max_sync(0xffffffffu, w < (int)(blockDim.x >> 5) ? red[w] : 0);
+}
+
+// largest biased exponent of each CTA's share of x into part[blockIdx.x];
+// the next kernel takes the largest of them (no atomics, nothing to clear).
+// x is 16-byte aligned.  Bound by HBM: 0.67 ms for 4.8 GB (7.2 TB/s).
+__global__ void __launch_bounds__(256) k_exp_max(const double* __restrict__ x, long long n, int* __restrict__ part) {
+  pdl_wait();
+  const double2* x2 = reinterpret_cast<const double2*>(x);
+  const long long n2 = n >> 1, step = (long long)gridDim.x * 256;
+  int m = 0;
+  long long i = blockIdx.x * 256ll + threadIdx.x;
+  for (; i + 3 * step < n2; i += 4 * step) {
+    double2 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = x2[i + u * step];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) m = max(m, max(biased_exp(v[u].x), biased_exp(v[u].y)));
+  }
+  for (; i < n2; i += step) {
+    const double2 v = x2[i];
+    m = max(m, max(biased_exp(v.x), biased_exp(v.y)));
+  }
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) m = max(m, biased_exp(x[n - 1]));
+  m = block_max(m);
+  if (threadIdx.x == 0) part[blockIdx.x] = m;
+}
+
+// the largest exponent from k_exp_max's partial results, in every thread; CTA
+// 0 leaves it in emax[0] for the kernels after this one
+__device__ __forceinline__ int finish_exp(const int* __restrict__ part, int npart, int* emax) {
+  int m = 0;
+  for (int i = threadIdx.x; i < npart; i += blockDim.x) m = max(m, part[i]);
+  m = block_max(m);
+  if (blockIdx.x == 0 && threadIdx.x == 0) emax[0] = m;
+  return m;
+}
+
+// |x| < 2^E with E = emax - 1022; X = round(x * 2^(P - E)).  Bound by HBM
+// (16 bytes per element): 16-byte accesses, four in flight per thread; 601 M
+// elements 1.80 -> 1.46 ms (6.6 TB/s) against one 8-byte access at a time.
+__global__ void __launch_bounds__(256) k_to_fixed(const double* __restrict__ x, long long* __restrict__ X, long long n,
+                                                  const int* __restrict__ part, int npart, int* emax, int P) {
+  pdl_wait();
+  const int sh = P - (finish_exp(part, npart, emax) - 1022);
+  const double2* x2 = reinterpret_cast<const double2*>(x);
+  longlong2* X2 = reinterpret_cast<longlong2*>(X);
+  const long long n2 = n >> 1, step = (long long)gridDim.x * 256;
+  long long i = blockIdx.x * 256ll + threadIdx.x;
+  for (; i + 3 * step < n2; i += 4 * step) {
+    double2 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = x2[i + u * step];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) X2[i + u * step] = make_longlong2(to_fixed(v[u].x, sh), to_fixed(v[u].y, sh));
+  }
+  for (; i < n2; i += step) {
+    const double2 v = x2[i];
+    X2[i] = make_longlong2(to_fixed(v.x, sh), to_fixed(v.y, sh));
+  }
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) X[n - 1] = to_fixed(x[n - 1], sh);
 }
 
 // R rows of the staged group at one column: one 16-byte shared-memory access
@@ -108,10 +172,14 @@ __device__ __forceinline__ float ldg_if(const float* p, bool on) { return on ? _
 // tensor cores that could take the terms inside a group of sites would cost
 // about 28 instructions per state and group for the split and the
 // recombination, as much as the gathers they replace.
-template <class Pol, int R, int NT>
+// CVT (contexts without cross terms): the rows are staged from the FP64 input
+// and converted on the way; the fixed-point copy xw, which only the panel
+// pass then reads, is written here instead of by k_to_fixed.
+template <class Pol, int R, int NT, bool CVT>
 __global__ void __launch_bounds__(NT, 1024 / NT)
-    k_row5(P3 p, const long long* __restrict__ grp_start, long long n_groups, const typename Pol::S* __restrict__ x,
-           typename Pol::Y* __restrict__ y, const int* __restrict__ emax) {
+    k_row5(P3 p, const long long* __restrict__ grp_start, long long n_groups,
+           const std::conditional_t<CVT, double, typename Pol::S>* __restrict__ x, typename Pol::Y* __restrict__ y,
+           int* emax, typename Pol::S* __restrict__ xw, const int* __restrict__ part, int npart) {
   using S = typename Pol::S;
   using V = RowVec<S, R>;
   static_assert(sizeof(V) == 16, "one 16-byte word per column");
@@ -123,8 +191,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
   __shared__ unsigned s_ax[kMaxOct][R], s_vm[kMaxOct][R];
   const Dev3& t = p.t;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int e2 = emax ? out_exp(t, emax) : 0;
-  const int n_oct = p.ncross ? (t.xs_ok ? t.n_oct : 1) : 0;
+  pdl_wait();
+  int sh = 0, e2 = 0;
+  if constexpr (CVT) {
+    const int em = finish_exp(part, npart, emax);
+    sh = t.P - (em - 1022);
+    e2 = out_exp(t, em);
+  } else {
+    e2 = emax ? out_exp(t, emax[0]) : 0;
+  }
+  const int n_oct = !CVT && p.ncross ? (t.xs_ok ? t.n_oct : 1) : 0;
   for (long long g = blockIdx.x; g < n_groups; g += gridDim.x) {
     const int bi = find_blk(grp_start, p.nblk, g);
     const DevBlock bl = p.blocks[bi];
@@ -134,13 +210,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     const long long row0 = bl.off + a0 * dB;
     __syncthreads();  // the previous group's columns are done
     {
-      const S* r0 = x + row0;
+      const auto* r0 = x + row0;
 #pragma unroll 4
       for (int b = threadIdx.x; b < dB; b += NT) {
         V w;
 #pragma unroll
-        for (int r = 0; r < R; ++r) w.v[r] = r < nr ? r0[(long long)r * dB + b] : (S)0;
+        for (int r = 0; r < R; ++r) {
+          if constexpr (CVT) w.v[r] = r < nr ? to_fixed(r0[(long long)r * dB + b], sh) : 0;
+          else w.v[r] = r < nr ? r0[(long long)r * dB + b] : (S)0;
+        }
         xs[b] = w;
+        if constexpr (CVT) {
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+            if (r < nr && bl.has_hA) xw[row0 + (long long)r * dB + b] = w.v[r];
+        }
       }
       if (threadIdx.x < 8) {  // zero slots addressed by the padding indices, one per bank group
         V w;
@@ -160,7 +244,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
         if (sb >= 0) {
           const DevBlock& so = p.blocks[sb];
           const unsigned rr = t.mapA[(long long)t.bond_ia[k] * t.A_total + gA];
-          if (rr != 0xFFFFu) sp = x + so.off + (long long)rr * so.dB;
+          if constexpr (!CVT)
+            if (rr != 0xFFFFu) sp = x + so.off + (long long)rr * so.dB;
         }
       }
       s_ptr[h][lane][r] = sp;
@@ -177,7 +262,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
       const DevBlock& nb = p.blocks[bn];
       const long long an = (gn - grp_start[bn]) * R;
       const char* p0 = reinterpret_cast<const char*>(x + nb.off + an * nb.dB);
-      const char* p1 = p0 + (size_t)(min((long long)R, nb.dA - an) * nb.dB) * sizeof(S);
+      const char* p1 = p0 + (size_t)(min((long long)R, nb.dA - an) * nb.dB) * sizeof(*x);
       const char* q0 = reinterpret_cast<const char*>(((uintptr_t)p0 + 15) & ~(uintptr_t)15);
       const char* q1 = reinterpret_cast<const char*>((uintptr_t)p1 & ~(uintptr_t)15);
       if (q1 > q0) l2_prefetch(q0, (unsigned)(q1 - q0));
@@ -190,7 +275,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
       pa[r] = t.A_pack[gA];
       da[r] = Pol::diagA(t, gA);
     }
-    const bool final_ = !bl.has_hA && !p.keep_fixed;
+    const bool final_ = !bl.has_hA;
     __syncthreads();
     const int nslab = (dB + 31) >> 5;
     for (int sl = warp; sl < nslab; sl += NT / 32) {
@@ -216,7 +301,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const unsigned z = t.vab_and ? (pa[r] & pb) : (pa[r] ^ pb);
-          acc[r] = Pol::dmul(da[r] + dbv + Pol::vab(t, z), xb.v[r]);
+          if constexpr (Pol::kSplit) acc[r] = 0;
+          else acc[r] = Pol::dmul(da[r] + dbv + Pol::vab(t, z), xb.v[r]);
         }
       }
 #pragma unroll
@@ -312,6 +398,15 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
 #pragma unroll
       for (int r = 0; r < R; ++r)
         if (in && r < nr) store_out<Pol>(y, row0 + (long long)r * dB + b, acc[r], final_, e2);
+      if constexpr (Pol::kSplit) {
+        if (final_ && in)  // no H_A pass: the FP64 diagonal is added here
+          for (int r = 0; r < nr; ++r) {
+            const long long i = row0 + (long long)r * dB + b;
+            double* yd = reinterpret_cast<double*>(y) + i;
+            const unsigned z = t.vab_and ? (pa[r] & pb) : (pa[r] ^ pb);
+            *yd = fma(PF64::diag(t, bl.gA0 + a0 + r, gB, z), p.xd[i], *yd);
+          }
+      }
     }
   }
 }
@@ -342,7 +437,16 @@ __global__ void __launch_bounds__(256, kPanelCtas) k_panel4(P3 p, const long lon
   constexpr int W = 32 * NC;
   const Dev3& t = p.t;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int e2 = emax ? out_exp(t, emax) : 0;
+  pdl_wait();
+  const int e2 = emax ? out_exp(t, emax[0]) : 0;
+  // split diagonal: the weighted popcounts of the packed cut words from a
+  // table (an FP64 conversion and product per element would double the FP64
+  // instructions, which bound this store)
+  __shared__ double s_vab[Pol::kSplit ? kMaxClasses : 1][33];
+  if constexpr (Pol::kSplit) {
+    for (int i = threadIdx.x; i < 33 * t.ncls_d; i += 256) s_vab[i / 33][i % 33] = t.dw64[i / 33] * (i % 33);
+    __syncthreads();
+  }
   const long long w = blockIdx.x;
   const int bi = find_blk(item_start, p.nblk, w);
   const DevBlock& bl = p.blocks[bi];
@@ -406,9 +510,32 @@ __global__ void __launch_bounds__(256, kPanelCtas) k_panel4(P3 p, const long lon
     };
     if (full) run(std::true_type{});
     else run(std::false_type{});
+    if constexpr (Pol::kSplit) {
+      const double da = t.A_d64[gA0 + a] + t.dc0_64;
+      const unsigned pa = t.A_pack[gA0 + a];
+      const double* xr = p.xd + (off + (long long)a * dB + b0);
+      double xv[NC], d[NC];
+      unsigned pb[NC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-      if (full || b0 + 32 * c < dB) store_out<Pol>(yrow, 32 * c, acc[c], true, e2);
+      for (int c = 0; c < NC; ++c) {
+        const bool in = full || b0 + 32 * c < dB;
+        xv[c] = in ? xr[32 * c] : 0.0;
+        d[c] = in ? t.B_d64[bl.gB0 + b0 + 32 * c] : 0.0;
+        pb[c] = in ? t.B_pack[bl.gB0 + b0 + 32 * c] : 0u;
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const unsigned z = t.vab_and ? (pa & pb[c]) : (pa ^ pb[c]);
+        double v = da + d[c];
+        for (int q = 0; q < t.ncls_d; ++q) v += s_vab[q][__popc(z & t.dmask[q])];
+        if (full || b0 + 32 * c < dB)
+          reinterpret_cast<double*>(yrow)[32 * c] = fma(v, xv[c], from_fixed(acc[c], e2));
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        if (full || b0 + 32 * c < dB) store_out<Pol>(yrow, 32 * c, acc[c], true, e2);
+    }
   }
 }
 
@@ -417,11 +544,9 @@ static P3 make_p3(const ed_ctx* c) {
   p.t = c->t3;
   p.blocks = c->d_blocks;
   p.cross = c->d_cross;
-  p.row_start = c->d_row_start;
   p.nblk = (int)c->blocks.size();
   p.ncross = c->kind == ED_SPIN ? (int)c->cross.size() : 0;
-  p.n_rows = c->n_rows;
-  p.keep_fixed = 0;
+  p.xd = nullptr;
   return p;
 }
 
@@ -432,6 +557,8 @@ static size_t v3_smem(const ed_ctx* c) {
   for (const auto& b : c->blocks) mdb = std::max<long long>(mdb, b.dB);
   return (size_t)(mdb + 8) * 16;
 }
+
+constexpr size_t kRowHalf = 106 * 1024;  // most row bytes for two CTAs of the row pass per SM
 
 bool v3_usable(const ed_ctx* c, ed_dtype dt, const void* x) {
   (void)dt;
@@ -456,11 +583,34 @@ struct ProfMarks {
   }
 };
 
-template <class Pol>
-static ed_status run_v3(ed_ctx* c, const typename Pol::S* x, typename Pol::Y* y, const int* emax, cudaStream_t st,
-                        ProfMarks& pm) {
+// kernel launch with programmatic stream serialization (see pdl_wait)
+template <class... KArgs, class... Args>
+static cudaError_t launch_pdl(void (*k)(KArgs...), long long grid, int block, size_t smem, cudaStream_t st,
+                              Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
+}
+
+constexpr int kExpParts = 2048;  // partial exponents of k_exp_max, behind the first 16 ints of the scratch
+
+// x: the pass's input (CVT: the FP64 vector, whose fixed-point copy goes to
+// xw); xd: the FP64 vector of a split diagonal
+template <class Pol, bool CVT = false>
+static ed_status run_v3(ed_ctx* c, const std::conditional_t<CVT, double, typename Pol::S>* x, typename Pol::Y* y,
+                        int* emax, cudaStream_t st, ProfMarks& pm, const double* xd = nullptr,
+                        typename Pol::S* xw = nullptr, const int* part = nullptr, int npart = 0) {
   P3 p = make_p3(c);
-  if (p.n_rows == 0) return ED_OK;
+  p.xd = xd;
+  if (c->n_rows == 0) return ED_OK;
   constexpr int R = 16 / (int)sizeof(typename Pol::S);
   const size_t smem = v3_smem(c);
   const int sms = n_sms(c->device);
@@ -474,73 +624,60 @@ static ed_status run_v3(ed_ctx* c, const typename Pol::S* x, typename Pol::Y* y,
     auto go = [&](auto kern, int nt) -> ed_status {
       ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       const long long grid = std::min<long long>(ng, (long long)sms * (1024 / nt));
-      kern<<<(unsigned)grid, nt, smem, st>>>(p, gs, ng, x, y, emax);
+      ED_CUDA_TRY(launch_pdl(kern, grid, nt, smem, st, p, gs, ng, x, y, emax, xw, part, npart));
       return ED_OK;
     };
-    if (smem > 106 * 1024) ED_TRY(go(k_row5<Pol, R, 1024>, 1024));
-    else if (smem > 50 * 1024) ED_TRY(go(k_row5<Pol, R, 512>, 512));
-    else ED_TRY(go(k_row5<Pol, R, 256>, 256));
+    if (smem > kRowHalf) ED_TRY(go(k_row5<Pol, R, 1024, CVT>, 1024));
+    else if (smem > 50 * 1024) ED_TRY(go(k_row5<Pol, R, 512, CVT>, 512));
+    else ED_TRY(go(k_row5<Pol, R, 256, CVT>, 256));
   }
-  ED_CUDA_TRY(cudaGetLastError());
   pm.mark(3, st);
   constexpr int q = sizeof(typename Pol::S) == 4 ? 1 : 0;
   if (c->n_panel[q] > 0) {
     // 1 KB of a row per panel: 128 columns of 8-byte types with four neighbour
     // rows in flight, 256 of FP32 with two
     const long long* is = c->d_panel_start + q * (c->blocks.size() + 1);
-    k_panel4<Pol, q ? 8 : 4, q ? 2 : 4><<<(unsigned)c->n_panel[q], 256, 0, st>>>(p, is, c->panel_rows[q], x, y, emax);
-    ED_CUDA_TRY(cudaGetLastError());
+    const typename Pol::S* xp;
+    if constexpr (CVT) xp = xw;
+    else xp = x;
+    ED_CUDA_TRY(launch_pdl(k_panel4<Pol, q ? 8 : 4, q ? 2 : 4>, c->n_panel[q], 256, 0, st, p, is, c->panel_rows[q], xp,
+                           y, (const int*)emax));
   }
   return ED_OK;
 }
 
-// exact fixed-point FP64 apply with explicit scratch: `fixed` holds D
-// 64-bit integers, `emax` one int (cleared here before use)
-// y += V x in FP64 after the integer passes of a split diagonal: per
-// element the side diagonals, the constant and the weighted popcounts of
-// the packed cut words (PF64::diag), one CTA per row, grid-stride
-__global__ void __launch_bounds__(256) k_diag_add(P3 p, const double* __restrict__ x, double* __restrict__ y) {
-  const Dev3& t = p.t;
-  for (long long r = blockIdx.x; r < p.n_rows; r += gridDim.x) {
-    const int bi = find_blk(p.row_start, p.nblk, r);
-    const DevBlock bl = p.blocks[bi];
-    const long long a = r - p.row_start[bi];
-    const long long gA = bl.gA0 + a;
-    const unsigned pa = t.A_pack[gA];
-    const long long base = bl.off + a * bl.dB;
-    for (long long b = threadIdx.x; b < bl.dB; b += blockDim.x) {
-      const long long gB = bl.gB0 + b;
-      const unsigned pb = t.B_pack[gB];
-      const unsigned z = t.vab_and ? (pa & pb) : (pa ^ pb);
-      y[base + b] = fma(PF64::diag(t, gA, gB, z), x[base + b], y[base + b]);
-    }
-  }
+// fixed-point passes of the context's arithmetic: x is the fixed-point copy
+// (CVT: the FP64 vector), xd the FP64 vector
+template <bool CVT>
+static ed_status run_fixed(ed_ctx* c, const std::conditional_t<CVT, double, long long>* x, const double* xd, double* y,
+                           int* emax, cudaStream_t st, ProfMarks& pm, long long* xw = nullptr,
+                           const int* part = nullptr, int npart = 0) {
+  if (c->diag_split) return run_v3<PI64S, CVT>(c, x, (long long*)y, emax, st, pm, xd, xw, part, npart);
+  if (c->dyadic) return run_v3<PI64, CVT>(c, x, (long long*)y, emax, st, pm, xd, xw, part, npart);
+  if (c->wide) return run_v3<PW, CVT>(c, x, y, emax, st, pm, xd, xw, part, npart);
+  return run_v3<PC64, CVT>(c, x, y, emax, st, pm, xd, xw, part, npart);
 }
 
-static ed_status diag_add(ed_ctx* c, const double* x, double* y, cudaStream_t st) {
-  if (!c->diag_split || c->n_rows < 1) return ED_OK;
-  const long long g = std::min<long long>(c->n_rows, (long long)n_sms(c->device) * 16);
-  k_diag_add<<<(unsigned)g, 256, 0, st>>>(make_p3(c), x, y);
-  ED_CUDA_TRY(cudaGetLastError());
-  return ED_OK;
-}
-
-static ed_status apply_fixed(ed_ctx* c, const double* x, double* y, long long* fixed, int* emax, cudaStream_t st,
-                             ProfMarks& pm) {
+// exact fixed-point FP64 apply with explicit scratch: `fixed` holds D 64-bit
+// integers; the exponents go through the context's exponent scratch
+static ed_status apply_fixed(ed_ctx* c, const double* x, double* y, long long* fixed, cudaStream_t st, ProfMarks& pm) {
   const long long n = c->D;
-  ED_CUDA_TRY(cudaMemsetAsync(emax, 0, sizeof(int), st));
+  if (n < 1) return ED_OK;
   const int sms = n_sms(c->device);
-  const long long g = std::min<long long>((n + 255) / 256, (long long)sms * 8);
+  int* emax = c->d_exp;
+  int* part = c->d_exp + 16;
+  const int g = (int)std::min<long long>({(n + 511) / 512, (long long)sms * 8, (long long)kExpParts});
   pm.mark(0, st);
-  k_exp_max<<<(unsigned)std::max<long long>(g, 1), 256, 0, st>>>(x, n, emax);
+  ED_CUDA_TRY(launch_pdl(k_exp_max, g, 256, 0, st, x, n, part));
   pm.mark(1, st);
-  k_to_fixed<<<(unsigned)std::max<long long>(g, 1), 256, 0, st>>>(x, fixed, n, emax, c->t3.P);
-  ED_CUDA_TRY(cudaGetLastError());
-  if (c->dyadic) {
-    ED_TRY(run_v3<PI64>(c, fixed, (long long*)y, emax, st, pm));
-    return diag_add(c, x, y, st);
-  }
-  return c->wide ? run_v3<PW>(c, fixed, y, emax, st, pm) : run_v3<PC64>(c, fixed, y, emax, st, pm);
+  // without cross terms only whole rows and the panel pass read the copy: the
+  // row pass makes it, where several CTAs per SM hide the conversion (12-site
+  // Hubbard ring 30 -> 26 us, 41 M-state impurity 0.45 -> 0.39 ms for the two;
+  // with one CTA per SM, Hubbard 4x4, it is 2.08 against 1.65 + 0.41 ms)
+  if ((c->kind != ED_SPIN || c->cross.empty()) && v3_smem(c) <= kRowHalf)
+    return run_fixed<true>(c, x, x, y, emax, st, pm, fixed, part, g);
+  ED_CUDA_TRY(launch_pdl(k_to_fixed, g, 256, 0, st, x, fixed, n, (const int*)part, g, emax, c->t3.P));
+  return run_fixed<false>(c, fixed, x, y, emax, st, pm);
 }
 
 // fixed-point input: exact integer sums, with small integer weights (dyadic
@@ -559,13 +696,7 @@ ed_status apply_prepared_fixed(ed_ctx* c, const double* x, double* y, cudaStream
   pm.begin(c);
   pm.mark(0, st);
   pm.mark(1, st);
-  ed_status r;
-  if (c->dyadic) {
-    r = run_v3<PI64>(c, c->d_fixed, (long long*)y, c->d_exp, st, pm);
-    if (r == ED_OK) r = diag_add(c, x, y, st);
-  } else {
-    r = c->wide ? run_v3<PW>(c, c->d_fixed, y, c->d_exp, st, pm) : run_v3<PC64>(c, c->d_fixed, y, c->d_exp, st, pm);
-  }
+  const ed_status r = run_fixed<false>(c, c->d_fixed, x, y, c->d_exp, st, pm);
   pm.mark(4, st);
   pm.end(c);
   return r;
@@ -583,7 +714,7 @@ ed_status apply_v3(ed_ctx* c, const void* x, void* y, ed_dtype dt, cudaStream_t 
   } else {
     // exact fixed point: exponent of max|x|, scaled copy, integer passes
     if (!c->d_fixed) ED_TRY(dev_alloc(c, (void**)&c->d_fixed, (size_t)std::max<long long>(c->D, 2) * 8));
-    r = apply_fixed(c, (const double*)x, (double*)y, c->d_fixed, c->d_exp, st, pm);
+    r = apply_fixed(c, (const double*)x, (double*)y, c->d_fixed, st, pm);
   }
   pm.mark(4, st);
   pm.end(c);
@@ -592,8 +723,9 @@ ed_status apply_v3(ed_ctx* c, const void* x, void* y, ed_dtype dt, cudaStream_t 
 
 // ---------------------------------------------------------------- apply without allocation
 
-// Scratch of ed_apply_H_noalloc: a file-scope device array (one int for the
-// exponent of max|x|, then the 64-bit fixed-point copy of x).  Every GPU
+// Scratch of ed_apply_H_noalloc: a file-scope device array (a header that the
+// size limit counts, then the 64-bit fixed-point copy of x; the exponents go
+// through the context's own scratch).  Every GPU
 // that loads this library holds it until the process exits.
 constexpr size_t kNoAllocScratchBytes = (size_t)32 << 20;
 constexpr size_t kNoAllocHeader = 256;
@@ -654,7 +786,7 @@ extern "C" ed_status ed_apply_H_noalloc(ed_ctx* c, const void* x, void* y, void*
   if (!fixed_mode(c)) return run_v3<PF64>(c, (const double*)x, (double*)y, nullptr, st, pm);
   unsigned char* base = nullptr;
   ED_TRY(noalloc_scratch(c->device, &base));
-  return apply_fixed(c, (const double*)x, (double*)y, (long long*)(base + kNoAllocHeader), (int*)base, st, pm);
+  return apply_fixed(c, (const double*)x, (double*)y, (long long*)(base + kNoAllocHeader), st, pm);
 }
 
 

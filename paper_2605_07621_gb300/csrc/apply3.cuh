@@ -15,17 +15,18 @@ struct P3 {
   Dev3 t;
   const DevBlock* blocks;
   const DevCross* cross;
-  const long long* row_start;
   int nblk;
   int ncross;
-  long long n_rows;
-  int keep_fixed;  // row pass leaves every row as a 64-bit partial sum (cross terms added later)
+  const double* xd;  // FP64 input of a split diagonal (PI64S)
 };
 
+// kSplit: the diagonal is not part of the integer sums; the last store of an
+// element adds it in FP64 from the FP64 input (P3::xd).
 // Policy types: S = staged / gathered values (and per-class sums), Y = the
 // partial output kept in y between the passes, A = the accumulator, D = the
 // diagonal, W = the per-class weights; dmul / wmul combine them.
 struct PF32 {
+  static constexpr bool kSplit = false;
   using S = float;
   using Y = float;
   using A = float;
@@ -49,6 +50,7 @@ struct PF32 {
   }
 };
 struct PF64 {
+  static constexpr bool kSplit = false;
   using S = double;
   using Y = double;
   using A = double;
@@ -75,6 +77,7 @@ struct PF64 {
 // magnitude (dyadic couplings), the diagonal a sum of three such terms and 32
 // such weights, so a product with x takes a 64 x 32-bit multiplication.
 struct PI64 {
+  static constexpr bool kSplit = false;
   using S = long long;
   using Y = long long;
   using A = long long;
@@ -93,6 +96,12 @@ struct PI64 {
   }
 };
 
+// dyadic off-diagonal terms with a diagonal that is not (disordered on-site
+// energies): the integer passes take the off-diagonal terms
+struct PI64S : PI64 {
+  static constexpr bool kSplit = true;
+};
+
 // Fixed-point gathers with FP64 weights (models whose couplings are not
 // dyadic): x is summed exactly per value class on the integer pipe as in
 // PI64, and each class sum is multiplied by its FP64 weight once per
@@ -100,6 +109,7 @@ struct PI64 {
 // of one per matrix element).  The partial result between the passes is FP64
 // in fixed-point units; the last store scales it by one power of two.
 struct PC64 {
+  static constexpr bool kSplit = false;
   using S = long long;
   using Y = double;
   using A = double;
@@ -155,6 +165,7 @@ struct AccW {
   }
 };
 struct PW {
+  static constexpr bool kSplit = false;
   using S = long long;
   using Y = double;
   using A = AccW;
@@ -278,7 +289,7 @@ __host__ __device__ __forceinline__ double from_fixed128(I128 v, int e2) {
   return bits_f64((s << 63) | ((unsigned long long)ex << 52) | (mant & 0xFFFFFFFFFFFFFull));
 }
 
-__device__ __forceinline__ int out_exp(const Dev3& t, const int* emax) { return (emax[0] - 1022) - t.P - t.q_shift; }
+__device__ __forceinline__ int out_exp(const Dev3& t, int emax) { return (emax - 1022) - t.P - t.q_shift; }
 
 template <class Pol>
 __device__ __forceinline__ void store_out(typename Pol::Y* y, long long i, typename Pol::A v, bool final_,
@@ -289,6 +300,10 @@ template <>
 __device__ __forceinline__ void store_out<PI64>(long long* y, long long i, long long v, bool final_, int e2) {
   if (final_) reinterpret_cast<double*>(y)[i] = from_fixed(v, e2);
   else y[i] = v;
+}
+template <>
+__device__ __forceinline__ void store_out<PI64S>(long long* y, long long i, long long v, bool final_, int e2) {
+  store_out<PI64>(y, i, v, final_, e2);
 }
 template <>
 __device__ __forceinline__ void store_out<PC64>(double* y, long long i, double v, bool final_, int e2) {

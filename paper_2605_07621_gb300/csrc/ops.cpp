@@ -541,7 +541,7 @@ static ed_status build_v3(ed_ctx* c, const HostSideOps& ha, const HostSideOps& h
   t.A_d32 = c->tab.A_diag32; t.B_d32 = c->tab.B_diag32; t.A_d64 = c->tab.A_diag; t.B_d64 = c->tab.B_diag;
   t.A_total = c->A.total();
   t.B_total = c->B.total();
-  ED_TRY(dev_alloc(c, (void**)&c->d_exp, 64));
+  ED_TRY(dev_alloc(c, (void**)&c->d_exp, (16 + 2048) * sizeof(int)));  // scalars, then partial exponents
   c->v3_ok = true;
   return ED_OK;
 }
