@@ -42,14 +42,6 @@ void host_mul_wide(long long a, long long b, long long* hi, unsigned long long* 
   *lo = v.lo;
 }
 
-// Programmatic dependent launch: the kernel is set up while the previous one
-// of the stream drains, and waits here until that one has finished and its
-// writes are visible.  Called before any access to global memory.  (H|psi> of
-// 12,870 / 853,776 states: 22.5 -> 16.3 / 32.8 -> 25.6 us.  Releasing the next
-// kernel earlier, by launch_dependents, costs the large sectors 7 %: its CTAs
-// take slots from the running kernel's last wave.)
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ int biased_exp(double v) {
   return (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffull);
 }
@@ -582,23 +574,6 @@ struct ProfMarks {
     for (auto& e : ev) c->prof_ev.push_back(e);
   }
 };
-
-// kernel launch with programmatic stream serialization (see pdl_wait)
-template <class... KArgs, class... Args>
-static cudaError_t launch_pdl(void (*k)(KArgs...), long long grid, int block, size_t smem, cudaStream_t st,
-                              Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
-}
 
 constexpr int kExpParts = 2048;  // partial exponents of k_exp_max, behind the first 16 ints of the scratch
 

@@ -231,21 +231,17 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
       ED_TRY(apply_H_impl(c, v, w, dtype_of<T>(), st));
     }
     launch_lz_a<T>(c, w, v, vprev, j > 0 ? 1 : 0, n, st);
-    if constexpr (std::is_same<T, double>::value) {
-      if (fuse)
-        launch_lz_b_emax(c, w, v, n, ew, st);
-      else
-        launch_lz_b<T>(c, w, v, n, st);
-    } else {
-      launch_lz_b<T>(c, w, v, n, st);
-    }
-    if (reorth && basis && basis->kind == BASIS_SAME && basis->complete && basis->count <= kMaxBasis) {
+    // lz_b writes the history entry itself unless an orthogonalisation follows
+    const bool full = reorth && basis && basis->kind == BASIS_SAME && basis->complete && basis->count <= kMaxBasis;
+    const bool part = pro && basis->complete && basis->count <= kMaxBasis;
+    launch_lz_b<T>(c, w, v, n, fuse ? ew : nullptr, full || part ? nullptr : hist, hcount, st);
+    if (full) {
       // classical Gram-Schmidt against all kept vectors, applied twice
       for (int pass = 0; pass < 2; ++pass)
         launch_reorth<T>(c, (const T*)basis->base, n, basis->count, w, n, hcoef(c), st);
       ED_TRY(dot_dev<T>(c, w, w, n, slot(c, 1), st, 1));
     }
-    if (pro && basis->complete && basis->count <= kMaxBasis) {
+    if (part) {
       double ab[2];
       ED_TRY(read_scalars(c, 0, 2, ab, st));  // alpha_j, beta_{j+1} (synchronises)
       anorm = std::max(anorm, std::fabs(ab[0]) + ab[1]);
@@ -259,7 +255,7 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
         ortho_now = true;
       }
     }
-    launch_hist_push(c, hist, hcount, st);
+    if (full || part) launch_hist_push(c, hist, hcount, st);
     ED_CUDA_TRY(cudaGetLastError());
     return ED_OK;
   };

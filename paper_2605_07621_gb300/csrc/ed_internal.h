@@ -275,7 +275,7 @@ struct ed_ctx {
   long long* d_panel_start = nullptr;  // class-sorted H_A pass, [8-byte types, FP32][block]: first item (plus total)
   long long n_panel[2] = {0, 0};
   int panel_rows[2] = {8, 8};        // rows per item
-  int* d_err = nullptr;              // set by kernels whose bounded waits ran out
+  int* d_err = nullptr;              // [0]: set by kernels whose bounded waits ran out; [2]: ticket of k_lz_a, k_lz_b
   // class-sorted path
   bool v3_ok = false;                // tables below are valid
   bool dyadic = false;               // FP64 apply may use exact fixed point

@@ -7,6 +7,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "apply3.cuh"
@@ -37,10 +38,37 @@ __global__ void k_dot(const T* __restrict__ a, const T* __restrict__ b, long lon
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// w -= beta * vprev (beta from device memory; skipped when use_beta == 0); alpha partial <v, w>
+// true in every thread of the CTA that is the last of its grid to arrive here
+// (a ticket on *ctr, left at zero again); what the other CTAs' thread 0 wrote
+// before is visible to it then.  Saves the separate one-CTA launch that sums
+// the partial results: a Lanczos step of 12,870 states took nine launches.
+__device__ __forceinline__ bool last_cta(unsigned* ctr) {
+  __shared__ unsigned s_last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(ctr, 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (s_last) {
+      *ctr = 0u;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return s_last != 0u;
+}
+
+// sum of the grid's partial results in a fixed order, valid in thread 0
+__device__ __forceinline__ double sum_parts(const double* part) {
+  double v = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(part + i);
+  return block_sum(v);
+}
+
+// w -= beta * vprev (beta from device memory; skipped when use_beta == 0);
+// alpha = <v, w>, summed by the last CTA
 template <typename T>
 __global__ void k_lz_a(T* __restrict__ w, const T* __restrict__ v, const T* __restrict__ vprev, const double* beta,
-                       int use_beta, long long n, double* part) {
+                       int use_beta, long long n, double* part, double* alpha, unsigned* ctr) {
+  pdl_wait();
   const T bt = use_beta ? (T)beta[0] : (T)0;
   DotAcc<T> acc;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -53,39 +81,63 @@ __global__ void k_lz_a(T* __restrict__ w, const T* __restrict__ v, const T* __re
   }
   double s = block_sum(acc.value());
   if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (!last_cta(ctr)) return;
+  s = sum_parts(part);
+  if (threadIdx.x == 0) alpha[0] = s;
 }
 
-// w -= alpha * v; partial ||w||^2
-template <typename T>
-__global__ void k_lz_b(T* __restrict__ w, const T* __restrict__ v, const double* alpha, long long n, double* part) {
+// w -= alpha * v; beta = ||w||, summed by the last CTA, which also appends
+// alpha and beta to the history hist (if any) at the step index *hcount (so
+// the same launch serves every step of a graph).  EMAX (FP64 with the exact
+// fixed-point H|psi>): the largest biased exponent of w into *ew, from the
+// CTAs' partial results epart.
+template <typename T, bool EMAX>
+__global__ void k_lz_b(T* __restrict__ w, const T* __restrict__ v, const double* alpha, long long n, double* part,
+                       double* beta, unsigned* ctr, double* hist, int* hcount, int* epart, int* ew) {
+  pdl_wait();
   const T al = (T)alpha[0];
   DotAcc<T> acc;
+  int em = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     T wi = w[i] - al * v[i];
     w[i] = wi;
     acc.add_prod(wi, wi);
+    if constexpr (EMAX) em = max(em, (int)(((unsigned long long)__double_as_longlong(wi) >> 52) & 0x7ffull));
+  }
+  __shared__ int s_em;
+  if constexpr (EMAX) {
+    if (threadIdx.x == 0) s_em = 0;
+    __syncthreads();
+    em = __reduce_max_sync(0xffffffffu, em);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_em, em);
   }
   double s = block_sum(acc.value());
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// FP64 with the exact fixed-point H|psi>: w -= alpha * v, partial ||w||^2,
-// and the largest biased exponent of w (atomic max into *ew, zeroed before)
-__global__ void k_lz_b_emax(double* __restrict__ w, const double* __restrict__ v, const double* alpha, long long n,
-                            double* part, int* ew) {
-  const double al = alpha[0];
-  DotAcc<double> acc;
-  int em = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const double wi = w[i] - al * v[i];
-    w[i] = wi;
-    acc.add_prod(wi, wi);
-    em = max(em, (int)(((unsigned long long)__double_as_longlong(wi) >> 52) & 0x7ffull));
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = s;
+    if constexpr (EMAX) {
+      epart[blockIdx.x] = s_em;
+      s_em = 0;
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) em = max(em, __shfl_down_sync(0xffffffffu, em, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(ew, em);
-  double s = block_sum(acc.value());
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (!last_cta(ctr)) return;
+  if constexpr (EMAX) {
+    em = 0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) em = max(em, __ldcg(epart + i));
+    em = __reduce_max_sync(0xffffffffu, em);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_em, em);
+  }
+  s = sum_parts(part);
+  if (threadIdx.x == 0) {
+    const double b = sqrt(s > 0.0 ? s : 0.0);
+    beta[0] = b;
+    if constexpr (EMAX) *ew = s_em;
+    if (hist) {
+      const int j = *hcount;
+      hist[2 * j] = alpha[0];
+      hist[2 * j + 1] = b;
+      *hcount = j + 1;
+    }
+  }
 }
 
 // out = w / beta, and the fixed-point copy X of out that the next H|psi>
@@ -94,6 +146,7 @@ __global__ void k_lz_b_emax(double* __restrict__ w, const double* __restrict__ v
 // (E + 1022) goes to *ex for the apply's output scale
 __global__ void k_lz_c_fixed(const double* __restrict__ w, double* __restrict__ out, long long* __restrict__ X,
                              const double* beta, const int* ew, int* ex, int P, long long n) {
+  pdl_wait();
   const double b = beta[0];
   const double inv = b > 0.0 ? 1.0 / b : 0.0;
   const int eb = (int)(((unsigned long long)__double_as_longlong(b) >> 52) & 0x7ffull);
@@ -110,6 +163,7 @@ __global__ void k_lz_c_fixed(const double* __restrict__ w, double* __restrict__ 
 // out = w / beta
 template <typename T>
 __global__ void k_lz_c(const T* __restrict__ w, T* __restrict__ out, const double* beta, long long n) {
+  pdl_wait();
   const double b = beta[0];
   const T inv = (T)(b > 0.0 ? 1.0 / b : 0.0);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -164,8 +218,8 @@ __global__ void k_axpy_basis(const TB* __restrict__ v, TO* __restrict__ x, doubl
     x[i] = from_d<TO>(to_d(x[i]) + s * to_d(v[i]));
 }
 
-// appends this step's alpha and beta to the device history at the step
-// index the device keeps (so the same launch serves every step of a graph)
+// the same history entry as k_lz_b's, for steps whose vector is orthogonalised
+// after it
 __global__ void k_hist_push(const double* __restrict__ sl, double* __restrict__ hist, int* counter) {
   const int j = *counter;
   hist[2 * j] = sl[0];
@@ -461,29 +515,31 @@ void tridiag_vector(const double* a, const double* b, int m, double theta, std::
 
 template <typename T>
 void launch_lz_a(ed_ctx* c, T* w, const T* v, const T* vprev, int use_beta, long long n, cudaStream_t st) {
-  int g = grid_for(c, n);
-  k_lz_a<T><<<g, kRedThreads, 0, st>>>(w, v, vprev, slot(c, 1), use_beta, n, c->d_partials);
-  k_finalize<<<1, kRedThreads, 0, st>>>(c->d_partials, g, slot(c, 0), 0);
+  launch_pdl(k_lz_a<T>, grid_for(c, n), kRedThreads, 0, st, w, v, vprev, slot(c, 1), use_beta, n, c->d_partials,
+             slot(c, 0), (unsigned*)c->d_err + 2);
 }
 template <typename T>
-void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, cudaStream_t st) {
-  int g = grid_for(c, n);
-  k_lz_b<T><<<g, kRedThreads, 0, st>>>(w, v, slot(c, 0), n, c->d_partials);
-  k_finalize<<<1, kRedThreads, 0, st>>>(c->d_partials, g, slot(c, 1), 1);
+void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, int* ew, double* hist, int* hcount, cudaStream_t st) {
+  const int g = grid_for(c, n);
+  double *alpha = slot(c, 0), *beta = slot(c, 1);
+  unsigned* ctr = (unsigned*)c->d_err + 2;
+  if constexpr (std::is_same<T, double>::value) {
+    if (ew) {
+      launch_pdl(k_lz_b<T, true>, g, kRedThreads, 0, st, w, v, alpha, n, c->d_partials, beta, ctr, hist, hcount,
+                 c->d_exp + 16, ew);
+      return;
+    }
+  }
+  launch_pdl(k_lz_b<T, false>, g, kRedThreads, 0, st, w, v, alpha, n, c->d_partials, beta, ctr, hist, hcount,
+             (int*)nullptr, (int*)nullptr);
 }
 template <typename T>
 void launch_lz_c(ed_ctx* c, const T* w, T* out, long long n, cudaStream_t st) {
-  k_lz_c<T><<<grid_for(c, n), kRedThreads, 0, st>>>(w, out, slot(c, 1), n);
-}
-void launch_lz_b_emax(ed_ctx* c, double* w, const double* v, long long n, int* ew, cudaStream_t st) {
-  int g = grid_for(c, n);
-  cudaMemsetAsync(ew, 0, sizeof(int), st);
-  k_lz_b_emax<<<g, kRedThreads, 0, st>>>(w, v, slot(c, 0), n, c->d_partials, ew);
-  k_finalize<<<1, kRedThreads, 0, st>>>(c->d_partials, g, slot(c, 1), 1);
+  launch_pdl(k_lz_c<T>, grid_for(c, n), kRedThreads, 0, st, w, out, slot(c, 1), n);
 }
 void launch_lz_c_fixed(ed_ctx* c, const double* w, double* out, long long* X, const int* ew, int* ex, long long n,
                        cudaStream_t st) {
-  k_lz_c_fixed<<<grid_for(c, n), kRedThreads, 0, st>>>(w, out, X, slot(c, 1), ew, ex, c->t3.P, n);
+  launch_pdl(k_lz_c_fixed, grid_for(c, n), kRedThreads, 0, st, w, out, X, slot(c, 1), ew, ex, c->t3.P, n);
 }
 template <typename T>
 void launch_lz_rerun(ed_ctx* c, const T* w, const T* v, const T* vprev, double alpha, double beta, double inv_next,
@@ -555,7 +611,7 @@ void launch_fermion_remap(ed_ctx* c, const double* psi, long long dA_src, long l
 
 #define ED_INST(T)                                                                                        \
   template void launch_lz_a<T>(ed_ctx*, T*, const T*, const T*, int, long long, cudaStream_t);          \
-  template void launch_lz_b<T>(ed_ctx*, T*, const T*, long long, cudaStream_t);                         \
+  template void launch_lz_b<T>(ed_ctx*, T*, const T*, long long, int*, double*, int*, cudaStream_t);    \
   template void launch_lz_c<T>(ed_ctx*, const T*, T*, long long, cudaStream_t);                        \
   template void launch_lz_rerun<T>(ed_ctx*, const T*, const T*, const T*, double, double, double, T*,   \
                                    long long, cudaStream_t);                                            \

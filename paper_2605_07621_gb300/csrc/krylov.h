@@ -25,17 +25,17 @@ ed_status read_scalars(ed_ctx* c, int first, int count, double* out, cudaStream_
 double tridiag_lowest(const double* a, const double* b, int m);
 void tridiag_vector(const double* a, const double* b, int m, double theta, std::vector<double>& s);
 
-// kernel launchers (krylov_launch.cu)
+// kernel launchers.  lz_a: alpha to slot 0; lz_b: beta to slot 1, and the
+// history entry j = *hcount of the step when hist is not NULL
 template <typename T>
 void launch_lz_a(ed_ctx* c, T* w, const T* v, const T* vprev, int use_beta, long long n, cudaStream_t st);
 template <typename T>
-void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, cudaStream_t st);
+void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, int* ew, double* hist, int* hcount, cudaStream_t st);
 template <typename T>
 void launch_lz_c(ed_ctx* c, const T* w, T* out, long long n, cudaStream_t st);
 // FP64 Lanczos steps that hand the next H|psi> its fixed-point input:
-// lz_b also records the largest exponent of w in *ew; lz_c also writes the
+// lz_b (ew not NULL) also records the largest exponent of w; lz_c also writes the
 // fixed-point copy X of w / beta and its scale (biased exponent) to *ex
-void launch_lz_b_emax(ed_ctx* c, double* w, const double* v, long long n, int* ew, cudaStream_t st);
 void launch_lz_c_fixed(ed_ctx* c, const double* w, double* out, long long* X, const int* ew, int* ex, long long n,
                        cudaStream_t st);
 // H|psi> of the exact fixed-point path from an input already converted

@@ -680,7 +680,7 @@ extern "C" ed_status ed_build_local_ops(ed_ctx* c, int flags) {
     ED_TRY(upload(c, &c->d_panel_start, ps));
   }
   {
-    std::vector<int> z(4, 0);
+    std::vector<int> z(8, 0);
     ED_TRY(upload(c, &c->d_err, z));
   }
   ED_TRY(build_v3(c, ha, hb));
