@@ -58,59 +58,79 @@ constexpr long long kGraphStates = 1ll << 22;
 // Green's function runs re-orthogonalise only sectors up to this size
 constexpr long long kGfReorthStates = 1ll << 22;
 
-// Lanczos basis kept on the device as one contiguous array of `cap`
-// vectors (same type as the recurrence, or BF16 when only a restart vector
-// is needed).  When it does not fit the budget the vectors are recomputed
-// in a second pass instead.
+// Lanczos basis kept on the device (same type as the recurrence, or BF16
+// when only a restart vector is needed), at most `cap` vectors.  `whole`: one
+// contiguous array, as the orthogonalisation kernels need it; otherwise
+// chunks of `per` vectors allocated as the run reaches them (allocating the
+// 401 vectors that a run may need but seldom does took 30 of 130 ms on a
+// 40 M-state sector).  When it does not fit the budget the vectors are
+// recomputed in a second pass instead.
+constexpr int kBasisPer = 32;
+constexpr size_t kBasisWhole = (size_t)256 << 20;  // up to this size in one piece
+
 struct Basis {
   BasisKind kind = BASIS_NONE;
   size_t elem = 0;
   long long n = 0;
-  int cap = 0, count = 0;
+  int cap = 0, count = 0, per = 0;
   bool complete = false;
-  void* base = nullptr;
-  ~Basis() {
-    if (base) cudaFree(base);
-  }
-  bool init(BasisKind k, size_t e, long long len, int capacity, size_t budget) {
+  std::vector<void*> chunks;
+  ~Basis() { release(); }
+  bool init(BasisKind k, size_t e, long long len, int capacity, size_t budget, bool whole = false) {
+    release();
     kind = k;
     elem = e;
     n = len;
     cap = capacity;
-    count = 0;
-    complete = false;
     if (k == BASIS_NONE || capacity <= 0 || len <= 0) return false;
     // as many vectors as fit the budget; a longer run falls back to a second pass
-    const size_t per = (size_t)len * e;
-    if ((size_t)capacity * per > budget) capacity = (int)(budget / per);
+    const size_t bytes = (size_t)len * e;
+    if ((size_t)capacity * bytes > budget) capacity = (int)(budget / bytes);
     if (capacity < 2) return false;
     cap = capacity;
-    size_t bytes = (size_t)capacity * per;
-    if (cudaMalloc(&base, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      base = nullptr;
-      return false;
+    per = whole || (size_t)capacity * bytes <= kBasisWhole ? capacity : std::min(capacity, kBasisPer);
+    complete = reserve(0);
+    return complete;
+  }
+  // memory for vector j (called in ascending j); false: out of it
+  bool reserve(int j) {
+    if (j >= cap) return false;
+    while ((int)chunks.size() <= j / per) {
+      void* p = nullptr;
+      const int first = (int)chunks.size() * per;
+      if (cudaMalloc(&p, (size_t)std::min(per, cap - first) * (size_t)n * elem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+      }
+      chunks.push_back(p);
     }
-    complete = true;
     return true;
   }
-  void* at(int j) const { return (char*)base + (size_t)j * (size_t)n * elem; }
+  void* at(int j) const { return (char*)chunks[j / per] + (size_t)(j % per) * (size_t)n * elem; }
+  const void* whole() const { return chunks[0]; }
   void release() {
-    if (base) cudaFree(base);
-    base = nullptr;
+    for (void* p : chunks) cudaFree(p);
+    chunks.clear();
     complete = false;
     count = 0;
   }
 };
 
+// the place of the next basis vector, or null (and the basis is incomplete)
+// when there is none
+void* basis_next(Basis* B) {
+  if (!B || !B->complete) return nullptr;
+  if (!B->reserve(B->count)) {
+    B->complete = false;
+    return nullptr;
+  }
+  return B->at(B->count++);
+}
+
 template <typename T>
 void basis_store(ed_ctx* c, Basis* B, const T* v, long long n, cudaStream_t st) {
-  if (!B || !B->complete) return;
-  if (B->count >= B->cap) {
-    B->complete = false;
-    return;
-  }
-  void* p = B->at(B->count++);
+  void* p = basis_next(B);
+  if (!p) return;
   if (B->kind == BASIS_SAME)
     cudaMemcpyAsync(p, v, (size_t)n * sizeof(T), cudaMemcpyDeviceToDevice, st);
   else
@@ -238,7 +258,7 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     if (full) {
       // classical Gram-Schmidt against all kept vectors, applied twice
       for (int pass = 0; pass < 2; ++pass)
-        launch_reorth<T>(c, (const T*)basis->base, n, basis->count, w, n, hcoef(c), st);
+        launch_reorth<T>(c, (const T*)basis->whole(), n, basis->count, w, n, hcoef(c), st);
       ED_TRY(dot_dev<T>(c, w, w, n, slot(c, 1), st, 1));
     }
     if (part) {
@@ -247,7 +267,7 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
       anorm = std::max(anorm, std::fabs(ab[0]) + ab[1]);
       if (om.need(ab[0], ab[1], anorm)) {
         for (int pass = 0; pass < 2; ++pass)
-          launch_reorth<T>(c, (const T*)basis->base, n, basis->count, w, n, hcoef(c), st);
+          launch_reorth<T>(c, (const T*)basis->whole(), n, basis->count, w, n, hcoef(c), st);
         ED_TRY(dot_dev<T>(c, w, w, n, slot(c, 1), st, 1));
         double bn;
         ED_TRY(read_scalars(c, 1, 1, &bn, st));
@@ -259,22 +279,30 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     ED_CUDA_TRY(cudaGetLastError());
     return ED_OK;
   };
-  // the rest of the step: the next Lanczos vector (and its fixed-point copy)
+  // the rest of the step: the next Lanczos vector (and its fixed-point copy),
+  // written to its place in the basis where one of the same type is kept (and
+  // its rows are 16-byte aligned, as H|psi> wants its input), else to the
+  // caller's buffer that does not hold v
+  const bool in_place = basis && basis->kind == BASIS_SAME && (n * (long long)sizeof(T)) % 16 == 0;
   auto tail = [&](bool ortho_now) {
+    T* out = in_place ? (T*)basis_next(basis) : nullptr;
+    const bool stored = out != nullptr;
+    if (!out) out = v == bufs[0] ? bufs[1] : bufs[0];
     if constexpr (std::is_same<T, double>::value) {
       // (after an orthogonalisation the exponent lz_b recorded may be stale)
       if (fuse && c->d_fixed && !ortho_now) {
-        launch_lz_c_fixed(c, w, vprev, c->d_fixed, ew, c->d_exp, n, st);
+        launch_lz_c_fixed(c, w, out, c->d_fixed, ew, c->d_exp, n, st);
         prepared = true;
       } else {
-        launch_lz_c<T>(c, w, vprev, n, st);
+        launch_lz_c<T>(c, w, out, n, st);
         prepared = false;
       }
     } else {
-      launch_lz_c<T>(c, w, vprev, n, st);
+      launch_lz_c<T>(c, w, out, n, st);
     }
-    std::swap(vprev, v);
-    basis_store<T>(c, basis, v, n, st);
+    vprev = v;
+    v = out;
+    if (!stored && !in_place) basis_store<T>(c, basis, v, n, st);
   };
   // read the scalars of the steps since the last read and examine them in order
   auto examine = [&](int m) -> ed_status {
@@ -394,8 +422,6 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
   out.theta = tridiag_lowest(out.alpha.data(), out.beta.data(), steps);
   out.orthogonalised = pro ? om.count : (reorth ? steps : 0);
   if (basis && basis->count > steps) basis->count = steps;
-  bufs[0] = vprev;
-  bufs[1] = v;
   return ED_OK;
 }
 
@@ -408,11 +434,11 @@ ed_status lz_vector(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, const R
   std::vector<double> s;
   tridiag_vector(r.alpha.data(), r.beta.data(), m, r.theta, s);
   const bool combine = std::is_same<T, float>::value && basis && basis->complete && basis->count >= m &&
-                       basis->kind == BASIS_SAME && m <= kMaxBasis;
+                       basis->kind == BASIS_SAME && m <= kMaxBasis && (int)basis->chunks.size() <= kMaxChunks;
   if (!combine) ED_CUDA_TRY(cudaMemsetAsync(x, 0, (size_t)n * sizeof(double), st));
   if (combine) {
     // one pass over the stored FP32 vectors, float-float sums
-    ED_TRY(launch_combine_f32(c, (const float*)basis->base, n, s.data(), m, x, st));
+    ED_TRY(launch_combine_f32(c, basis->chunks.data(), (int)basis->chunks.size(), basis->per, n, s.data(), m, x, st));
   } else if (basis && basis->complete && basis->count >= m) {
     for (int j = 0; j < m; ++j) {
       if (basis->kind == BASIS_BF16)
@@ -534,7 +560,7 @@ extern "C" ed_status ed_lanczos_ground(ed_ctx* c, const ed_lanczos_opts* opts_in
     double* bufs[3];
     for (auto& b : bufs) ED_TRY(mem.get((void**)&b, n * sizeof(double)));
     Basis B;
-    if (o.reorth || want_vec) B.init(BASIS_SAME, sizeof(double), n, max_iter + 1, budget);
+    if (o.reorth || want_vec) B.init(BASIS_SAME, sizeof(double), n, max_iter + 1, budget, o.reorth != 0);
     RunOut r;
     ED_TRY(lz_run<double>(c, st, bufs, v0, max_iter, o.tol, o.check_every, o.fixed_iter != 0, o.reorth != 0, &B, r,
                           want_vec ? kVecResid : 0.0));
@@ -565,7 +591,7 @@ extern "C" ed_status ed_lanczos_ground(ed_ctx* c, const ed_lanczos_opts* opts_in
       const size_t later = (size_t)n * sizeof(double) * (mixed ? 6 : 2) + ((size_t)1 << 30);
       const size_t fr = free_device_bytes();
       const size_t budget32 = fr > later ? fr - later : 0;
-      if (!B.init(BASIS_SAME, sizeof(float), n, max_iter + 1, budget32) && !o.reorth)
+      if (!B.init(BASIS_SAME, sizeof(float), n, max_iter + 1, budget32, o.reorth != 0) && !o.reorth)
         B.init(BASIS_BF16, 2, n, max_iter + 1, budget32);
     }
     // mixed: the FP32 run goes on until its Ritz vector is close to the
@@ -758,7 +784,7 @@ extern "C" ed_status ed_lanczos_gf(ed_ctx* c, const void* psi0, double e0, int s
     const bool want = reorth != ED_GF_REORTH_NONE;
     const bool fits = want && steps <= kMaxBasis &&
                       (size_t)(steps + 1) * (size_t)n2 * sizeof(double) <= free_device_bytes() / 2 &&
-                      B.init(BASIS_SAME, sizeof(double), n2, steps + 1, free_device_bytes() / 2) &&
+                      B.init(BASIS_SAME, sizeof(double), n2, steps + 1, free_device_bytes() / 2, true) &&
                       B.cap >= steps + 1;
     if (!fits && (reorth == ED_GF_REORTH_FULL || reorth == ED_GF_REORTH_PARTIAL)) {
       set_error("the Krylov basis (%d x %lld states) does not fit in half of the free device memory", steps + 1,

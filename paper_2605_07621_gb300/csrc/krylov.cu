@@ -244,22 +244,30 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float2 c, float v) 
   lo = __fadd_rn(lo, __fadd_rn(e, pe));
 }
 
-__global__ void k_combine_f32(const float* __restrict__ V, long long n, int m, const float2* __restrict__ s,
+struct BasisChunks {
+  const float* p[kMaxChunks];
+};
+
+__global__ void k_combine_f32(BasisChunks V, int per, long long n, int m, const float2* __restrict__ s,
                               double* __restrict__ x) {
   extern __shared__ float2 sc[];
   for (int j = threadIdx.x; j < m; j += blockDim.x) sc[j] = s[j];
   __syncthreads();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     float hi = 0.f, lo = 0.f;
-    int j = 0;
-    for (; j + 4 <= m; j += 4) {
-      float v[4];
+    for (int q = 0; q * per < m; ++q) {
+      const float* vq = V.p[q] + i;
+      const int j0 = q * per, jn = min(per, m - j0);
+      int j = 0;
+      for (; j + 4 <= jn; j += 4) {
+        float v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = __ldg(V + (long long)(j + u) * n + i);
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(vq + (long long)(j + u) * n);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) ff_acc(hi, lo, sc[j + u], v[u]);
+        for (int u = 0; u < 4; ++u) ff_acc(hi, lo, sc[j0 + j + u], v[u]);
+      }
+      for (; j < jn; ++j) ff_acc(hi, lo, sc[j0 + j], __ldg(vq + (long long)j * n));
     }
-    for (; j < m; ++j) ff_acc(hi, lo, sc[j], __ldg(V + (long long)j * n + i));
     x[i] = (double)hi + (double)lo;
   }
 }
@@ -554,9 +562,9 @@ template <typename TB, typename TO>
 void launch_axpy_basis(ed_ctx* c, const TB* v, TO* x, double s, long long n, cudaStream_t st) {
   k_axpy_basis<TB, TO><<<grid_for(c, n), kRedThreads, 0, st>>>(v, x, s, n);
 }
-ed_status launch_combine_f32(ed_ctx* c, const float* V, long long n, const double* s, int m, double* x,
-                             cudaStream_t st) {
-  if (m < 1 || m > kMaxBasis) {
+ed_status launch_combine_f32(ed_ctx* c, void* const* chunks, int nchunks, int per, long long n, const double* s, int m,
+                             double* x, cudaStream_t st) {
+  if (m < 1 || m > kMaxBasis || nchunks > kMaxChunks || per < 1 || (long long)nchunks * per < m) {
     set_error("basis combination of %d vectors outside 1..%d", m, kMaxBasis);
     return ED_EINVAL;
   }
@@ -569,7 +577,9 @@ ed_status launch_combine_f32(ed_ctx* c, const float* V, long long n, const doubl
   // (kMaxBasis 8-byte slots)
   float2* d = reinterpret_cast<float2*>(hcoef(c));
   ED_CUDA_TRY(cudaMemcpyAsync(d, h.data(), (size_t)m * sizeof(float2), cudaMemcpyHostToDevice, st));
-  k_combine_f32<<<grid_for(c, n), kRedThreads, (size_t)m * sizeof(float2), st>>>(V, n, m, d, x);
+  BasisChunks V{};
+  for (int q = 0; q < nchunks; ++q) V.p[q] = (const float*)chunks[q];
+  k_combine_f32<<<grid_for(c, n), kRedThreads, (size_t)m * sizeof(float2), st>>>(V, per, n, m, d, x);
   ED_CUDA_TRY(cudaGetLastError());
   return ED_OK;
 }
