@@ -11,6 +11,7 @@
 // splits the blocks of x (as rows for Psi H_R^T, as columns for H_L Psi and
 // L Psi) and the intermediate L Psi, and every stage is one launch over all
 // blocks.
+#include <algorithm>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -185,6 +186,8 @@ extern "C" ed_status ed_dense_create(int nq, const int64_t* chi, const double* c
     return put(by_cols ? 1 : 0, v.data(), v.size() * sizeof(OzSliceJob), (int)v.size(), u);
   };
   auto products = [&](std::vector<OzProblem>& v) -> ed_status {
+    // longest tiles first, so that the launch does not end with them
+    std::stable_sort(v.begin(), v.end(), [](const OzProblem& a, const OzProblem& b) { return a.K > b.K; });
     long long tiles = 0;
     for (auto& p : v) {
       p.tile0 = tiles;

@@ -345,7 +345,7 @@ ed_status oz_slice(OzContext* o, const OzSliceJob* d_jobs, int njobs, long long 
 // ---------------------------------------------------------------- the GEMM
 
 constexpr int kOzThreads = 192;          // warps 0-3 epilogue, 4 TMA producer, 5 MMA issuer
-constexpr int kOzAStages = 3;
+constexpr int kOzAStages = 6;
 constexpr int kOzATile = kOzBM * kOzBK * 2;   // 16 KB
 constexpr int kOzBTile = kOzBN * kOzBK * 2;   // 8 KB
 constexpr int kOzBBuf = kOzDigits * kOzBTile; // the 8 digit planes of one K step: 64 KB
@@ -368,15 +368,15 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)sm_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* sB = sm;                       // [2][8 planes][64 rows][128 B]
-  unsigned char* sA = sm + 2 * kOzBBuf;         // [3][128 rows][128 B]
+  unsigned char* sA = sm + 2 * kOzBBuf;         // [kOzAStages][128 rows][128 B]
   uint64_t* bar = (uint64_t*)(sA + kOzAStages * kOzATile);
   uint64_t* b_full = bar;          // 2
   uint64_t* b_empty = bar + 2;     // 2
-  uint64_t* a_full = bar + 4;      // 3
-  uint64_t* a_empty = bar + 7;     // 3
-  uint64_t* acc_full = bar + 10;
-  uint64_t* acc_empty = bar + 11;
-  uint64_t* mma_done = bar + 12;
+  uint64_t* a_full = bar + 4;      // kOzAStages
+  uint64_t* a_empty = a_full + kOzAStages;
+  uint64_t* acc_full = a_empty + kOzAStages;
+  uint64_t* acc_empty = acc_full + 1;
+  uint64_t* mma_done = acc_full + 2;
   __shared__ unsigned s_tmem;
   __shared__ volatile int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -446,7 +446,6 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   } else if (warp == 5) {
     // ---- MMA issuer: accumulator g (TMEM columns 64 g) sums the digit pairs p + q = g
     if (lane == 0) {
-      const unsigned idesc = tc::idesc_bf16_f32(kOzBM, kOzBN);
       long long na = 0;
       for (int c = 0; c < nchunk && !s_abort; ++c) {
         if (c > 0 && !tc::mbar_wait(acc_empty, (c - 1) & 1, kOzSpin)) { s_abort = 1; break; }
@@ -462,7 +461,14 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             if (!tc::mbar_wait(&a_full[s], (unsigned)((na / kOzAStages) & 1), kOzSpin)) { s_abort = 1; break; }
             tc::tc_fence_after();
             const uint64_t da = tc::sdesc_kmajor_sw128(sA + s * kOzATile);
-            for (int q = 0; q + p < kOzDigits; ++q) {
+            // the B planes q, q + 1, ... lie behind one another in shared
+            // memory and their accumulators p + q, ... in TMEM, so one
+            // instruction takes up to four of them (N = 256): the A plane is
+            // read once per four products.  At N = 64 the operands' shared-
+            // memory reads (192 bytes a cycle) bound the tensor cores to half
+            for (int q = 0; q + p < kOzDigits; q += 4) {
+              const int np = min(4, kOzDigits - p - q);
+              const unsigned idesc = tc::idesc_bf16_f32(kOzBM, kOzBN * np);
               const uint64_t db = tc::sdesc_kmajor_sw128(sB + b * kOzBBuf + q * kOzBTile);
               const unsigned dt = tmem + (unsigned)((p + q) * kOzBN);
 #pragma unroll
