@@ -9,8 +9,9 @@
 // Every product runs on the tensor cores in FP64-accurate digit-split form
 // (ozaki.cu): the side operators are split once at creation; each apply
 // splits the blocks of x (as rows for Psi H_R^T, as columns for H_L Psi and
-// L Psi) and the intermediate L Psi, and every stage is one launch over all
-// blocks.
+// L Psi) and the intermediates L Psi, and every stage is one launch over all
+// blocks: the slices of x, the products L Psi, their slices, and every block
+// of y as one chain of products.
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -69,6 +70,7 @@ OzProblem oz_problem(const OzOperand& A, const OzOperand& B, double* C, long lon
   p.tiles_n = (B.R + kOzBN - 1) / kOzBN;
   p.tri = 0;
   p.tile0 = 0;
+  p.more = 0;
   return p;
 }
 
@@ -152,7 +154,6 @@ extern "C" ed_status ed_dense_create(int nq, const int64_t* chi, const double* c
     t.R.assign(nq, OzOperand{});
     t.T.assign(nq, OzOperand{});
     t.toff.assign(nq, -1);
-    int64_t s = 0;
     for (int q = 0; q < nq; ++q) {
       const double* l = Lm[(size_t)m * nq + q];
       if (!l) continue;
@@ -160,10 +161,9 @@ extern "C" ed_status ed_dense_create(int nq, const int64_t* chi, const double* c
       ED_TRY(oz_operand_host(&d->oz, l, ct, c, true, &t.L[q]));
       ED_TRY(oz_operand_host(&d->oz, Rm[(size_t)m * nq + q], ct, c, false, &t.R[q]));
       ED_TRY(oz_operand_device(&d->oz, ct, c, true, &t.T[q]));
-      t.toff[q] = s;
-      s += (int64_t)ct * c;
+      t.toff[q] = scratch;
+      scratch += (int64_t)ct * c;
     }
-    scratch = std::max(scratch, s);
     d->terms.push_back(std::move(t));
   }
   if (scratch > 0) ED_TRY(dense_alloc(d, (void**)&d->scratch, (size_t)scratch * sizeof(double)));
@@ -185,13 +185,25 @@ extern "C" ed_status ed_dense_create(int nq, const int64_t* chi, const double* c
     if (v.empty()) return ED_OK;
     return put(by_cols ? 1 : 0, v.data(), v.size() * sizeof(OzSliceJob), (int)v.size(), u);
   };
-  auto products = [&](std::vector<OzProblem>& v) -> ed_status {
+  // one launch over the tiles of the given chains (each: products of one C)
+  auto products = [&](std::vector<std::vector<OzProblem>>& chains) -> ed_status {
     // longest tiles first, so that the launch does not end with them
-    std::stable_sort(v.begin(), v.end(), [](const OzProblem& a, const OzProblem& b) { return a.K > b.K; });
+    auto cost = [](const std::vector<OzProblem>& ch) {
+      long long k = 0;
+      for (const auto& p : ch) k += p.K;
+      return k;
+    };
+    std::stable_sort(chains.begin(), chains.end(),
+                     [&](const std::vector<OzProblem>& a, const std::vector<OzProblem>& b) { return cost(a) > cost(b); });
+    std::vector<OzProblem> v;
     long long tiles = 0;
-    for (auto& p : v) {
-      p.tile0 = tiles;
-      tiles += oz_tiles(p.M, p.N);
+    for (auto& ch : chains) {
+      for (auto& p : ch) {
+        p.tile0 = tiles;
+        p.more = (int)ch.size() - 1;
+        v.push_back(p);
+      }
+      tiles += oz_tiles(ch[0].M, ch[0].N);
     }
     if (tiles > 0x7fffffffLL) {
       set_error("dense-block stage of %lld tiles exceeds one launch", tiles);
@@ -210,31 +222,27 @@ extern "C" ed_status ed_dense_create(int nq, const int64_t* chi, const double* c
     ED_TRY(slices(ja, false));
     ED_TRY(slices(jb, true));
   }
-  {
-    std::vector<OzProblem> s1, s2;
-    for (int q = 0; q < nq; ++q) {
-      const long long c = chi[q];
-      s1.push_back(oz_problem(d->HL[q], d->XB[q], nullptr, d->off[q], 1, c, 0));  // Y = H_L Psi
-      s2.push_back(oz_problem(d->XA[q], d->HR[q], nullptr, d->off[q], 1, c, 1));  // Y += Psi H_R^T
-    }
-    ED_TRY(products(s1));
-    ED_TRY(products(s2));
+  // T = L Psi of every cross term in one launch, their digit planes in
+  // another, then every block of Y as one chain of products
+  std::vector<std::vector<OzProblem>> tc, yc(nq);
+  std::vector<OzSliceJob> jt;
+  for (int q = 0; q < nq; ++q) {
+    const long long c = chi[q];
+    yc[q].push_back(oz_problem(d->HL[q], d->XB[q], nullptr, d->off[q], 1, c, 0));  // H_L Psi
+    yc[q].push_back(oz_problem(d->XA[q], d->HR[q], nullptr, d->off[q], 1, c, 0));  // Psi H_R^T
   }
-  for (const auto& t : d->terms) {
-    std::vector<OzProblem> s3, s4;
-    std::vector<OzSliceJob> jt;
+  for (const auto& t : d->terms)
     for (int q = 0; q < nq; ++q) {
       if (!t.L[q].slices) continue;
       const long long c = chi[q], ct = chi[q + t.delta];
       double* T = d->scratch + t.toff[q];
-      s3.push_back(oz_problem(t.L[q], d->XB[q], T, 0, 0, c, 0));                   // T = L Psi
+      tc.push_back({oz_problem(t.L[q], d->XB[q], T, 0, 0, c, 0)});
       jt.push_back(slice_job(T, 0, 0, c, (int)ct, (int)c, t.T[q]));
-      s4.push_back(oz_problem(t.T[q], t.R[q], nullptr, d->off[q + t.delta], 1, ct, 1));  // Y' += T R^T
+      yc[q + t.delta].push_back(oz_problem(t.T[q], t.R[q], nullptr, d->off[q + t.delta], 1, ct, 0));  // T R^T
     }
-    ED_TRY(products(s3));
-    ED_TRY(slices(jt, false));
-    ED_TRY(products(s4));
-  }
+  ED_TRY(products(tc));
+  ED_TRY(slices(jt, false));
+  ED_TRY(products(yc));
   g.d = nullptr;
   *out = d;
   return ED_OK;
@@ -252,7 +260,7 @@ extern "C" ed_status ed_dense_apply(ed_dense* d, const double* x, double* y, voi
     if (s.kind == 2)
       ED_TRY(oz_gemm(&d->oz, (const OzProblem*)s.list, s.count, s.units, y, st));
     else
-      ED_TRY(oz_slice(&d->oz, (const OzSliceJob*)s.list, s.count, s.units, s.kind == 1, x, st));
+      ED_TRY(oz_slice(&d->oz, (const OzSliceJob*)s.list, s.count, s.units, s.kind == 1, *std::max_element(d->chi.begin(), d->chi.end()), x, st));
   }
   return ED_OK;
 }

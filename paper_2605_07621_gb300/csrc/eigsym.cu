@@ -818,7 +818,7 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_host,
     }
     ED_CUDA_TRY(launch_pdl(k_pbal, P.jb, 256, st, m, P.k0, tb.WVf, shp, tb.WV, tb.NVW));
     // trailing matrix (rows and columns >= t0): A -= V W^T + W V^T
-    ED_TRY(oz_slice(tb.oz, tb.d_jobs + 2 * q, 2, 2LL * (m - P.t0), false, nullptr, st));
+    ED_TRY(oz_slice(tb.oz, tb.d_jobs + 2 * q, 2, 2LL * (m - P.t0), false, 0, nullptr, st));
     ED_TRY(oz_gemm(tb.oz, tb.d_probs + q, 1, oz_tiles(m - P.t0, m - P.t0, 1), nullptr, st));
   }
   k_tail<<<1, 32, 0, st>>>(A, m, d, e);

@@ -327,7 +327,7 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       double* he = hd + std::max(m, 1);
       ed_status s = ED_OK;
       if (cudaEventRecord(ev_g0.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
-      if ((s = oz_slice(&oz, d_jobs + bi, 1, units[bi], b.dA > b.dB, nullptr, ln.s)) != ED_OK) return fail(s);
+      if ((s = oz_slice(&oz, d_jobs + bi, 1, units[bi], b.dA > b.dB, b.dA, nullptr, ln.s)) != ED_OK) return fail(s);
       if ((s = oz_gemm(&oz, d_probs + bi, 1, tiles[bi], nullptr, ln.s)) != ED_OK) return fail(s);
       if (cudaEventRecord(ev_g1.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
       TriBlocked tb{&oz, ln.NVW, ln.WV, ln.WVf, ln.F, tridiag_ldF(m), {}, oz.d_err, d_tjobs + 2 * toff[bi],

@@ -257,8 +257,16 @@ __device__ inline int find_job(const OzSliceJob* jobs, int n, long long u) {
   return lo;
 }
 
+// the digit planes of two neighbouring K entries, one 4-byte store per plane
+__device__ __forceinline__ void store_digits(uint16_t* row, long long plane, int k, const int* d0, const int* d1) {
+#pragma unroll
+  for (int p = 0; p < kOzDigits; ++p)
+    *reinterpret_cast<uint32_t*>(row + p * plane + k) =
+        bf16_of_small_int(d0[p]) | (uint32_t)bf16_of_small_int(d1[p]) << 16;
+}
+
 // operand rows = source rows: one warp per row (exponent by a warp max, then
-// the digits of every element, one BF16 plane store per digit)
+// the digits of every element)
 __global__ void __launch_bounds__(256) k_oz_slice_rows(const OzSliceJob* __restrict__ jobs, int njobs, long long units,
                                                        const double* __restrict__ x) {
   const long long u = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -275,76 +283,105 @@ __global__ void __launch_bounds__(256) k_oz_slice_rows(const OzSliceJob* __restr
   if (lane == 0) J.exps[i] = E;
   const long long plane = (long long)J.rows * J.Kpad;
   uint16_t* row = J.dst + (long long)i * J.Kpad;
-  for (int k = lane; k < J.Kpad; k += 32) {
-    int d[kOzDigits];
-    digits_dev(k < J.cols ? src[k] : 0.0, E, d);
-#pragma unroll
-    for (int p = 0; p < kOzDigits; ++p) row[p * plane + k] = bf16_of_small_int(d[p]);
+  for (int k = 2 * lane; k < J.Kpad; k += 64) {
+    int d0[kOzDigits], d1[kOzDigits];
+    digits_dev(k < J.cols ? src[k] : 0.0, E, d0);
+    digits_dev(k + 1 < J.cols ? src[k + 1] : 0.0, E, d1);
+    store_digits(row, plane, k, d0, d1);
   }
 }
 
-// operand rows = source columns (the transpose): one CTA per strip of 32
-// source columns -- per-column exponent over all rows, then 32 x 32 tiles
-// transposed through shared memory so both reads and digit stores coalesce
-__global__ void __launch_bounds__(256) k_oz_slice_cols(const OzSliceJob* __restrict__ jobs, int njobs,
-                                                       long long units, const double* __restrict__ x) {
-  __shared__ double tile[32][33];
+// operand rows = source columns (the transpose), in strips of 32 source
+// columns times runs of kOzColRows rows, so that a few wide blocks fill the
+// GPU (one CTA per strip took 245 us for the 21 blocks of the dense-block
+// state, 142 strips).  The exponents come first: cleared (k_oz_col_clear),
+// then the largest of the runs (k_oz_col_exp); an all-zero column keeps
+// kOzNoExp, which counts as 0.
+constexpr int kOzColRows = 256;
+constexpr int kOzNoExp = -(1 << 30);
+
+__global__ void __launch_bounds__(32) k_oz_col_clear(const OzSliceJob* __restrict__ jobs, int njobs) {
+  const OzSliceJob J = jobs[find_job(jobs, njobs, blockIdx.x)];
+  const int c = (int)(blockIdx.x - J.first) * 32 + threadIdx.x;
+  if (c < J.cols) J.exps[c] = kOzNoExp;
+}
+
+__global__ void __launch_bounds__(256) k_oz_col_exp(const OzSliceJob* __restrict__ jobs, int njobs,
+                                                    const double* __restrict__ x) {
   __shared__ double cmax[8][32];
-  __shared__ int cexp[32];
-  const long long u = blockIdx.x;
-  if (u >= units) return;
-  const OzSliceJob J = jobs[find_job(jobs, njobs, u)];
-  const int c0 = (int)(u - J.first) * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const OzSliceJob J = jobs[find_job(jobs, njobs, blockIdx.x)];
+  const int c = (int)(blockIdx.x - J.first) * 32 + (threadIdx.x & 31), ty = threadIdx.x >> 5;
+  const int r0 = blockIdx.y * kOzColRows, r1 = min(J.rows, r0 + kOzColRows);
+  if (r0 >= J.rows) return;
   const double* src = J.sbase == 1 ? x + J.soff : J.src;
   double mx = 0.0;
-  if (c0 + tx < J.cols)
-    for (int r = ty; r < J.rows; r += 8) mx = fmax(mx, fabs(src[(long long)r * J.ld + c0 + tx]));
-  cmax[ty][tx] = mx;
+  if (c < J.cols)
+#pragma unroll 8
+    for (int r = r0 + ty; r < r1; r += 8) mx = fmax(mx, fabs(src[(long long)r * J.ld + c]));
+  cmax[ty][threadIdx.x & 31] = mx;
   __syncthreads();
-  if (ty == 0) {
-    double m = 0.0;
-    for (int q = 0; q < 8; ++q) m = fmax(m, cmax[q][tx]);
-    const int E = exp_of(m);
-    cexp[tx] = E;
-    if (c0 + tx < J.cols) J.exps[c0 + tx] = E;
+  if (ty == 0 && c < J.cols) {
+    for (int q = 1; q < 8; ++q) mx = fmax(mx, cmax[q][threadIdx.x]);
+    if (mx > 0.0) atomicMax(&J.exps[c], exp_of(mx));
   }
-  __syncthreads();
+}
+
+// 32 x 64 tiles transposed through shared memory so both reads and digit
+// stores coalesce
+__global__ void __launch_bounds__(256) k_oz_slice_cols(const OzSliceJob* __restrict__ jobs, int njobs,
+                                                       const double* __restrict__ x) {
+  __shared__ double tile[64][33];
+  const OzSliceJob J = jobs[find_job(jobs, njobs, blockIdx.x)];
+  const int c0 = (int)(blockIdx.x - J.first) * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const double* src = J.sbase == 1 ? x + J.soff : J.src;
   const long long plane = (long long)J.cols * J.Kpad;  // operand rows = source columns
-  for (int r0 = 0; r0 < J.Kpad; r0 += 32) {
-    for (int q = ty; q < 32; q += 8) {
-      const int r = r0 + q, c = c0 + tx;
-      tile[q][tx] = (r < J.rows && c < J.cols) ? src[(long long)r * J.ld + c] : 0.0;
+  const int r1 = min(J.Kpad, (int)(blockIdx.y + 1) * kOzColRows);
+  for (int r0 = blockIdx.y * kOzColRows; r0 < r1; r0 += 64) {
+#pragma unroll
+    for (int q = 0; q < 64; q += 8) {
+      const int r = r0 + ty + q, c = c0 + tx;
+      tile[ty + q][tx] = (r < J.rows && c < J.cols) ? src[(long long)r * J.ld + c] : 0.0;
     }
     __syncthreads();
-    for (int q = ty; q < 32; q += 8) {
-      const int c = c0 + q, k = r0 + tx;  // operand row c, column k
-      if (c < J.cols && k < J.Kpad) {
-        int d[kOzDigits];
-        digits_dev(tile[tx][q], cexp[q], d);
-        uint16_t* row = J.dst + (long long)c * J.Kpad;
 #pragma unroll
-        for (int p = 0; p < kOzDigits; ++p) row[p * plane + k] = bf16_of_small_int(d[p]);
+    for (int q = 0; q < 32; q += 8) {
+      const int c = c0 + ty + q, k = r0 + 2 * tx;  // operand row c, columns k, k + 1
+      if (c < J.cols && k < J.Kpad) {
+        int E = J.exps[c];
+        if (E == kOzNoExp) E = 0;
+        int d0[kOzDigits], d1[kOzDigits];
+        digits_dev(tile[2 * tx][ty + q], E, d0);
+        digits_dev(tile[2 * tx + 1][ty + q], E, d1);
+        store_digits(J.dst + (long long)c * J.Kpad, plane, k, d0, d1);
       }
     }
     __syncthreads();
   }
+  // every other CTA reads kOzNoExp or this zero alike
+  if (blockIdx.y == 0 && threadIdx.x < 32 && c0 + tx < J.cols && J.exps[c0 + tx] == kOzNoExp) J.exps[c0 + tx] = 0;
 }
 
 ed_status oz_slice(OzContext* o, const OzSliceJob* d_jobs, int njobs, long long units, bool transpose,
-                   const double* x, cudaStream_t st) {
+                   long long max_rows, const double* x, cudaStream_t st) {
   if (units <= 0) return ED_OK;
-  if (transpose)
-    k_oz_slice_cols<<<(unsigned)units, 256, 0, st>>>(d_jobs, njobs, units, x);
-  else
+  if (transpose) {
+    // (the last run also writes the padding columns up to Kpad)
+    const dim3 g((unsigned)units, (unsigned)((max_rows + 7) / 8 * 8 + kOzColRows - 1) / kOzColRows);
+    k_oz_col_clear<<<(unsigned)units, 32, 0, st>>>(d_jobs, njobs);
+    k_oz_col_exp<<<g, 256, 0, st>>>(d_jobs, njobs, x);
+    k_oz_slice_cols<<<g, 256, 0, st>>>(d_jobs, njobs, x);
+  } else {
     k_oz_slice_rows<<<(unsigned)((units + 7) / 8), 256, 0, st>>>(d_jobs, njobs, units, x);
+  }
   ED_CUDA_TRY(cudaGetLastError());
   return ED_OK;
 }
 
 // ---------------------------------------------------------------- the GEMM
 
-constexpr int kOzThreads = 192;          // warps 0-3 epilogue, 4 TMA producer, 5 MMA issuer
+constexpr int kOzEpi = 8;                  // epilogue warps: two per 32 TMEM lanes, 32 columns each
+constexpr int kOzThreads = 32 * (kOzEpi + 2);  // then the TMA producer and the MMA issuer
 constexpr int kOzAStages = 6;
 constexpr int kOzATile = kOzBM * kOzBK * 2;   // 16 KB
 constexpr int kOzBTile = kOzBN * kOzBK * 2;   // 8 KB
@@ -362,6 +399,14 @@ __device__ inline int find_prob(const OzProblem* probs, int n, long long tile) {
   return lo;
 }
 
+// One output tile per CTA.  Bound: the tensor pipe waits for its operands and
+// for the drain of the accumulators (active 50 % of the time on the 572 tiles
+// of the dense-block Y stage, 54 % on its 1,644 T tiles; one K step moves 192 KB
+// from L2 for 38 MFLOP).  Dense-block H|psi> (alpha = 0.95, 4,003 states of bond
+// dimension): 5.28 ms with N = 64 instructions and three A stages, 3.72 with N
+// = 256 and six, 2.67 with chains (one launch for all blocks of Y, C written
+// once), eight epilogue warps and column slicing split over rows; the digit
+// products alone would take 1.43 ms at the burst BF16 rate.
 __global__ void __launch_bounds__(kOzThreads, 1)
     k_oz_gemm(const OzProblem* __restrict__ probs, int nprob, const CUtensorMap* __restrict__ maps, double* y,
               int* err) {
@@ -381,7 +426,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   __shared__ volatile int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  const OzProblem P = probs[find_prob(probs, nprob, (long long)blockIdx.x)];
+  const int last = find_prob(probs, nprob, (long long)blockIdx.x);
+  const int nparts = probs[last].more + 1;
+  const OzProblem* const parts = probs + (last - nparts + 1);  // the tile's products
+  const OzProblem P = parts[0];
   long long t = (long long)blockIdx.x - P.tile0;
   int m0, n0;
   if (!P.tri) {
@@ -396,9 +444,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     m0 = tm * kOzBM;
     n0 = (int)t * kOzBN;
   }
-  const int nkb = (P.K + kOzBK - 1) / kOzBK;
   const int kb_per_chunk = kOzKChunk / kOzBK;
-  const int nchunk = (nkb + kb_per_chunk - 1) / kb_per_chunk;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -410,7 +456,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       tc::mbar_init(&a_empty[i], 1);
     }
     tc::mbar_init(acc_full, 1);
-    tc::mbar_init(acc_empty, 128);
+    tc::mbar_init(acc_empty, 32 * kOzEpi);
     tc::mbar_init(mma_done, 1);
     tc::fence_mbar_init();
     s_abort = 0;
@@ -421,65 +467,74 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   tc::tc_fence_after();
   const unsigned tmem = s_tmem;
 
-  if (warp == 4) {
+  if (warp == kOzEpi) {
     // ---- TMA producer: per K step the 8 digit planes of B^T, then A's planes one by one
     if (lane == 0) {
-      const CUtensorMap* ma = maps + P.mapA;
-      const CUtensorMap* mb = maps + P.mapB;
-      long long na = 0;
-      for (int kb = 0; kb < nkb && !s_abort; ++kb) {
-        const int b = kb & 1, ub = kb >> 1;
-        if (ub > 0 && !tc::mbar_wait(&b_empty[b], (ub - 1) & 1, kOzSpin)) { s_abort = 1; break; }
-        tc::mbar_expect_tx(&b_full[b], kOzBBuf);
-        for (int q = 0; q < kOzDigits; ++q)
-          tc::tma_load_3d(sB + b * kOzBBuf + q * kOzBTile, mb, kb * kOzBK, n0, q, &b_full[b]);
-        for (int p = 0; p < kOzDigits; ++p, ++na) {
-          const int s = (int)(na % kOzAStages);
-          const long long ua = na / kOzAStages;
-          if (ua > 0 && !tc::mbar_wait(&a_empty[s], (unsigned)((ua - 1) & 1), kOzSpin)) { s_abort = 1; break; }
-          tc::mbar_expect_tx(&a_full[s], kOzATile);
-          tc::tma_load_3d(sA + s * kOzATile, ma, kb * kOzBK, m0, p, &a_full[s]);
+      long long na = 0, kg = 0;  // A planes, K steps over all parts
+      for (int pt = 0; pt < nparts; ++pt) {
+        const CUtensorMap* ma = maps + parts[pt].mapA;
+        const CUtensorMap* mb = maps + parts[pt].mapB;
+        const int nkb = (parts[pt].K + kOzBK - 1) / kOzBK;
+        for (int kb = 0; kb < nkb && !s_abort; ++kb, ++kg) {
+          const int b = (int)(kg & 1);
+          const long long ub = kg >> 1;
+          if (ub > 0 && !tc::mbar_wait(&b_empty[b], (unsigned)((ub - 1) & 1), kOzSpin)) { s_abort = 1; break; }
+          tc::mbar_expect_tx(&b_full[b], kOzBBuf);
+          for (int q = 0; q < kOzDigits; ++q)
+            tc::tma_load_3d(sB + b * kOzBBuf + q * kOzBTile, mb, kb * kOzBK, n0, q, &b_full[b]);
+          for (int p = 0; p < kOzDigits; ++p, ++na) {
+            const int s = (int)(na % kOzAStages);
+            const long long ua = na / kOzAStages;
+            if (ua > 0 && !tc::mbar_wait(&a_empty[s], (unsigned)((ua - 1) & 1), kOzSpin)) { s_abort = 1; break; }
+            tc::mbar_expect_tx(&a_full[s], kOzATile);
+            tc::tma_load_3d(sA + s * kOzATile, ma, kb * kOzBK, m0, p, &a_full[s]);
+          }
         }
       }
       if (s_abort) atomicExch(err, 1);
     }
-  } else if (warp == 5) {
+  } else if (warp == kOzEpi + 1) {
     // ---- MMA issuer: accumulator g (TMEM columns 64 g) sums the digit pairs p + q = g
     if (lane == 0) {
-      long long na = 0;
-      for (int c = 0; c < nchunk && !s_abort; ++c) {
-        if (c > 0 && !tc::mbar_wait(acc_empty, (c - 1) & 1, kOzSpin)) { s_abort = 1; break; }
-        tc::tc_fence_after();
-        const int kb_end = min(nkb, (c + 1) * kb_per_chunk);
-        for (int kb = c * kb_per_chunk; kb < kb_end && !s_abort; ++kb) {
-          const int b = kb & 1, ub = kb >> 1;
-          if (!tc::mbar_wait(&b_full[b], ub & 1, kOzSpin)) { s_abort = 1; break; }
+      long long na = 0, kg = 0;
+      int cg = 0;  // chunks over all parts
+      for (int pt = 0; pt < nparts; ++pt) {
+        const int nkb = (parts[pt].K + kOzBK - 1) / kOzBK;
+        const int nchunk = (nkb + kb_per_chunk - 1) / kb_per_chunk;
+        for (int c = 0; c < nchunk && !s_abort; ++c, ++cg) {
+          if (cg > 0 && !tc::mbar_wait(acc_empty, (unsigned)((cg - 1) & 1), kOzSpin)) { s_abort = 1; break; }
           tc::tc_fence_after();
-          const bool first_kb = kb == c * kb_per_chunk;
-          for (int p = 0; p < kOzDigits; ++p, ++na) {
-            const int s = (int)(na % kOzAStages);
-            if (!tc::mbar_wait(&a_full[s], (unsigned)((na / kOzAStages) & 1), kOzSpin)) { s_abort = 1; break; }
+          const int kb_end = min(nkb, (c + 1) * kb_per_chunk);
+          for (int kb = c * kb_per_chunk; kb < kb_end && !s_abort; ++kb, ++kg) {
+            const int b = (int)(kg & 1);
+            if (!tc::mbar_wait(&b_full[b], (unsigned)((kg >> 1) & 1), kOzSpin)) { s_abort = 1; break; }
             tc::tc_fence_after();
-            const uint64_t da = tc::sdesc_kmajor_sw128(sA + s * kOzATile);
-            // the B planes q, q + 1, ... lie behind one another in shared
-            // memory and their accumulators p + q, ... in TMEM, so one
-            // instruction takes up to four of them (N = 256): the A plane is
-            // read once per four products.  At N = 64 the operands' shared-
-            // memory reads (192 bytes a cycle) bound the tensor cores to half
-            for (int q = 0; q + p < kOzDigits; q += 4) {
-              const int np = min(4, kOzDigits - p - q);
-              const unsigned idesc = tc::idesc_bf16_f32(kOzBM, kOzBN * np);
-              const uint64_t db = tc::sdesc_kmajor_sw128(sB + b * kOzBBuf + q * kOzBTile);
-              const unsigned dt = tmem + (unsigned)((p + q) * kOzBN);
-#pragma unroll
-              for (int kk = 0; kk < kOzBK / 16; ++kk)  // 32 bytes of K per instruction
-                tc::mma_bf16(dt, da + 2 * kk, db + 2 * kk, idesc, !(first_kb && p == 0 && kk == 0));
+            const bool first_kb = kb == c * kb_per_chunk;
+            for (int p = 0; p < kOzDigits; ++p, ++na) {
+              const int s = (int)(na % kOzAStages);
+              if (!tc::mbar_wait(&a_full[s], (unsigned)((na / kOzAStages) & 1), kOzSpin)) { s_abort = 1; break; }
+              tc::tc_fence_after();
+              const uint64_t da = tc::sdesc_kmajor_sw128(sA + s * kOzATile);
+              // the B planes q, q + 1, ... lie behind one another in shared
+              // memory and their accumulators p + q, ... in TMEM, so one
+              // instruction takes up to four of them (N = 256): the A plane is
+              // read once per four products.  At N = 64 the operands' shared-
+              // memory reads (192 bytes a cycle) bound the tensor cores to half
+              for (int q = 0; q + p < kOzDigits; q += 4) {
+                const int np = min(4, kOzDigits - p - q);
+                const unsigned idesc = tc::idesc_bf16_f32(kOzBM, kOzBN * np);
+                const uint64_t db = tc::sdesc_kmajor_sw128(sB + b * kOzBBuf + q * kOzBTile);
+                const unsigned dt = tmem + (unsigned)((p + q) * kOzBN);
+  #pragma unroll
+                for (int kk = 0; kk < kOzBK / 16; ++kk)  // 32 bytes of K per instruction
+                  tc::mma_bf16(dt, da + 2 * kk, db + 2 * kk, idesc, !(first_kb && p == 0 && kk == 0));
+              }
+              tc::mma_commit(&a_empty[s]);
             }
-            tc::mma_commit(&a_empty[s]);
+            tc::mma_commit(&b_empty[b]);
           }
-          tc::mma_commit(&b_empty[b]);
+          tc::mma_commit(acc_full);
         }
-        tc::mma_commit(acc_full);
       }
       // every issued MMA finishes before the accumulators are released
       tc::mma_commit(mma_done);
@@ -487,19 +542,23 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       if (s_abort) atomicExch(err, 1);
     }
   } else {
-    // ---- epilogue: thread = one output row.  The 8 digit-order sums S_g of
-    // a chunk are exact integers below 2^24 held in FP32; per column they
-    // become one 128-bit integer T = sum_g S_g 2^(42 - 6g) (orders 0-3 and
-    // 4-7 summed in two 64-bit integers first) on the integer pipe, rounded
-    // once to FP64 by bit manipulation (C = T 2^(E_A + E_B - 52)).  With
-    // more than one K chunk the chunks' rounded values add in FP64.
-    const int row = warp * 32 + lane;
+    // ---- epilogue: thread = one output row, half of the tile's columns.  The
+    // 8 digit-order sums S_g of a chunk are exact integers below 2^24 held in
+    // FP32; per column they become one 128-bit integer T = sum_g S_g
+    // 2^(42 - 6g) (orders 0-3 and 4-7 summed in two 64-bit integers first) on
+    // the integer pipe, rounded once to FP64 by bit manipulation (C = T
+    // 2^(E_A + E_B - 52)).  With more than one K chunk or product the rounded
+    // values add in FP64 registers; C is read and written once per chain.
+    // Eight warps instead of four halve the time in which the tensor cores
+    // wait (the 8 accumulators fill TMEM, so a drain does not overlap).
+    constexpr int kCols = kOzBN / 2;
+    const int row = (warp & 3) * 32 + lane, ch = (warp >> 2) * kCols;
     const int i = m0 + row;
     const bool rv = i < P.M;
-    const int ea = rv ? P.ea[i] : 0;
-    double* crow = rv ? (P.cbase == 1 ? y + P.coff : P.C) + (long long)i * P.ldc : nullptr;
-    const unsigned tl = tmem + ((unsigned)(warp * 32) << 16);
-    // T of the 8 columns 8q .. 8q + 7 of the tile
+    double* crow = rv ? (P.cbase == 1 ? y + P.coff : P.C) + (long long)i * P.ldc + n0 + ch : nullptr;
+    const int nc = P.N - n0 - ch;  // columns of this half inside the matrix
+    const unsigned tl = tmem + ((unsigned)((warp & 3) * 32) << 16) + ch;
+    // T of the 8 columns 8q .. 8q + 7 of the half
     auto group = [&](int q, I128* T) {
       long long H[8], L[8];
 #pragma unroll
@@ -529,10 +588,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     // tile's rows into L2 now, while the tensor cores run
     if (P.acc && rv) {
 #pragma unroll
-      for (int q = 0; q < kOzBN * 8 / 128; ++q) {
-        const int col = n0 + q * 16;
-        if (col < P.N) asm volatile("prefetch.global.L2 [%0];" ::"l"(crow + col));
-      }
+      for (int q = 0; q < kCols * 8 / 128; ++q)
+        if (q * 16 < nc) asm volatile("prefetch.global.L2 [%0];" ::"l"(crow + q * 16));
     }
     auto wait_chunk = [&](int c) -> bool {
       bool ok = false;
@@ -543,18 +600,19 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       if (!ok) s_abort = 1;
       return ok;
     };
-    if (nchunk == 1) {
+    if (nparts == 1 && P.K <= kOzKChunk) {
+      const int ea = rv ? P.ea[i] : 0;
       if (wait_chunk(0)) {
         tc::tc_fence_after();
 #pragma unroll 1
-        for (int q = 0; q < kOzBN / 8; ++q) {
+        for (int q = 0; q < kCols / 8; ++q) {
           I128 T[8];
           group(q, T);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const int col = n0 + 8 * q + j;
-            if (rv && col < P.N) {
-              const double v = from_fixed128(T[j], ea + P.eb[col] - 52);
+            const int col = 8 * q + j;
+            if (rv && col < nc) {
+              const double v = from_fixed128(T[j], ea + P.eb[n0 + ch + col] - 52);
               crow[col] = P.acc ? crow[col] + v : v;
             }
           }
@@ -563,31 +621,34 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         tc::mbar_arrive(acc_empty);
       }
     } else {
-      double acc[kOzBN];
+      double acc[kCols];
 #pragma unroll
-      for (int j = 0; j < kOzBN; ++j) acc[j] = 0.0;
-      for (int c = 0; c < nchunk; ++c) {
-        if (!wait_chunk(c)) break;
-        tc::tc_fence_after();
+      for (int j = 0; j < kCols; ++j) acc[j] = 0.0;
+      int cg = 0;
+      for (int pt = 0; pt < nparts && !s_abort; ++pt) {
+        const int nkb = (parts[pt].K + kOzBK - 1) / kOzBK;
+        const int nchunk = (nkb + kb_per_chunk - 1) / kb_per_chunk;
+        const int ea = rv ? parts[pt].ea[i] : 0;
+        const int* eb = parts[pt].eb + n0 + ch;
+        for (int c = 0; c < nchunk; ++c, ++cg) {
+          if (!wait_chunk(cg)) break;
+          tc::tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < kOzBN / 8; ++q) {
-          I128 T[8];
-          group(q, T);
+          for (int q = 0; q < kCols / 8; ++q) {
+            I128 T[8];
+            group(q, T);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) acc[8 * q + j] += from_fixed128(T[j], -42);
+            for (int j = 0; j < 8; ++j)
+              if (8 * q + j < nc) acc[8 * q + j] += from_fixed128(T[j], ea + eb[8 * q + j] - 52);
+          }
+          tc::tc_fence_before();
+          tc::mbar_arrive(acc_empty);
         }
-        tc::tc_fence_before();
-        tc::mbar_arrive(acc_empty);
       }
       if (!s_abort && rv) {
 #pragma unroll
-        for (int j = 0; j < kOzBN; ++j) {
-          const int col = n0 + j;
-          if (col < P.N) {
-            const double v = acc[j] * pow2(ea + P.eb[col] - 10);
-            crow[col] = P.acc ? crow[col] + v : v;
-          }
-        }
+        for (int j = 0; j < kCols; ++j)
+          if (j < nc) crow[j] = P.acc ? crow[j] + acc[j] : acc[j];
       }
     }
   }

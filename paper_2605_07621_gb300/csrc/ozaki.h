@@ -37,7 +37,9 @@ struct OzOperand {
 };
 
 // One product of a launch: C (M x N, row stride ldc) = or += A B, with A the
-// M x K operand `a` and B^T the N x K operand `b` (both as digit planes).
+// M x K operand `a` and B^T the N x K operand `b` (both as digit planes).  A
+// chain C (+)= A_0 B_0 + A_1 B_1 + ... is several consecutive problems that
+// share C, M, N, tile0 and acc; each of them holds the chain's length - 1.
 struct OzProblem {
   int mapA, mapB;
   const int* ea;       // exponents of A's rows
@@ -50,6 +52,7 @@ struct OzProblem {
   int tiles_n;
   int tri;             // 1: only the tiles on or below the diagonal (C symmetric, its lower triangle)
   long long tile0;
+  int more;            // further products of the same tiles (a chain), 0: none
 };
 
 // Tensor maps and device buffers of one set of operands.
@@ -99,8 +102,10 @@ struct OzSliceJob {
   int Kpad;            // of the destination operand
   long long first;     // first work unit of this job in the launch
 };
+// units: the jobs' rows (rows) or 32-column strips (cols), whose sources have
+// at most max_rows rows
 ed_status oz_slice(OzContext* o, const OzSliceJob* d_jobs, int njobs, long long units, bool transpose,
-                   const double* x, cudaStream_t st);
+                   long long max_rows, const double* x, cudaStream_t st);
 ed_status oz_gemm(OzContext* o, const OzProblem* d_probs, int nprob, long long tiles, double* y, cudaStream_t st);
 long long oz_tiles(int M, int N, int tri = 0);
 // host-side digit planes (for tests and static operands): U and digits of v
