@@ -42,20 +42,6 @@ void host_mul_wide(long long a, long long b, long long* hi, unsigned long long* 
   *lo = v.lo;
 }
 
-__device__ __forceinline__ int biased_exp(double v) {
-  return (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffull);
-}
-
-// largest of the CTA's values, in every thread (blockDim a multiple of 32)
-__device__ __forceinline__ int block_max(int m) {
-  __shared__ int red[32];
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  const int w = threadIdx.x & 31;
-  return __reduce_max_sync(0xffffffffu, w < (int)(blockDim.x >> 5) ? red[w] : 0);
-}
-
 // largest biased exponent of each CTA's share of x into part[blockIdx.x];
 // the next kernel takes the largest of them (no atomics, nothing to clear).
 // x is 16-byte aligned.  Bound by HBM: 0.67 ms for 4.8 GB (7.2 TB/s).
@@ -79,16 +65,6 @@ __global__ void __launch_bounds__(256) k_exp_max(const double* __restrict__ x, l
   if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) m = max(m, biased_exp(x[n - 1]));
   m = block_max(m);
   if (threadIdx.x == 0) part[blockIdx.x] = m;
-}
-
-// the largest exponent from k_exp_max's partial results, in every thread; CTA
-// 0 leaves it in emax[0] for the kernels after this one
-__device__ __forceinline__ int finish_exp(const int* __restrict__ part, int npart, int* emax) {
-  int m = 0;
-  for (int i = threadIdx.x; i < npart; i += blockDim.x) m = max(m, part[i]);
-  m = block_max(m);
-  if (blockIdx.x == 0 && threadIdx.x == 0) emax[0] = m;
-  return m;
 }
 
 // |x| < 2^E with E = emax - 1022; X = round(x * 2^(P - E)).  Bound by HBM
@@ -574,8 +550,6 @@ struct ProfMarks {
     for (auto& e : ev) c->prof_ev.push_back(e);
   }
 };
-
-constexpr int kExpParts = 2048;  // partial exponents of k_exp_max, behind the first 16 ints of the scratch
 
 // x: the pass's input (CVT: the FP64 vector, whose fixed-point copy goes to
 // xw); xd: the FP64 vector of a split diagonal

@@ -341,6 +341,37 @@ inline cudaError_t launch_pdl(void (*k)(KArgs...), long long grid, int block, si
   return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// ---------------------------------------------------------------- exponents
+
+constexpr int kExpParts = 2048;  // partial exponents of k_exp_max, behind the first 16 ints of the scratch
+
+__device__ __forceinline__ int biased_exp(double v) {
+  return (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffull);
+}
+
+// largest of the CTA's values, in every thread (blockDim a multiple of 32)
+__device__ __forceinline__ int block_max(int m) {
+  __shared__ int red[32];
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  const int w = threadIdx.x & 31;
+  return __reduce_max_sync(0xffffffffu, w < (int)(blockDim.x >> 5) ? red[w] : 0);
+}
+
+// largest biased exponent of each CTA's share of x into part[blockIdx.x] (apply3.cu)
+__global__ void k_exp_max(const double* __restrict__ x, long long n, int* __restrict__ part);
+
+// the largest exponent from k_exp_max's partial results, in every thread; CTA
+// 0 leaves it in emax[0] for the kernels after this one
+__device__ __forceinline__ int finish_exp(const int* __restrict__ part, int npart, int* emax) {
+  int m = 0;
+  for (int i = threadIdx.x; i < npart; i += blockDim.x) m = max(m, part[i]);
+  m = block_max(m);
+  if (blockIdx.x == 0 && threadIdx.x == 0) emax[0] = m;
+  return m;
+}
+
 __device__ __forceinline__ int find_blk(const long long* row_start, int nblk, long long row) {
   int lo = 0, hi = nblk - 1;
   while (lo < hi) {

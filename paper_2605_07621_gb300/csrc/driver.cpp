@@ -75,6 +75,9 @@ struct Basis {
   int cap = 0, count = 0, per = 0;
   bool complete = false;
   std::vector<void*> chunks;
+  // FP32 copy of a whole FP64 basis (the updates of its orthogonalisation),
+  // cap rows of fp32_ld(n) elements; null: none
+  float* plane = nullptr;
   ~Basis() { release(); }
   bool init(BasisKind k, size_t e, long long len, int capacity, size_t budget, bool whole = false) {
     release();
@@ -106,11 +109,19 @@ struct Basis {
     }
     return true;
   }
+  void init_plane() {
+    if (complete && cudaMalloc((void**)&plane, (size_t)cap * (size_t)fp32_ld(n) * sizeof(float)) != cudaSuccess) {
+      cudaGetLastError();
+      plane = nullptr;
+    }
+  }
   void* at(int j) const { return (char*)chunks[j / per] + (size_t)(j % per) * (size_t)n * elem; }
   const void* whole() const { return chunks[0]; }
   void release() {
     for (void* p : chunks) cudaFree(p);
     chunks.clear();
+    if (plane) cudaFree(plane);
+    plane = nullptr;
     complete = false;
     count = 0;
   }
@@ -127,6 +138,14 @@ void* basis_next(Basis* B) {
   return B->at(B->count++);
 }
 
+// the FP32 copy of the latest basis vector
+template <typename T>
+void basis_plane(ed_ctx* c, Basis* B, const T* v, long long n, cudaStream_t st) {
+  if constexpr (std::is_same<T, double>::value)
+    if (B && B->complete && B->plane)
+      launch_cvt<double, float>(c, v, B->plane + (size_t)(B->count - 1) * (size_t)fp32_ld(n), n, st);
+}
+
 template <typename T>
 void basis_store(ed_ctx* c, Basis* B, const T* v, long long n, cudaStream_t st) {
   void* p = basis_next(B);
@@ -135,6 +154,7 @@ void basis_store(ed_ctx* c, Basis* B, const T* v, long long n, cudaStream_t st) 
     cudaMemcpyAsync(p, v, (size_t)n * sizeof(T), cudaMemcpyDeviceToDevice, st);
   else
     launch_cvt<float, __nv_bfloat16>(c, (const float*)v, (__nv_bfloat16*)p, n, st);
+  basis_plane<T>(c, B, v, n, st);
 }
 
 struct RunOut {
@@ -239,6 +259,21 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
   int* hcount = nullptr;  // device index of the next history entry
   ED_TRY(mem.get((void**)&hcount, sizeof(int)));
   ED_CUDA_TRY(cudaMemsetAsync(hcount, 0, sizeof(int), st));
+  // w orthogonalised against the kept vectors (classical Gram-Schmidt, twice),
+  // its norm to slot 1
+  double* ro = nullptr;
+  if constexpr (std::is_same<T, double>::value)
+    if ((reorth || pro) && basis && basis->kind == BASIS_SAME && basis->complete)
+      ED_TRY(mem.get((void**)&ro, (size_t)reorth64_doubles(std::min(basis->cap, kMaxBasis)) * sizeof(double)));
+  auto orthogonalise = [&]() -> ed_status {
+    if constexpr (std::is_same<T, double>::value) {
+      return launch_reorth64(c, (const double*)basis->whole(), basis->plane, basis->count, w, n, ro, st);
+    } else {
+      for (int pass = 0; pass < 2; ++pass)
+        launch_reorth<T>(c, (const T*)basis->whole(), n, basis->count, w, n, hcoef(c), st);
+      return dot_dev<T>(c, w, w, n, slot(c, 1), st, 1);
+    }
+  };
   // one step up to its history entry (apply, alpha, beta, orthogonalisation)
   auto head = [&](int j, bool& ortho_now) -> ed_status {
     ortho_now = false;
@@ -256,19 +291,14 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     const bool part = pro && basis->complete && basis->count <= kMaxBasis;
     launch_lz_b<T>(c, w, v, n, fuse ? ew : nullptr, full || part ? nullptr : hist, hcount, st);
     if (full) {
-      // classical Gram-Schmidt against all kept vectors, applied twice
-      for (int pass = 0; pass < 2; ++pass)
-        launch_reorth<T>(c, (const T*)basis->whole(), n, basis->count, w, n, hcoef(c), st);
-      ED_TRY(dot_dev<T>(c, w, w, n, slot(c, 1), st, 1));
+      ED_TRY(orthogonalise());
     }
     if (part) {
       double ab[2];
       ED_TRY(read_scalars(c, 0, 2, ab, st));  // alpha_j, beta_{j+1} (synchronises)
       anorm = std::max(anorm, std::fabs(ab[0]) + ab[1]);
       if (om.need(ab[0], ab[1], anorm)) {
-        for (int pass = 0; pass < 2; ++pass)
-          launch_reorth<T>(c, (const T*)basis->whole(), n, basis->count, w, n, hcoef(c), st);
-        ED_TRY(dot_dev<T>(c, w, w, n, slot(c, 1), st, 1));
+        ED_TRY(orthogonalise());
         double bn;
         ED_TRY(read_scalars(c, 1, 1, &bn, st));
         om.reset(bn);
@@ -302,7 +332,8 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     }
     vprev = v;
     v = out;
-    if (!stored && !in_place) basis_store<T>(c, basis, v, n, st);
+    if (stored) basis_plane<T>(c, basis, v, n, st);
+    else if (!in_place) basis_store<T>(c, basis, v, n, st);
   };
   // read the scalars of the steps since the last read and examine them in order
   auto examine = [&](int m) -> ed_status {
@@ -791,6 +822,7 @@ extern "C" ed_status ed_lanczos_gf(ed_ctx* c, const void* psi0, double e0, int s
                 (long long)n2);
       return ED_ENOMEM;
     }
+    if (fits) B.init_plane();
     const bool full = fits && (reorth == ED_GF_REORTH_FULL || (reorth == ED_GF_REORTH_AUTO && n2 <= kGfReorthStates));
     const bool partial = fits && !full;
     RunOut r;

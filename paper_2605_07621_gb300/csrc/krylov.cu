@@ -604,7 +604,6 @@ void launch_reorth(ed_ctx* c, const T* V, long long ldv, int m, T* w, long long 
   k_finalize_many<<<(m + 127) / 128, 128, 0, st>>>(c->d_partials, chunks, m, h);
   k_basis_update<T><<<grid_for(c, n), kRedThreads, m * sizeof(double), st>>>(V, ldv, m, h, w, n);
 }
-template void launch_reorth<double>(ed_ctx*, const double*, long long, int, double*, long long, double*, cudaStream_t);
 template void launch_reorth<float>(ed_ctx*, const float*, long long, int, float*, long long, double*, cudaStream_t);
 
 void launch_green_cf(const double* omega, int n_omega, double eta, double e0, const double* ap, const double* bp, int mp,

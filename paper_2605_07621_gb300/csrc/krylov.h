@@ -64,6 +64,13 @@ template <typename T>
 void launch_axpy_dev(ed_ctx* c, const T* x, T* y, const double* s, double sign, long long n, cudaStream_t st);
 template <typename T>
 void launch_reorth(ed_ctx* c, const T* V, long long ldv, int m, T* w, long long n, double* h, cudaStream_t st);
+// FP64, twice over (reorth.cu), and the norm of the result to slot 1 (which
+// holds the norm of w before).  F: FP32 copy of the basis, rows of fp32_ld(n)
+// elements (16-byte aligned), or null; scratch: reorth64_doubles(m) doubles
+long long fp32_ld(long long n);
+long long reorth64_doubles(int cap);
+ed_status launch_reorth64(ed_ctx* c, const double* V, const float* F, int m, double* w, long long n, double* scratch,
+                          cudaStream_t st);
 void launch_green_cf(const double* omega, int n_omega, double eta, double e0, const double* ap, const double* bp, int mp,
                      double wp, const double* ah, const double* bh, int mh, double wh, double* G, cudaStream_t st);
 void launch_fermion_remap(ed_ctx* c, const double* psi, long long dA_src, long long dB_src, double* phi,

@@ -2,7 +2,7 @@
 // splitting, see ozaki.h): digit planes formed on the host or by the slicing
 // kernels here, tiles staged by TMA with 128-byte swizzle, products issued
 // by one thread with tcgen05.mma into FP32 accumulators in TMEM (one per
-// digit order), drained by four warps and combined in FP64.
+// digit order), drained by eight warps and combined on the integer pipe.
 #include <atomic>
 
 #include "ozaki.h"
