@@ -69,7 +69,18 @@ constexpr int kRowCtas = 4096;     // most CTAs of k_psum2 (partial-sum slots)
 constexpr int kAmaxCtas = 1024;    // most CTAs of k_amax
 constexpr int kPr = 8;             // rows per warp and step of k_pcol
 constexpr int kPsT = 16;           // threads per row of k_psum2
-static_assert(kPcolCtas == 128 && kRowCtas == 4096 && kAmaxCtas == 1024 && kU == 64,
+// Most rows of k_panel_tri's trailing matrix.  It reads the full copy, 8 n^2
+// bytes per column, and wins while most of that stays in L2 (129 MB: n =
+// 4100); beyond, k_symv's triangle is half the bytes from HBM.  Device time of
+// one reduction, m = 924 / 1716 / 3432 / 5005: three kernels per column 28.4 /
+// 56.9 / 124.7 / 216.5 ms, one launch per panel 10.1 / 19.6 / 48.0 / 122.8 ms;
+// m = 6435 / 11440 with the line at 64: 331 / 1037 ms, at 6144: 250 / 957, at
+// 8192: 254 / 986.
+constexpr int kPtMax = 6144;
+constexpr int kPtSmem = 216 * 1024;  // its dynamic shared memory at most
+constexpr int kPtRows = 24;        // rows per CTA it aims at (two warps per four rows, 12 warps)
+constexpr int kPtCtas = 160;       // most CTAs of k_panel_tri (partial-sum slots)
+static_assert(kPcolCtas == 128 && kRowCtas == 4096 && kAmaxCtas == 1024 && kU == 64 && kPtCtas == 160,
               "tridiag_blocked_work_doubles counts these slots");
 
 __device__ inline unsigned long long warp_umax(unsigned long long x) {
@@ -582,6 +593,438 @@ __global__ void __launch_bounds__(256) k_psum2(const float2* __restrict__ part, 
   }
 }
 
+// ---- one launch per panel, for matrices whose float-float copy stays in L2
+// (kPtMax).  The copy F is then the full symmetric matrix, and every CTA owns
+// a run of rows: it keeps their part of the panel's W and V in shared memory,
+// forms their part of the column x, of the product p and of w, and needs from
+// the others only x itself and a few sums, so a column takes two grid
+// barriers instead of three kernels:
+//   A  K and w of the previous column; x_r = F[r][c] - V[r] (sigma W)[c]^T -
+//      (sigma W)[r] V[c]^T for the owned rows; partial sums (sigma W)^T x, V^T x
+//      and |x|^2 below the first entry -> barrier 1
+//   B  the sums' totals (slot k by one warp of the grid, awaited only after the
+//      product); p0 = F x for the owned rows; the reflector's scalars (every
+//      CTA alike); v = tau (x - alpha e), p = tau (p0 - alpha F e) - pending
+//      terms; partial sums of p.v -> barrier 2.
+// The product runs on x, before the scalars are known: F v = tau (F x - alpha F
+// e).  Data that other CTAs wrote is read past L1 (__ldcg).
+constexpr int kPtWarps = 12;                            // warps of the rows' work
+constexpr int kPtHelp = 4;                              // warps of the totals and scalars of step B
+constexpr int kPtThreads = 32 * (kPtWarps + kPtHelp);
+static_assert(kPtSmem / ((kKw + 7) * (int)sizeof(float2)) < 32 * kPtWarps, "a thread takes at most one row's entry");
+constexpr int kPtSlots = kKw + 1;                       // totals per column
+constexpr int kPtCp = kKw + 4;                          // row stride of the partial sums
+constexpr long long kPtSpin = 1LL << 21;  // polls of a barrier (a second or two) before the kernel gives up
+
+struct PanelBufs {
+  float2* xg;    // [m] the column x
+  float2* prow;  // [2][kKw] W and V of row c + 1 (two columns alternate)
+  float2* rpv;   // [2] p and v of row c + 1
+  float2* cp;    // [CTAs][kPtCp] partial sums
+  float2* tot;   // [kPtSlots] totals
+  float2* pvp;   // [CTAs] partial sums of p.v
+  unsigned* ctr;  // [0]: barrier, [1]: totals written
+};
+
+__device__ __forceinline__ bool pt_poll(unsigned* ctr, unsigned target) {
+  for (long long i = 0; i < kPtSpin; ++i) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+    if ((int)(v - target) >= 0) return true;
+  }
+  return false;
+}
+
+// 1 / a and sqrt(a) as float-float values: the FP32 approximation and two
+// steps of Newton's iteration with the residual in float-float (one FP64
+// division or square root takes thousands of cycles on one thread here)
+__device__ __forceinline__ float2 df_recip(float2 a) {
+  const float q = 1.f / a.x;
+  float2 y = make_float2(q, 0.f);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    float2 r = make_float2(1.f, 0.f);
+    df_fma(r, df_neg(a), y);
+    y = df_norm(y);
+    df_add(y, make_float2(df_norm(r).x * q, 0.f));
+    y = df_norm(y);
+  }
+  return y;
+}
+__device__ __forceinline__ float2 df_sqrt(float2 a) {
+  const float g = sqrtf(a.x), h = 0.5f / g;
+  float2 y = make_float2(g, 0.f);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    float2 r = a;
+    df_fma(r, df_neg(y), y);
+    df_add(y, make_float2(df_norm(r).x * h, 0.f));
+    y = df_norm(y);
+  }
+  return y;
+}
+
+// sum over the CTAs b = 0 .. G - 1 of base[b * stride] (G <= kPtCtas), by one warp
+__device__ __forceinline__ float2 pt_sum(const float2* base, int stride, int G, int lane) {
+  float2 v[(kPtCtas + 31) / 32];
+#pragma unroll
+  for (int u = 0; u < (kPtCtas + 31) / 32; ++u) {
+    const int b = lane + 32 * u;
+    v[u] = b < G ? __ldcg(base + (long long)b * stride) : make_float2(0.f, 0.f);
+  }
+#pragma unroll
+  for (int u = 1; u < (kPtCtas + 31) / 32; ++u) df_add(v[0], v[u]);
+  return df_warp_sum(v[0]);
+}
+
+__global__ void __launch_bounds__(kPtThreads, 1)
+    k_panel_tri(const float2* __restrict__ F, long long ldF, int m, int k0, int jb, int chunk,
+                const int* __restrict__ shp, float2* __restrict__ WVf, double* d, double* e, PanelBufs B, int* err) {
+  extern __shared__ __align__(16) unsigned char pt_smem[];
+  float2* const sWV = reinterpret_cast<float2*>(pt_smem);  // [chunk][kKw]: sigma W, V of the owned rows
+  float2* const sxr = sWV + (long long)chunk * kKw;         // [chunk] x of the owned rows
+  float2* const sp = sxr + chunk;                           // [2][chunk] F x by column halves, then p
+  float2* const sv = sp + 2 * chunk;                        // [chunk] v
+  float2* const sf0 = sv + chunk;                           // [2][chunk] F[c][r], F[c + 1][r]
+  float2* const sdg = sf0 + 2 * chunk;                      // [chunk] diagonal of the panel's own rows
+  // x from column q0 on, zeros to the end (16-byte aligned)
+  float2* const sx = sWV + (((long long)chunk * (kKw + 7) + 1) & ~1LL);
+  __shared__ float2 s_prow[kKw], s_tu[kKw], s_half[kPtWarps * 32 / kKw][kKw], s_red[kPtWarps], s_e[kNb];
+  __shared__ float2 s_alpha, s_tau, s_beta, s_K, s_v0;
+  __shared__ int s_abort;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool help = warp >= kPtWarps;
+  const int G = gridDim.x, cta = blockIdx.x;
+  const int R0 = k0 + cta * chunk, nrow = max(0, min(m, R0 + chunk) - R0);
+  const float2 z2 = make_float2(0.f, 0.f);
+  for (int i = tid; i < nrow * kKw; i += kPtThreads) sWV[i] = z2;
+  for (int i = tid; i < nrow; i += kPtThreads) {
+    sp[i] = sv[i] = sdg[i] = z2;
+    sf0[i] = F[(long long)k0 * ldF + R0 + i];
+  }
+  if (tid == 0) s_abort = 0;
+  unsigned bars = 0;
+  auto barrier = [&]() -> bool {
+    __syncthreads();
+    ++bars;
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(B.ctr, 1u);
+      if (!pt_poll(B.ctr, bars * (unsigned)G)) {
+        atomicExch(err, 4);
+        s_abort = 1;
+      }
+    }
+    __syncthreads();
+    return s_abort == 0;
+  };
+  // K and w of column j - 1 (whose p and v are in sp, sv), as column j - 1 of sWV
+  auto finish_w = [&](int j) {
+    if (warp == 0) {
+      float2 s = pt_sum(B.pvp, 1, G, lane);
+      if (lane == 0) s_K = df_mul(df_mul(s_beta, make_float2(0.5f * s_beta.x, 0.5f * s_beta.y)), df_norm(s));
+    }
+    __syncthreads();
+    const float2 b = s_beta, K = df_neg(s_K);
+    for (int i = tid; i < nrow; i += kPtThreads) {
+      float2 s = z2;
+      df_fma(s, b, sp[i]);
+      df_fma(s, K, sv[i]);
+      sWV[i * kKw + j - 1] = df_norm(s);
+      sWV[i * kKw + kNb + j - 1] = sv[i];
+    }
+  };
+  __syncthreads();
+  for (int j = 0; j < jb; ++j) {
+    const int c = k0 + j;
+    float2* const fc = sf0 + (j & 1) * chunk;        // F[c][r]
+    float2* const fn = sf0 + ((j & 1) ^ 1) * chunk;  // F[c + 1][r]
+    // ---- A
+    if (j > 0) {
+      const int hk = tid - 32 * kPtWarps;  // the helper warps fetch row c's W and V
+      float2 pc = z2, vc = z2;
+      if (hk >= 0 && (hk & (kNb - 1)) < j - 1) s_prow[hk] = __ldcg(B.prow + ((j - 1) & 1) * kKw + hk);
+      if (hk == 0) {
+        pc = __ldcg(B.rpv);
+        vc = __ldcg(B.rpv + 1);
+      }
+      finish_w(j);
+      if (hk == 0) {
+        float2 s = z2;
+        df_fma(s, s_beta, pc);
+        df_fma(s, df_neg(s_K), vc);
+        s_prow[j - 1] = df_norm(s);
+        s_prow[kNb + j - 1] = vc;
+      }
+      __syncthreads();
+    }
+    if (!help)
+      for (int l0 = warp; l0 < nrow; l0 += 2 * kPtWarps) {
+        float2 t[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int l = l0 + q * kPtWarps;
+          t[q] = z2;
+          if (l < nrow)
+            for (int i = lane; i < j; i += 32) {
+              df_fma(t[q], sWV[l * kKw + kNb + i], s_prow[i]);
+              df_fma(t[q], sWV[l * kKw + i], s_prow[kNb + i]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) t[q] = df_warp_sum(t[q]);
+        if (lane < 2) {
+          const int l = l0 + lane * kPtWarps, r = R0 + l;
+          if (l < nrow) {
+            float2 x = fc[l];
+            df_add(x, df_neg(lane ? t[1] : t[0]));
+            x = df_norm(x);
+            if (r == c) sdg[l] = x;  // the diagonal: both pending terms are in t
+            if (r <= c) x = z2;
+            sxr[l] = x;
+            if (r > c) __stcg(B.xg + r, x);
+          }
+        }
+      }
+    __syncthreads();
+    if (!help) {
+      const int k = tid & (kKw - 1), h = tid / kKw;
+      float2 s = z2;
+      if ((k & (kNb - 1)) < j)
+        for (int l = h; l < nrow; l += kPtWarps * 32 / kKw) df_fma(s, sWV[l * kKw + k], sxr[l]);
+      s_half[h][k] = s;
+    } else if (warp == kPtWarps) {
+      float2 s = z2;
+      for (int l = lane; l < nrow; l += 32)
+        if (R0 + l > c + 1) df_fma(s, sxr[l], sxr[l]);
+      s = df_warp_sum(s);
+      if (lane == 0) __stcg(B.cp + (long long)cta * kPtCp + kKw, s);
+    }
+    __syncthreads();
+    if (tid < kKw) {
+      float2 s = s_half[0][tid];
+#pragma unroll
+      for (int h = 1; h < kPtWarps * 32 / kKw; ++h) df_add(s, s_half[h][tid]);
+      __stcg(B.cp + (long long)cta * kPtCp + tid, s);
+      const int l = c + 1 - R0;
+      if (l >= 0 && l < nrow) __stcg(B.prow + (j & 1) * kKw + tid, sWV[l * kKw + tid]);
+    }
+    if (!barrier()) return;
+    // ---- B
+    const int q0 = (c + 1) & ~1;  // even, so that two entries are one aligned 16-byte load
+    if (!help) {
+      // x into shared memory, two entries per load, four loads of a thread in flight
+      const float4* xg4 = reinterpret_cast<const float4*>(B.xg + q0);
+      const int n4 = (int)(ldF - q0) / 2;
+      float2 fv = z2;  // (a CTA's rows are fewer than its threads: kPtSmem)
+      if (tid < nrow) fv = F[(long long)(c + 1) * ldF + R0 + tid];
+      for (int i0 = tid; i0 < n4; i0 += 4 * 32 * kPtWarps) {
+        float4 xv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * 32 * kPtWarps;
+          if (i < n4) xv[u] = __ldcg(xg4 + i);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * 32 * kPtWarps;
+          if (i < n4) {
+            if (q0 + 2 * i <= c) xv[u].x = xv[u].y = 0.f;
+            if (q0 + 2 * i + 1 >= m) xv[u].z = xv[u].w = 0.f;
+            reinterpret_cast<float4*>(sx)[i] = xv[u];
+          }
+        }
+      }
+      if (tid < nrow) fn[tid] = fv;
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kPtWarps) : "memory");
+      // F x of four rows per warp, over half of the columns
+      const int hf = warp & 1;
+      for (int l0 = 4 * (warp >> 1); l0 < nrow; l0 += 2 * kPtWarps) {
+        const float2* f[4];
+        float2 a[4], b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          f[q] = F + (long long)(R0 + min(l0 + q, nrow - 1)) * ldF + q0;
+          a[q] = b[q] = z2;
+        }
+#pragma unroll 2
+        for (int q = 2 * lane + 64 * hf; q < (int)(ldF - q0); q += 128) {
+          float4 u[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) u[r] = __ldg(reinterpret_cast<const float4*>(f[r] + q));
+          const float4 x = *reinterpret_cast<const float4*>(sx + q);
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            df_fma(a[r].x, a[r].y, u[r].x, u[r].y, x.x, x.y);
+            df_fma(b[r].x, b[r].y, u[r].z, u[r].w, x.z, x.w);
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          df_add(a[r], b[r]);
+          a[r] = df_warp_sum(a[r]);
+          if (lane == 0 && l0 + r < nrow) sp[hf * chunk + l0 + r] = a[r];
+        }
+      }
+    } else {
+      // the totals of the slots this CTA takes, then (all written) the
+      // reflector's scalars and the products with the pending columns
+      unsigned done = 0;
+      for (int s0 = cta + G * (warp - kPtWarps); s0 < kPtSlots; s0 += G * kPtHelp, ++done) {
+        const float2 s = pt_sum(B.cp + s0, kPtCp, G, lane);
+        if (lane == 0) __stcg(B.tot + s0, df_norm(s));
+      }
+      if (lane == 0) {
+        if (done) {
+          __threadfence();
+          atomicAdd(B.ctr + 1, done);
+        }
+        if (!pt_poll(B.ctr + 1, (unsigned)kPtSlots * (unsigned)(j + 1))) {
+          atomicExch(err, 4);
+          s_abort = 1;
+        }
+      }
+      __syncwarp();
+      const int k = tid - 32 * kPtWarps;
+      const float2 tk = __ldcg(B.tot + k), pk = __ldcg(B.prow + (j & 1) * kKw + k);
+      // every helper thread forms the same scalars
+      const float2 tail = __ldcg(B.tot + kKw), x0 = __ldcg(B.xg + c + 1);
+      float2 s = tail;
+      df_fma(s, x0, x0);
+      s = df_norm(s);
+      float2 alpha = z2, tau = z2, beta = z2, off = x0, v0 = x0;
+      if ((tail.x != 0.f || tail.y != 0.f) && s.x >= 0x1p-120f) {  // else nothing to annihilate
+        const float2 nrm = df_sqrt(s);
+        alpha = x0.x >= 0.f ? df_neg(nrm) : nrm;
+        df_add(v0, df_neg(alpha));
+        v0 = df_norm(v0);
+        tau = df_recip(v0);
+        // (nrm + |x0|) / nrm
+        beta = make_float2(1.f, 0.f);
+        df_fma(beta, x0.x >= 0.f ? x0 : df_neg(x0), df_recip(nrm));
+        beta = df_norm(beta);
+        off = alpha;
+      }
+      if ((k & (kNb - 1)) < j) {
+        float2 u = tk;
+        df_fma(u, df_neg(alpha), pk);
+        s_tu[k] = df_mul(df_norm(u), tau);
+      }
+      if (k == 0) {
+        s_alpha = alpha;
+        s_tau = tau;
+        s_beta = beta;
+        s_v0 = v0;
+        s_e[j] = off;
+      }
+    }
+    __syncthreads();
+    if (s_abort) return;
+    if (!help) {
+      const float2 tau = s_tau, na = df_neg(s_alpha);
+      float2 pv = z2;
+      for (int l0 = warp; l0 < nrow; l0 += 2 * kPtWarps) {
+        float2 t[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int l = l0 + q * kPtWarps;
+          t[q] = z2;
+          if (l < nrow)
+            for (int i = lane; i < j; i += 32) {
+              df_fma(t[q], sWV[l * kKw + kNb + i], s_tu[i]);
+              df_fma(t[q], sWV[l * kKw + i], s_tu[kNb + i]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) t[q] = df_warp_sum(t[q]);
+        if (lane < 2) {
+          const int l = l0 + lane * kPtWarps, r = R0 + l;
+          if (l < nrow) {
+            float2 p = z2, v = z2;
+            if (r > c) {
+              v = df_mul(r == c + 1 ? s_v0 : sxr[l], tau);
+              float2 s = sp[l];
+              df_add(s, sp[chunk + l]);
+              df_fma(s, na, fn[l]);
+              p = df_mul(df_norm(s), tau);
+              df_add(p, df_neg(lane ? t[1] : t[0]));
+              p = df_norm(p);
+              df_fma(pv, p, v);
+              if (r == c + 1) {
+                __stcg(B.rpv, p);
+                __stcg(B.rpv + 1, v);
+              }
+            }
+            sp[l] = p;
+            sv[l] = v;
+          }
+        }
+      }
+      pv = df_warp_sum(pv);
+      if (lane == 0) s_red[warp] = pv;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      float2 s = z2;
+#pragma unroll
+      for (int k = 0; k < kPtWarps; ++k) df_add(s, s_red[k]);
+      __stcg(B.pvp + cta, s);
+    }
+    if (!barrier()) return;
+  }
+  finish_w(jb);
+  __syncthreads();
+  for (int i = tid; i < nrow * kKw; i += kPtThreads) WVf[(long long)R0 * kKw + i] = sWV[i];
+  const int sh = *shp;
+  for (int i = tid; i < nrow && R0 + i < k0 + jb; i += kPtThreads) d[R0 + i] = ldexp(df_to_d(sdg[i]), -sh);
+  if (cta == 0 && tid < jb) e[k0 + tid] = ldexp(df_to_d(s_e[tid]), -sh);
+}
+
+// the full symmetric float-float copy F = split(A 2^sh) of the trailing matrix
+// (rows and columns >= r0) from its lower triangle, 32 x 32 tiles transposed
+// through shared memory; sh as in k_pconv
+__global__ void __launch_bounds__(256) k_pconv_full(const double* __restrict__ A, float2* __restrict__ F, long long ldF,
+                                                    int m, int r0, const unsigned long long* __restrict__ amx, int na,
+                                                    int* shp) {
+  pdl_enter();
+  __shared__ float2 tile[32][33];
+  __shared__ int s_sh;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  if (ty == 0) {
+    unsigned long long x = 0;
+    for (int b = tx; b < na; b += 32) x = amx[b] > x ? amx[b] : x;
+    x = warp_umax(x);
+    if (tx == 0) {
+      s_sh = x == 0 ? 0 : 1022 - (int)(x >> 52);
+      if (blockIdx.x == 0) *shp = s_sh;
+    }
+  }
+  __syncthreads();
+  const int sh = s_sh;
+  const int T = (m - r0 + 31) / 32;
+  for (long long t = blockIdx.x; t < (long long)T * (T + 1) / 2; t += gridDim.x) {
+    int I, J;
+    unit_ij(t, I, J);
+    const int i0 = r0 + 32 * I, j0 = r0 + 32 * J;
+#pragma unroll
+    for (int q = 0; q < 32; q += 8) {
+      const int r = i0 + ty + q, c = j0 + tx;
+      if (r < m && c <= r) {
+        const float2 f = split_scaled(A[(long long)r * m + c], sh);
+        F[(long long)r * ldF + c] = f;
+        tile[ty + q][tx] = f;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 32; q += 8) {
+      const int c = j0 + ty + q, r = i0 + tx;  // the transposed entry F[c][r], r > c
+      if (r < m && c < r) F[(long long)c * ldF + r] = tile[tx][ty + q];
+    }
+    __syncthreads();
+  }
+}
+
 // w = beta p - K v over rows c+1..m-1, stored with v as column j of the
 // panel (the panel's last column; the others are stored by the next
 // column's k_pcol)
@@ -703,37 +1146,72 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_host,
   int* shp = reinterpret_cast<int*>(Kf + 1);                // the panel's scale exponent
   unsigned* ctr = reinterpret_cast<unsigned*>(Kf + 2);      // tickets of k_pcol and k_psum2
   float2* tauf = Kf + 3;                                    // tau of the latest column
+  PanelBufs pb;                                             // of k_panel_tri
+  pb.xg = reinterpret_cast<float2*>(((uintptr_t)(tauf + 1) + 15) & ~(uintptr_t)15);  // 16-byte loads
+  pb.prow = pb.xg + m;
+  pb.rpv = pb.prow + 2 * kKw;
+  pb.tot = pb.rpv + 2;
+  pb.pvp = pb.tot + kPtSlots;
+  pb.cp = pb.pvp + kPtCtas;
+  pb.ctr = reinterpret_cast<unsigned*>(pb.cp + (long long)kPtCtas * kPtCp);
   ED_CUDA_TRY(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned), st));
   const std::vector<TriPanel> pan = tridiag_panels(m);  // none for m < 3: k_tail alone
   for (size_t q = 0; q < pan.size(); ++q) {
     const TriPanel& P = pan[q];
     ED_CUDA_TRY(cudaMemsetAsync(tb.WV + (long long)P.k0 * kKw, 0, (size_t)(m - P.k0) * kKw * sizeof(double), st));
     ED_CUDA_TRY(cudaMemsetAsync(tb.NVW + (long long)P.k0 * kKw, 0, (size_t)(m - P.k0) * kKw * sizeof(double), st));
-    // float-float copy of the panel's trailing triangle (rows and columns >= k0)
-    {
-      const int ga = (int)std::max(1LL, std::min((long long)kAmaxCtas, cdiv(m - P.k0, 8)));
-      k_amax<<<ga, 256, 0, st>>>(A, m, P.k0, amx);
-      const int gc = (int)std::max(1LL, std::min((long long)sms * 8, cdiv(m - P.k0, 8)));
-      ED_CUDA_TRY(launch_pdl(k_pconv, gc, 256, st, A, tb.F, tb.ldF, m, P.k0, amx, ga, shp));
-    }
-    for (int j = 0; j < P.jb; ++j) {
-      const int c = P.k0 + j;
-      const int n = m - c - 1;  // rows and columns of the product, from c + 1
-      const int g1 = (int)std::max(1LL, std::min((long long)kPcolCtas, cdiv(n, 8 * kPr)));
-      ED_CUDA_TRY(launch_pdl(k_pcol, g1, 256, st, tb.F, tb.ldF, m, c, j, tb.WVf, vf, pf, beta, betaf, Kf, shp, cp, ctr,
-                             d, e, tu, tauf));
-      const int u0 = (c + 1) & ~1;  // the units' origin: even, so that the boxes start 16-byte aligned
-      const long long Tn = cdiv(m - u0, kU), nu = Tn * (Tn + 1) / 2;
-      const int gs = (int)std::max(1LL, std::min((long long)sms * kSvCtas, cdiv(nu, kSvWarps)));
-      ED_CUDA_TRY(launch_pdl(k_symv, gs, 32 * kSvWarps, st, tb.tmF, m, c + 1, u0, vf, tauf, part, TU, nu, tb.err));
-      const int g4 = (int)std::max(1LL, std::min((long long)kRowCtas, cdiv(n, 256 / kPsT)));
-      ED_CUDA_TRY(launch_pdl(k_psum2, g4, 256, st, part, m, c + 1, u0, TU, (int)Tn, tb.WVf, tu, j, vf, tauf, pf, pvp,
-                             beta, c, ctr + 1, Kf));
-    }
-    {
-      const int c = P.k0 + P.jb - 1;
-      const int g5 = (int)std::max(1LL, std::min((long long)sms * 2, cdiv(m - c - 1, 256)));
-      ED_CUDA_TRY(launch_pdl(k_pw, g5, 256, st, m, c, P.jb - 1, vf, pf, Kf, betaf, tb.WVf));
+    const int ga = (int)std::max(1LL, std::min((long long)kAmaxCtas, cdiv(m - P.k0, 8)));
+    k_amax<<<ga, 256, 0, st>>>(A, m, P.k0, amx);
+    // one launch for the panel: at least kPtRows rows per CTA (a matrix of up
+    // to 64 rows in one), while a CTA's rows and the column fit shared memory
+    const int rows = m - P.k0;
+    const int g = rows <= 64 ? 1 : (int)std::min((long long)std::min(tb.ctas, kPtCtas), cdiv(rows, kPtRows));
+    const int chunk = (int)cdiv(rows, g);
+    const size_t smem = ((size_t)chunk * (kKw + 7) + (size_t)(tb.ldF - P.k0) + 4) * sizeof(float2);
+    if (rows <= kPtMax && smem <= kPtSmem) {
+      const long long T = cdiv(rows, 32);
+      const int gc = (int)std::max(1LL, std::min((long long)sms * 8, T * (T + 1) / 2));
+      ED_CUDA_TRY(launch_pdl(k_pconv_full, gc, 256, st, A, tb.F, tb.ldF, m, P.k0, amx, ga, shp));
+      ED_CUDA_TRY(cudaMemsetAsync(pb.ctr, 0, 2 * sizeof(unsigned), st));
+      // (the same value from every host thread: the attribute is the function's)
+      ED_CUDA_TRY(cudaFuncSetAttribute(k_panel_tri, cudaFuncAttributeMaxDynamicSharedMemorySize, kPtSmem));
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)cdiv(rows, chunk));
+      cfg.blockDim = dim3(kPtThreads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeCooperative;  // the CTAs wait for one another
+      at[0].val.cooperative = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      ED_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_tri, (const float2*)tb.F, tb.ldF, m, P.k0, P.jb, chunk,
+                                     (const int*)shp, tb.WVf, d, e, pb, tb.err));
+    } else {
+      // float-float copy of the panel's trailing triangle (rows and columns >= k0)
+      {
+        const int gc = (int)std::max(1LL, std::min((long long)sms * 8, cdiv(m - P.k0, 8)));
+        ED_CUDA_TRY(launch_pdl(k_pconv, gc, 256, st, A, tb.F, tb.ldF, m, P.k0, amx, ga, shp));
+      }
+      for (int j = 0; j < P.jb; ++j) {
+        const int c = P.k0 + j;
+        const int n = m - c - 1;  // rows and columns of the product, from c + 1
+        const int g1 = (int)std::max(1LL, std::min((long long)kPcolCtas, cdiv(n, 8 * kPr)));
+        ED_CUDA_TRY(launch_pdl(k_pcol, g1, 256, st, tb.F, tb.ldF, m, c, j, tb.WVf, vf, pf, beta, betaf, Kf, shp, cp, ctr,
+                               d, e, tu, tauf));
+        const int u0 = (c + 1) & ~1;  // the units' origin: even, so that the boxes start 16-byte aligned
+        const long long Tn = cdiv(m - u0, kU), nu = Tn * (Tn + 1) / 2;
+        const int gs = (int)std::max(1LL, std::min((long long)sms * kSvCtas, cdiv(nu, kSvWarps)));
+        ED_CUDA_TRY(launch_pdl(k_symv, gs, 32 * kSvWarps, st, tb.tmF, m, c + 1, u0, vf, tauf, part, TU, nu, tb.err));
+        const int g4 = (int)std::max(1LL, std::min((long long)kRowCtas, cdiv(n, 256 / kPsT)));
+        ED_CUDA_TRY(launch_pdl(k_psum2, g4, 256, st, part, m, c + 1, u0, TU, (int)Tn, tb.WVf, tu, j, vf, tauf, pf, pvp,
+                               beta, c, ctr + 1, Kf));
+      }
+      {
+        const int c = P.k0 + P.jb - 1;
+        const int g5 = (int)std::max(1LL, std::min((long long)sms * 2, cdiv(m - c - 1, 256)));
+        ED_CUDA_TRY(launch_pdl(k_pw, g5, 256, st, m, c, P.jb - 1, vf, pf, Kf, betaf, tb.WVf));
+      }
     }
     ED_CUDA_TRY(launch_pdl(k_pbal, P.jb, 256, st, m, P.k0, tb.WVf, shp, tb.WV, tb.NVW));
     // trailing matrix (rows and columns >= t0): A -= V W^T + W V^T

@@ -34,6 +34,7 @@ struct TriBlocked {
   int* err;
   const OzSliceJob* d_jobs;
   const OzProblem* d_probs;
+  int ctas;  // most CTAs of the panel kernel (they wait for one another: all must be resident)
 };
 // appends the jobs and products of an m x m reduction of A (tensor maps in oz;
 // opA / opB: digit-plane buffers for m x 2 kTriNb operands)
@@ -41,7 +42,8 @@ ed_status tridiag_blocked_setup(OzContext* oz, double* A, int m, const OzOperand
                                 const double* NVW, const double* WV, std::vector<OzSliceJob>& jobs,
                                 std::vector<OzProblem>& probs);
 inline long long tridiag_blocked_work_doubles(int m) {
-  return 6LL * m + 2LL * ((m + 63) / 64) * m + 128LL * (2 * kTriNb + 1) + 2 * kTriNb + 4096 + 1024 + 8;
+  return 7LL * m + 2LL * ((m + 63) / 64) * m + 128LL * (2 * kTriNb + 1) + 2 * kTriNb + 4096 + 1024 + 8 +
+         4LL * kTriNb + 2 + (2 * kTriNb + 1) + 160 + 160LL * (2 * kTriNb + 4) + 4;
 }
 // Reduce the symmetric m x m row-major A (device; only its lower triangle,
 // diagonal included, is read and overwritten) to tridiagonal form; the

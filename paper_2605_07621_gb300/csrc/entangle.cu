@@ -331,7 +331,7 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       if ((s = oz_gemm(&oz, d_probs + bi, 1, tiles[bi], nullptr, ln.s)) != ED_OK) return fail(s);
       if (cudaEventRecord(ev_g1.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
       TriBlocked tb{&oz, ln.NVW, ln.WV, ln.WVf, ln.F, tridiag_ldF(m), {}, oz.d_err, d_tjobs + 2 * toff[bi],
-                    d_tprobs + toff[bi]};
+                    d_tprobs + toff[bi], k == 0 && bi == lane_blocks[0][0] ? sms : std::max(1, sms / lanes)};
       if (m >= 3 && (s = tmap_8b_2d(&tb.tmF, ln.F, m, m, tb.ldF, 34, 32)) != ED_OK) return fail(s);
       if ((s = tridiag_reduce_blocked(ln.G, m, ln.work, hd, he, ln.s, sms, tb)) != ED_OK) return fail(s);
       if (cudaEventRecord(ev_done.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
