@@ -206,11 +206,10 @@ ed_status ed_lanczos_gf(ed_ctx* ctx, const void* psi0, double e0, int site, int 
  * smaller of d_A(s), d_B(s), formed on the device by this library; its
  * eigenvalues come from a blocked Householder reduction to tridiagonal form
  * on the device (float-float panel arithmetic, FP64-accurate tensor-core
- * trailing updates) and implicit QL steps on the host (one host thread per
- * block as soon as its tridiagonal matrix is ready; ED_ENOCONV if a QL
- * iteration does not converge).  The largest block is reduced first and
- * alone, the others concurrently on up to three internal streams that start
- * after the caller's prior work on `stream`.
+ * trailing updates), the blocks concurrently on up to three internal streams
+ * that start after the caller's prior work on `stream`, and from bisection by
+ * Sturm counts of all blocks' tridiagonal matrices in one batch on `stream`
+ * (each within a few eps of the matrix norm).
  *   psi      device FP64 vector of ctx (not normalised by the call)
  *   lambda   host, capacity cap: for every block in ed_blocks order, its
  *            min(d_A, d_B) eigenvalues in descending order (rounding can
@@ -222,8 +221,7 @@ ed_status ed_lanczos_gf(ed_ctx* ctx, const void* psi0, double e0, int site, int 
  *   entropy  host (nullable): -sum p ln p over p = lambda / sum(weight) > 0
  *   stage_ms host (nullable), 2 doubles: the Gram kernels' own device time
  *            (summed over blocks; they overlap other blocks' reductions),
- *            and the rest of the call's device time plus the host QL time
- *            left after the device work (milliseconds)
+ *            and the rest of the call's device time (milliseconds)
  * The Gram matrices are formed on the tensor cores in FP64-accurate
  * digit-split form (8 BF16 digit planes per value, exact FP32 sums per digit
  * order, FP64 combination).  Device memory, per stream sized for its largest
@@ -236,7 +234,7 @@ ed_status ed_lanczos_gf(ed_ctx* ctx, const void* psi0, double e0, int site, int 
 ed_status ed_entanglement_spectrum(ed_ctx* ctx, const double* psi, double* lambda, int64_t cap, int64_t* n_lambda,
                                    double* weight, double* entropy, double* stage_ms, void* stream);
 
-/* The last stage of ed_entanglement_spectrum on its own: all eigenvalues of
+/* The last stage of ed_entanglement_spectrum on the host: all eigenvalues of
  * the n x n symmetric tridiagonal matrix with diagonal d[0..n-1] and
  * off-diagonal e[0..n-2] (e[i] couples i and i+1), by the root-free implicit
  * QL iteration on the host (Pal, Walker and Kahan; Reinsch 1971), into

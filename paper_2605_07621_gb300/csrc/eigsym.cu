@@ -19,8 +19,9 @@
 //     float-float product is bound by HBM instead.  Per column three kernels:
 //     the column and its reflector (k_pcol), the product (k_symv), its sums
 //     and the pending terms (k_psum2).
-//  2. The eigenvalues of the tridiagonal matrix by implicit QL steps with
-//     shifts and deflation, on the host, one thread per matrix.
+//  2. The eigenvalues of the tridiagonal matrix (sturm.cu; the QL iteration
+//     at the end of this file serves ed_tridiag_eigenvalues, and the matrices
+//     with entries that are not finite).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -1126,7 +1127,7 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), unsigned grid, unsigned block
   return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
-ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_host, double* e_host, cudaStream_t st,
+ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, double* e_out, cudaStream_t st,
                                  int sms, const TriBlocked& tb) {
   if (m <= 0) return ED_OK;
   auto cdiv = [](long long a, long long b) { return (a + b - 1) / b; };
@@ -1220,8 +1221,8 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_host,
   }
   k_tail<<<1, 32, 0, st>>>(A, m, d, e);
   ED_CUDA_TRY(cudaGetLastError());
-  ED_CUDA_TRY(cudaMemcpyAsync(d_host, d, (size_t)m * sizeof(double), cudaMemcpyDeviceToHost, st));
-  if (m >= 2) ED_CUDA_TRY(cudaMemcpyAsync(e_host, e, (size_t)(m - 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
+  ED_CUDA_TRY(cudaMemcpyAsync(d_out, d, (size_t)m * sizeof(double), cudaMemcpyDeviceToDevice, st));
+  if (m >= 2) ED_CUDA_TRY(cudaMemcpyAsync(e_out, e, (size_t)(m - 1) * sizeof(double), cudaMemcpyDeviceToDevice, st));
   return ED_OK;
 }
 

@@ -1,5 +1,5 @@
 // Eigenvalues of dense symmetric FP64 matrices: Householder tridiagonal
-// reduction on the GPU, then implicit-shift QL on the tridiagonal matrix.
+// reduction (eigsym.cu), then the tridiagonal matrix's by counting (sturm.cu).
 #pragma once
 
 #include <vector>
@@ -47,12 +47,34 @@ inline long long tridiag_blocked_work_doubles(int m) {
 }
 // Reduce the symmetric m x m row-major A (device; only its lower triangle,
 // diagonal included, is read and overwritten) to tridiagonal form; the
-// diagonal (m) and off-diagonal (m - 1) entries are copied to the host
-// arrays (pinned), asynchronously on `st` (wait on the stream before use).
+// diagonal (m) and off-diagonal (m - 1) entries go to the device arrays d_out
+// and e_out.
 // work: device scratch of tridiag_blocked_work_doubles(m) doubles.
-ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_host, double* e_host, cudaStream_t st,
+ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, double* e_out, cudaStream_t st,
                                  int sms, const TriBlocked& tb);
-// all eigenvalues of the tridiagonal (d, e) into d (unordered); false if the
-// iteration did not converge
+// all eigenvalues of a batch of tridiagonal matrices on the device (sturm.cu):
+// block b's diagonal (n) and off-diagonal (n - 1) from de + 2 off, its
+// eigenvalues in descending order into lam + off; nrm[b] receives the
+// matrix's norm, NaN where an entry is not finite (lam is then undefined)
+struct SturmBlk {
+  int n;
+  long long off;
+  int w0, w1;  // first warp of each stage (sturm_plan)
+};
+struct SturmBatch {
+  const SturmBlk* d_blk;  // device, nb entries, n >= 1
+  size_t nb;
+  int S0, S1, warps0, warps1;  // lanes per eigenvalue and warps of each stage (sturm_plan)
+  const double* de;            // device [2 sum n]
+  double* lam;                 // device [sum n]
+  double* nrm;                 // device [nb]
+  float4* tf;                  // device scratch [sum n] each
+  double2 *td, *br;
+  int* shp;  // device scratch [nb]
+};
+void sturm_plan(std::vector<SturmBlk>& blk, int sms, SturmBatch* B);
+ed_status sturm_eigenvalues(const SturmBatch& B, cudaStream_t st);
+// all eigenvalues of the tridiagonal (d, e) on the host into d (unordered);
+// false if the iteration did not converge
 bool tridiag_eigenvalues(std::vector<double>& d, std::vector<double>& e);
 }  // namespace edk

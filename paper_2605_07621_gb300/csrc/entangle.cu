@@ -9,14 +9,11 @@
 // The Gram matrix is formed on the tensor cores by the FP64-accurate
 // digit-split GEMM (ozaki.cu; one digit-plane buffer serves as both
 // factors, only the tiles on or below the diagonal), reduced to tridiagonal
-// form on the GPU by Householder reflections (eigsym.cu), and its eigenvalues
-// come from implicit-shift QL on the host, one thread per block as soon as
-// its tridiagonal matrix is ready.  Blocks run concurrently on a few streams.
+// form on the GPU by Householder reflections (eigsym.cu), the blocks
+// concurrently on a few streams; then the eigenvalues of all blocks'
+// tridiagonal matrices by counting, in one batch (sturm.cu).
 #include <cmath>
 #include <algorithm>
-#include <chrono>
-#include <condition_variable>
-#include <mutex>
 #include <string>
 #include <thread>
 
@@ -86,13 +83,11 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
     sms = 148;
   }
 
-  // The blocks are reduced concurrently on up to kLanes streams ("lanes"):
-  // a column's kernels are short and leave most of the GPU idle on all but
-  // the largest blocks, so other blocks' columns fill it.  The largest block
-  // goes first and alone (its host QL is the longest and overlaps everything
-  // after it); the others go, largest first, to the lane with the least work
-  // so far (cost ~ m^3 / 3 for the products plus a fixed cost per column);
-  // each lane has its own buffers, sized for its largest block.
+  // The blocks are reduced concurrently on up to kLanes streams ("lanes"): a
+  // column is mostly latency and leaves most of the GPU idle.  They go, largest
+  // first, to the lane with the least work so far (cost ~ m^3 / 3 for the
+  // products plus a fixed cost per column); each lane has its own buffers,
+  // sized for its largest block, and its share of the SMs.
   constexpr int kLanes = 3;
   std::vector<size_t> order(nb);
   for (size_t i = 0; i < nb; ++i) order[i] = i;
@@ -121,11 +116,8 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
   std::vector<int> lane_of(nb, 0);
   std::vector<std::vector<size_t>> lane_blocks(lanes);
   {
-    // the largest block first, alone (lane 0; the other lanes start when it
-    // is done), so that its host QL, the longest, overlaps all the rest
     std::vector<double> load(lanes, 0.0);
-    if (nb) lane_blocks[0].push_back(order[0]);
-    for (size_t oi = 1; oi < nb; ++oi) {
+    for (size_t oi = 0; oi < nb; ++oi) {
       const size_t bi = order[oi];
       const double m = (double)bm(bi);
       const double cost = m * m * m / 3.0 + 4e7 * m;
@@ -227,16 +219,31 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
   ED_CUDA_TRY(cudaMemcpy(d_jobs, jobs.data(), nb * sizeof(OzSliceJob), cudaMemcpyHostToDevice));
   ED_CUDA_TRY(cudaMemcpy(d_probs, probs.data(), nb * sizeof(OzProblem), cudaMemcpyHostToDevice));
 
-  // pinned host arrays for every block's tridiagonal matrix
-  std::vector<size_t> hoff(nb + 1, 0);
-  for (size_t bi = 0; bi < nb; ++bi) hoff[bi + 1] = hoff[bi] + 2 * (size_t)std::max(bm(bi), 1LL);
-  struct Pinned {
-    double* p = nullptr;
-    ~Pinned() {
-      if (p) cudaFreeHost(p);
-    }
-  } hde;
-  ED_CUDA_TRY(cudaHostAlloc((void**)&hde.p, std::max<size_t>(hoff[nb], 1) * sizeof(double), cudaHostAllocDefault));
+  // the batch of tridiagonal matrices, largest first (the empty blocks have none)
+  std::vector<size_t> boff(nb + 1, 0);
+  for (size_t bi = 0; bi < nb; ++bi) boff[bi + 1] = boff[bi] + (size_t)bm(bi);
+  std::vector<SturmBlk> sblk;
+  for (size_t bi : order)
+    if (bm(bi) > 0) sblk.push_back(SturmBlk{(int)bm(bi), (long long)boff[bi], 0, 0});
+  SturmBatch sb{};
+  sturm_plan(sblk, sms, &sb);
+  double* d_de = nullptr;
+  SturmBlk* d_sblk = nullptr;
+  {
+    const size_t n1 = std::max<size_t>((size_t)need, 1), b1 = std::max<size_t>(sblk.size(), 1);
+    ED_TRY(mem.get((void**)&d_de, 2 * n1 * sizeof(double)));
+    ED_TRY(mem.get((void**)&sb.lam, (n1 + b1) * sizeof(double)));
+    ED_TRY(mem.get((void**)&sb.tf, n1 * sizeof(float4)));
+    ED_TRY(mem.get((void**)&sb.td, n1 * sizeof(double2)));
+    ED_TRY(mem.get((void**)&sb.br, n1 * sizeof(double2)));
+    ED_TRY(mem.get((void**)&sb.shp, b1 * sizeof(int)));
+    ED_TRY(mem.get((void**)&d_sblk, b1 * sizeof(SturmBlk)));
+    sb.nrm = sb.lam + need;
+    sb.de = d_de;
+    sb.d_blk = d_sblk;
+    if (!sblk.empty())
+      ED_CUDA_TRY(cudaMemcpy(d_sblk, sblk.data(), sblk.size() * sizeof(SturmBlk), cudaMemcpyHostToDevice));
+  }
   struct EventSet {
     std::vector<cudaEvent_t> e;
     ~EventSet() {
@@ -248,12 +255,11 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       for (cudaEvent_t& x : e) ED_CUDA_TRY(cudaEventCreate(&x));
       return ED_OK;
     }
-  } ev_g0, ev_g1, ev_done, ev_lane, ev_se;
+  } ev_g0, ev_g1, ev_lane, ev_se;
   ED_TRY(ev_g0.make(nb));
   ED_TRY(ev_g1.make(nb));
-  ED_TRY(ev_done.make(nb));
   ED_TRY(ev_lane.make(lanes));
-  ED_TRY(ev_se.make(3));
+  ED_TRY(ev_se.make(2));
   struct Streams {
     std::vector<cudaStream_t> s;
     ~Streams() {
@@ -273,11 +279,7 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
   for (int k = 0; k < lanes; ++k)
     ED_CUDA_TRY(cudaMemsetAsync(L[k].F, 0, (size_t)L[k].mmax * tridiag_ldF((int)L[k].mmax) * sizeof(float2), L[k].s));
 
-  // per lane one host thread enqueues its blocks; per block one host thread
-  // waits for its tridiagonal matrix and runs the QL steps
-  std::vector<std::vector<double>> dd(nb), ee(nb);
-  std::vector<char> ok(nb, 1);
-  std::vector<std::thread> qr[kLanes];
+  // per lane one host thread enqueues its blocks
   std::vector<std::thread> workers;
   struct Joiner {
     std::vector<std::thread>* t;
@@ -288,72 +290,30 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
           if (x.joinable()) x.join();
     }
   };
-  Joiner jq{qr, kLanes};
   Joiner jw{&workers, 1};
   std::vector<ed_status> lst(lanes, ED_OK);
   std::vector<std::string> lmsg(lanes);
-  // lane 0 records first_done after the largest block; the other lanes'
-  // streams wait for it (the host threads wait until it is recorded)
-  std::mutex fm;
-  std::condition_variable fcv;
-  int first_state = 0;  // 0: not yet, 1: recorded, 2: lane 0 failed before it
-  auto first_set = [&](int v) {
-    {
-      std::lock_guard<std::mutex> lk(fm);
-      first_state = v;
-    }
-    fcv.notify_all();
-  };
   auto lane_fn = [&](int k) {
     auto fail = [&](ed_status s) {
       lst[k] = s;
       lmsg[k] = ed_last_error();
-      if (k == 0) first_set(2);
     };
     DeviceGuard dg(c->device);
     if (dg.status() != ED_OK) return fail(ED_ECUDA);
     Lane& ln = L[k];
-    if (k > 0) {
-      std::unique_lock<std::mutex> lk(fm);
-      fcv.wait(lk, [&] { return first_state != 0; });
-      if (first_state == 2) return;
-      lk.unlock();
-      if (cudaStreamWaitEvent(ln.s, ev_se.e[2], 0) != cudaSuccess) return fail(ED_ECUDA);
-    }
     for (size_t bi : lane_blocks[k]) {
       const Block& b = c->blocks[bi];
       const int m = (int)bm(bi);
-      double* hd = hde.p + hoff[bi];
-      double* he = hd + std::max(m, 1);
+      double* bd = d_de + 2 * boff[bi];
       ed_status s = ED_OK;
       if (cudaEventRecord(ev_g0.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
       if ((s = oz_slice(&oz, d_jobs + bi, 1, units[bi], b.dA > b.dB, b.dA, nullptr, ln.s)) != ED_OK) return fail(s);
       if ((s = oz_gemm(&oz, d_probs + bi, 1, tiles[bi], nullptr, ln.s)) != ED_OK) return fail(s);
       if (cudaEventRecord(ev_g1.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
       TriBlocked tb{&oz, ln.NVW, ln.WV, ln.WVf, ln.F, tridiag_ldF(m), {}, oz.d_err, d_tjobs + 2 * toff[bi],
-                    d_tprobs + toff[bi], k == 0 && bi == lane_blocks[0][0] ? sms : std::max(1, sms / lanes)};
+                    d_tprobs + toff[bi], std::max(1, sms / lanes)};
       if (m >= 3 && (s = tmap_8b_2d(&tb.tmF, ln.F, m, m, tb.ldF, 34, 32)) != ED_OK) return fail(s);
-      if ((s = tridiag_reduce_blocked(ln.G, m, ln.work, hd, he, ln.s, sms, tb)) != ED_OK) return fail(s);
-      if (cudaEventRecord(ev_done.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
-      if (k == 0 && bi == lane_blocks[0][0]) {
-        if (cudaEventRecord(ev_se.e[2], ln.s) != cudaSuccess) return fail(ED_ECUDA);
-        first_set(1);
-      }
-      cudaEvent_t done = ev_done.e[bi];
-      auto ql = [&dd, &ee, &ok, hd, he, m, bi, done] {
-        if (cudaEventSynchronize(done) != cudaSuccess) {
-          ok[bi] = 2;
-          return;
-        }
-        dd[bi].assign(hd, hd + m);
-        ee[bi].assign(he, he + std::max(m - 1, 0));
-        ok[bi] = tridiag_eigenvalues(dd[bi], ee[bi]) ? 1 : 0;
-      };
-      try {
-        qr[k].emplace_back(ql);
-      } catch (...) {
-        ql();  // no thread to be had: wait for the block and reduce it here
-      }
+      if ((s = tridiag_reduce_blocked(ln.G, m, ln.work, bd, bd + m, ln.s, sms, tb)) != ED_OK) return fail(s);
     }
     if (cudaEventRecord(ev_lane.e[k], ln.s) != cudaSuccess) return fail(ED_ECUDA);
   };
@@ -372,7 +332,10 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       return lst[k];
     }
   for (int k = 0; k < lanes; ++k) ED_CUDA_TRY(cudaStreamWaitEvent(st, ev_lane.e[k], 0));
+  ED_TRY(sturm_eigenvalues(sb, st));
   ED_CUDA_TRY(cudaEventRecord(ev_se.e[1], st));
+  std::vector<double> lam((size_t)need + std::max<size_t>(sblk.size(), 1));
+  ED_CUDA_TRY(cudaMemcpyAsync(lam.data(), sb.lam, lam.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   // ||Psi_s||^2 (the trace of rho_A(s)) with the library's FP64 reduction
   std::vector<double> wt(nb);
   for (size_t bi = 0; bi < nb; ++bi) {
@@ -381,10 +344,6 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
     ED_TRY(read_scalars(c, 3, 1, &wt[bi], st));  // synchronises the stream
   }
   ED_TRY(oz_status(&oz, st));  // no bounded wait of the reduction's kernels ran out
-  const auto tq = std::chrono::steady_clock::now();
-  for (int k = 0; k < lanes; ++k)
-    for (auto& x : qr[k]) x.join();
-  const double t_qr = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tq).count();
   double t_gram = 0.0;
   float t_all = 0.f;
   for (size_t bi = 0; bi < nb; ++bi) {
@@ -393,24 +352,30 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
     t_gram += t1;
   }
   ED_CUDA_TRY(cudaEventElapsedTime(&t_all, ev_se.e[0], ev_se.e[1]));
-  int64_t pos = 0;
-  for (size_t bi = 0; bi < nb; ++bi) {
-    if (ok[bi] != 1) {
-      set_error(ok[bi] == 2 ? "waiting for block %zu's reduction failed" : "tridiagonal QL did not converge on block %zu",
-                bi);
-      return ED_ENOCONV;
+  for (size_t i = 0; i < sblk.size(); ++i) {
+    double* w = lam.data() + sblk[i].off;
+    const size_t n = (size_t)sblk[i].n;
+    if (!std::isfinite(lam[need + i])) {  // entries that are not finite: the host iteration's answer
+      std::vector<double> dd(n), ee(n);
+      ED_CUDA_TRY(cudaMemcpy(dd.data(), d_de + 2 * sblk[i].off, n * sizeof(double), cudaMemcpyDeviceToHost));
+      ED_CUDA_TRY(cudaMemcpy(ee.data(), d_de + 2 * sblk[i].off + n, (n - 1) * sizeof(double), cudaMemcpyDeviceToHost));
+      ee.resize(n - 1);
+      if (!tridiag_eigenvalues(dd, ee)) {
+        set_error("tridiagonal QL did not converge on a block of %zu levels", n);
+        return ED_ENOCONV;
+      }
+      std::copy(dd.begin(), dd.end(), w);
     }
-    std::vector<double>& w = dd[bi];
-    std::sort(w.begin(), w.end(), [](double u, double v) { return u > v; });  // descending
-    for (size_t i = 0; i < w.size(); ++i) lambda[pos + i] = w[i];
-    pos += (int64_t)w.size();
+    // descending (neighbours within the brackets' width may be swapped)
+    if (!std::is_sorted(w, w + n, std::greater<double>())) std::sort(w, w + n, std::greater<double>());
   }
+  std::copy(lam.begin(), lam.begin() + need, lambda);
   if (stage_ms) {
     // with the blocks on several streams the Gram products overlap other
     // blocks' reductions: [0] = the Gram products' own device time, [1] =
-    // the rest of the call's device time plus the host QL left at its end
+    // the rest of the call's device time
     stage_ms[0] = t_gram;
-    stage_ms[1] = std::max(0.0, (double)t_all - t_gram) + t_qr;
+    stage_ms[1] = std::max(0.0, (double)t_all - t_gram);
   }
   double tot = 0.0;
   for (double v : wt) tot += v;
