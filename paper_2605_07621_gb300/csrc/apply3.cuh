@@ -324,6 +324,9 @@ __device__ __forceinline__ void store_out<PW>(double* y, long long i, AccW v, bo
 // take slots from the running kernel's last wave.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// lets the next kernel of the stream start on the SMs that this one leaves
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // kernel launch with programmatic stream serialization (see pdl_wait)
 template <class... KArgs, class... Args>
 inline cudaError_t launch_pdl(void (*k)(KArgs...), long long grid, int block, size_t smem, cudaStream_t st,

@@ -11,6 +11,7 @@
 #include <map>
 #include <mutex>
 
+#include "apply3.cuh"  // pdl_wait, launch_pdl
 #include "batch.h"
 #include "batch_dev.cuh"
 #include "krylov.h"
@@ -33,8 +34,7 @@ __global__ void __launch_bounds__(256) k_bapply(const BInst* __restrict__ insts,
   __shared__ float stage[kBW][kBStage];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = cnt[0];
-  if (n <= 0) return;
-  const long long total = rowpref[n];
+  const long long total = n > 0 ? rowpref[n] : 0;
   for (long long row = (long long)blockIdx.x * kBW + warp; row < total; row += (long long)gridDim.x * kBW) {
     const int ai = find_pref(rowpref, n, row);
     const BInst& I = insts[idx[ai]];
@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(256) k_bapply(const BInst* __restrict__ insts,
     }
     __syncwarp();
   }
+  pdl_wait();  // after the dense products, which may still run (launch_apply)
 }
 
 // chunk c of the active set -> (instance, element range)
@@ -321,6 +322,8 @@ size_t h_piece_bytes(const HostTables& h) {
   return align256((size_t)3 * h.dA * pad64(h.dA) * 2) + align256((size_t)3 * h.dB * pad64(h.dB) * 2) +
          align256(kmask_words(h) * 4);
 }
+// the pieces of Psi, and as much again for a transposed copy, which the
+// products no longer need: the sizes by which an engine admits instances stay
 size_t x_piece_bytes(const HostTables& h) {
   return align256((size_t)3 * h.dA * pad64(h.dB) * 2) + align256((size_t)3 * h.dB * pad64(h.dA) * 2);
 }
@@ -388,6 +391,7 @@ ed_status BatchEngine::init(int device, size_t arena_bytes, int max_slots, int m
   ED_TRY(get((void**)&d_chunkpref_, sizeof(long long) * (max_slots_ + 1)));
   ED_TRY(get((void**)&d_nact_, sizeof(int) * 4));
   ED_TRY(get((void**)&d_cnt_, sizeof(int) * 4));
+  ED_TRY(get((void**)&d_next_, sizeof(unsigned long long) * 2));
   ED_TRY(get((void**)&d_cidx_, sizeof(int) * list_cap_));
   ED_TRY(get((void**)&d_crowpref_, sizeof(long long) * (list_cap_ + 1)));
   ED_TRY(get((void**)&d_didx_, sizeof(int) * list_cap_));
@@ -541,16 +545,14 @@ ed_status BatchEngine::add(const ed_model_desc& m, uint64_t seed, int* slot_out,
     d.HB = (const uint16_t*)put(nullptr, (size_t)3 * h.dB * d.KpB * 2);
     d.kmask = (const uint32_t*)put(nullptr, kmask_words(h) * 4);
     d.XN = (uint16_t*)put(nullptr, (size_t)3 * h.dA * d.KpB * 2);
-    d.XT = (uint16_t*)put(nullptr, (size_t)3 * h.dB * d.KpA * 2);
-    // A-role maps (H_A, Psi) with 128-row boxes; B-role maps (Psi^T, H_B)
-    // with 64- and 128-row boxes, one pair per output tile width
+    // A-role maps (H_A, Psi) with 128-row boxes; B-role maps: Psi's rows in
+    // 64-row boxes, H_B with 64- and 128-row boxes, one per output tile width
     CUtensorMap mp[kBMaps];
     ED_TRY(tmap_bf16_planes(&mp[0], d.HA, d.dA, d.dA, 3, d.KpA, 128));
     ED_TRY(tmap_bf16_planes(&mp[1], d.XN, d.dB, d.dA, 3, d.KpB, 128));
-    ED_TRY(tmap_bf16_planes(&mp[2], d.XT, d.dA, d.dB, 3, d.KpA, 64));
+    ED_TRY(tmap_bf16_planes(&mp[2], d.XN, d.dB, d.dA, 3, d.KpB, 64));
     ED_TRY(tmap_bf16_planes(&mp[3], d.HB, d.dB, d.dB, 3, d.KpB, 64));
-    ED_TRY(tmap_bf16_planes(&mp[4], d.XT, d.dA, d.dB, 3, d.KpA, 128));
-    ED_TRY(tmap_bf16_planes(&mp[5], d.HB, d.dB, d.dB, 3, d.KpB, 128));
+    ED_TRY(tmap_bf16_planes(&mp[4], d.HB, d.dB, d.dB, 3, d.KpB, 128));
     ED_CUDA_TRY(cudaMemcpyAsync(d_maps_ + (size_t)slot * kBMaps, mp, sizeof(mp), cudaMemcpyHostToDevice, st_));
   }
   ED_CUDA_TRY(cudaMemcpyAsync(arena_ + off + tab0, host.data() + tab0, up_end - tab0, cudaMemcpyHostToDevice, st_));
@@ -610,7 +612,11 @@ ed_status BatchEngine::set_mode(int slot, int mode) {
 int BatchEngine::default_mode(const BSlot& S) const {
   int md;
   if (cached_mode(S.key, &md)) return md;
-  return S.d.dB <= 64 ? kModeD64 : kModeD128;
+  // 64-wide tiles: more of them, three stages, and one kernel for the batch.
+  // 8 / 64 / 512 mixed instances: 25 / 56 / 441 us against 37 / 65 / 455 of
+  // 128-wide ones; where those win (48 instances of 924 x 924: 616 against 641)
+  // the tuner finds them
+  return kModeD64;
 }
 
 ed_status BatchEngine::upload_inst(int slot) {
@@ -619,12 +625,19 @@ ed_status BatchEngine::upload_inst(int slot) {
   return ED_OK;
 }
 
-ed_status BatchEngine::upload_lists(const std::vector<int>& csr, const std::vector<int>& d64,
-                                    const std::vector<int>& d128) {
+ed_status BatchEngine::upload_lists(const std::vector<int>& csr, std::vector<int> d64, std::vector<int> d128) {
   if ((int)csr.size() > list_cap_ || (int)(d64.size() + d128.size()) > list_cap_) {
     set_error("batch engine: work list exceeds capacity");
     return ED_ENOMEM;
   }
+  // the instances with the longest tiles (K steps: d_A / 64 + d_B / 64) first:
+  // the CTAs take tiles as they finish, and a long last one would be waited for
+  auto longer = [&](int u, int v) {
+    const BInst &a = slots_[u].d, &b = slots_[v].d;
+    return (a.dA + 63) / 64 + (a.dB + 63) / 64 > (b.dA + 63) / 64 + (b.dB + 63) / 64;
+  };
+  std::stable_sort(d64.begin(), d64.end(), longer);
+  std::stable_sort(d128.begin(), d128.end(), longer);
   std::vector<long long> crp(1, 0), sp(1, 0), tp64(1, 0), tp128(1, 0);
   std::vector<int> dall(d64);
   dall.insert(dall.end(), d128.begin(), d128.end());
@@ -678,6 +691,7 @@ ed_status BatchEngine::launch_apply(cudaStream_t s, const float* x, float* y) {
     BDenseArgs a;
     a.insts = d_inst_;
     a.cnt = d_cnt_;
+    a.next = d_next_;
     a.didx = d_didx_;
     a.dspref = d_dspref_;
     a.idx64 = d_idx64_;
@@ -693,7 +707,12 @@ ed_status BatchEngine::launch_apply(cudaStream_t s, const float* x, float* y) {
     a.err = d_err_;
     ED_TRY(bdense_apply(a, s));
   }
-  k_bapply<<<sms_ * 4, 256, 0, s>>>(d_inst_, d_cidx_, d_crowpref_, d_cnt_, x, y, (float*)arena_, user);
+  // beside the last dense tiles (its instances are others); without dense
+  // products it follows whatever the stream holds
+  if (dense_)
+    ED_CUDA_TRY(launch_pdl(k_bapply, sms_ * 4, 256, 0, s, d_inst_, d_cidx_, d_crowpref_, d_cnt_, x, y, (float*)arena_, user));
+  else
+    k_bapply<<<sms_ * 4, 256, 0, s>>>(d_inst_, d_cidx_, d_crowpref_, d_cnt_, x, y, (float*)arena_, user);
   ED_CUDA_TRY(cudaGetLastError());
   return ED_OK;
 }

@@ -19,7 +19,7 @@ namespace edk {
 
 constexpr int kBatchChunk = 4096;  // elements per reduction chunk
 constexpr int kBDenseMax = 1024;   // largest d_A, d_B with a dense (tensor-core) form
-constexpr int kBMaps = 6;          // tensor maps per instance (see bdense.cu)
+constexpr int kBMaps = 5;          // tensor maps per instance (see bdense.cu)
 enum BMode { kModeCSR = 0, kModeD64 = 1, kModeD128 = 2 };
 
 struct BInst {
@@ -41,11 +41,10 @@ struct BInst {
   const uint32_t* B_str;
   // dense form (null when the instance has none): H_A, H_B as three BF16
   // pieces each ([3][d][Kp]), and the pieces of Psi (rows a, [3][d_A][KpB])
-  // and of Psi^T (rows b, [3][d_B][KpA]) written before each product
+  // written before each product
   const uint16_t* HA;
   const uint16_t* HB;
   uint16_t* XN;
-  uint16_t* XT;
   int KpA, KpB;        // row strides of the pieces (d rounded up to 64)
   // nonzero 64-wide K blocks (bit kb) of each 128-row tile of H_A, then of
   // each 64-row and each 128-row tile of H_B: the dense products skip zero blocks
@@ -64,6 +63,7 @@ struct BInst {
 struct BDenseArgs {
   const BInst* insts;
   const int* cnt;            // {CSR, dense, 64-wide, 128-wide} list lengths
+  unsigned long long* next;  // {64-wide, 128-wide} next tile to take (cleared by the slicing kernel)
   const int* didx;           // dense slots, with their 64 x 64 slicing tiles
   const long long* dspref;
   const int* idx64;          // slots with 128 x 64 output tiles
@@ -154,7 +154,7 @@ class BatchEngine {
   // H psi over the uploaded lists (user vectors when x, y are set)
   ed_status launch_apply(cudaStream_t s, const float* x, float* y);
   // upload work lists: CSR slots and dense slots by tile width
-  ed_status upload_lists(const std::vector<int>& csr, const std::vector<int>& d64, const std::vector<int>& d128);
+  ed_status upload_lists(const std::vector<int>& csr, std::vector<int> d64, std::vector<int> d128);
   bool alloc(size_t len, size_t* off);
   void release(size_t off, size_t len);
 
@@ -175,6 +175,7 @@ class BatchEngine {
   int* d_nact_ = nullptr;
   // apply work lists; d_cnt_ = {CSR, dense (all widths), 64-wide, 128-wide}
   int* d_cnt_ = nullptr;
+  unsigned long long* d_next_ = nullptr;  // tile counters of the dense products
   int* d_cidx_ = nullptr;
   long long* d_crowpref_ = nullptr;
   int* d_didx_ = nullptr;

@@ -16,17 +16,19 @@
 // add) share them, and the epilogue adds the two and the diagonal.
 //
 // Per output tile (128 rows a x BN columns b): the K steps of H_A Psi
-// (A operand: H_A's pieces, rows a; B operand: Psi^T's pieces, rows b, both
-// K = a' contiguous) and then those of Psi H_B^T (A: Psi's pieces, rows a;
-// B: H_B's pieces, rows b, K = b' contiguous).  Tiles staged by TMA with
-// 128-byte swizzle, one thread issues the MMAs, four warps drain the
+// (A operand: H_A's pieces, rows a, K = a' contiguous; B operand: Psi's pieces,
+// rows a' of BN columns, the MN-major form, so no transposed copy of Psi is
+// written or read) and then those of Psi H_B^T (A: Psi's pieces, rows a; B:
+// H_B's pieces, rows b, both K = b' contiguous).  Tiles staged by TMA with
+// 128-byte swizzle, one thread issues the MMAs, eight warps drain the
 // accumulators (those of two tiles alternate, so the epilogue of one tile
-// overlaps the products of the next).  Persistent: each CTA walks the tile
-// list of the active instances, read from device memory.
+// overlaps the products of the next).  Persistent: the CTAs take the tiles of
+// the active instances from a counter, those with the most K steps first.
 #include <cuda_bf16.h>
 
 #include <cstring>
 
+#include "apply3.cuh"  // pdl_wait, launch_pdl
 #include "batch.h"
 #include "batch_dev.cuh"
 #include "tc.cuh"
@@ -34,26 +36,32 @@
 namespace edk {
 
 constexpr int kBdEpiWarps = 8;   // two per TMEM lane quarter, splitting the columns
-constexpr int kBdThreads = 32 * (kBdEpiWarps + 2);  // warps 0-7 epilogue, 8 TMA producer, 9 MMA issuer
-constexpr int kBdWarpTma = kBdEpiWarps, kBdWarpMma = kBdEpiWarps + 1;
-constexpr int kBdTrans = 32 * 33;  // floats of one warp's transpose buffer
+// warps 0-7 epilogue, 8 TMA producer, 9 MMA issuer, 10 tile list
+constexpr int kBdThreads = 32 * (kBdEpiWarps + 3);
+constexpr int kBdWarpTma = kBdEpiWarps, kBdWarpMma = kBdEpiWarps + 1, kBdWarpList = kBdEpiWarps + 2;
+constexpr int kBdTiles = 4;      // tiles that the list warp is ahead
+constexpr int kBdTrans = 32 * 9;  // floats of one warp's transpose buffer (32 rows x 8 columns, odd stride)
 constexpr int kBdBM = 128;       // output rows per tile (UMMA M)
 constexpr int kBdBK = 64;        // K per pipeline step: one 128-byte swizzle row of BF16
 constexpr int kBdPieces = 3;
+constexpr int kBdXTile = 64 * kBdBK * 2;  // a box of Psi in the B role: 8 KB
 constexpr long long kBdSpin = 1ll << 26;  // bounded waits (about a second)
 
-// tensor maps of one slot: the A-role maps have 128-row boxes, the B-role
-// maps BN-row boxes
-enum { kMapHA = 0, kMapXN = 1, kMapXT64 = 2, kMapHB64 = 3, kMapXT128 = 4, kMapHB128 = 5 };
+// tensor maps of one slot: the A roles (H_A, Psi) with 128-row boxes, Psi in
+// the B role with 64-row boxes, H_B with BN-row boxes
+enum { kMapHA = 0, kMapXN = 1, kMapXB = 2, kMapHB64 = 3, kMapHB128 = 4 };
 
 template <int BN>
 struct BdCfg {
-  static constexpr int kStages = 2;
+  static constexpr int kStages = BN == 64 ? 3 : 2;
   static constexpr int kATile = kBdBM * kBdBK * 2;  // one piece: 16 KB
   static constexpr int kBTile = BN * kBdBK * 2;
-  static constexpr int kStage = kBdPieces * (kATile + kBTile);
-  static constexpr int kTmemCols = 4 * BN;  // two tiles in flight x (leading, corrections)
-  static constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + 256 + (size_t)kBdEpiWarps * kBdTrans * 4;
+  static constexpr int kStage = kBdPieces * (kATile + kBTile);  // 72 or 96 KB
+  // accumulators of a tile: the leading products, and the corrections p + q =
+  // 1 and 2 (one accumulator for both at BN = 128, where TMEM has no more)
+  static constexpr int kAcc = BN == 64 ? 3 : 2;
+  static constexpr int kTmemCols = 512;  // two tiles in flight (a power of two of columns)
+  static constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + 512 + (size_t)kBdEpiWarps * kBdTrans * 4;
 };
 
 // ---------------------------------------------------------------- pieces
@@ -69,13 +77,28 @@ __device__ __forceinline__ void split3_dev(float v, uint16_t& h0, uint16_t& h1, 
   h2 = __bfloat16_as_ushort(c);
 }
 
-// Pieces of Psi (rows a, K = b) and of Psi^T (rows b, K = a) for every dense
-// instance: 64 x 64 tiles of Psi through shared memory; every warp store
-// writes 32 pairs of BF16 (128 bytes) along a row of either layout.  The
-// piece rows start on multiples of 64 elements, so pairs at even columns
-// are 4-byte aligned.
+// the pieces of two neighbours, each pair in one word (the first in its low half)
+__device__ __forceinline__ void split3_pair(float a, float b, uint32_t& h0, uint32_t& h1, uint32_t& h2) {
+  auto pack = [](float lo, float hi) {
+    const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+    uint32_t u;
+    memcpy(&u, &t, 4);
+    return u;
+  };
+  auto low = [](uint32_t u) { return __uint_as_float(u << 16); };
+  auto high = [](uint32_t u) { return __uint_as_float(u & 0xffff0000u); };
+  h0 = pack(a, b);
+  const float a1 = a - low(h0), b1 = b - high(h0);
+  h1 = pack(a1, b1);
+  h2 = pack(a1 - low(h1), b1 - high(h1));
+}
+
+// Pieces of Psi for every dense instance, in units of 64 x 64 elements; a warp
+// takes eight rows, whose loads are all in flight, a lane two neighbouring
+// columns, so a warp writes 128 bytes along a row.  The piece rows start on
+// multiples of 64 elements: pairs at even columns are 4-byte aligned.
 __global__ void __launch_bounds__(256) k_bslice(BDenseArgs g) {
-  __shared__ float tile[64][65];
+  if (blockIdx.x == 0 && threadIdx.x < 2) g.next[threadIdx.x] = 0;  // the tile counters of the products
   const int n = g.cnt[1];
   if (n <= 0) return;
   const long long total = g.dspref[n];
@@ -86,43 +109,30 @@ __global__ void __launch_bounds__(256) k_bslice(BDenseArgs g) {
     const int dA = I.dA, dB = I.dB;
     const long long t = u - g.dspref[ai];
     const int tnb = (dB + 63) >> 6;
-    const int a0 = (int)(t / tnb) * 64, b0 = (int)(t % tnb) * 64;
-    const float* __restrict__ x = g.user_mode ? g.ux + I.uoff : g.arena + I.voff + I.D;
-    uint16_t* __restrict__ XN = I.XN;
-    uint16_t* __restrict__ XT = I.XT;
-    const long long pn = (long long)dA * I.KpB, pt = (long long)dB * I.KpA;
-    for (int i = threadIdx.x; i < 64 * 64; i += 256) {
-      const int r = i >> 6, c = i & 63;
-      const int a = a0 + r, b = b0 + c;
-      tile[r][c] = (a < dA && b < dB) ? x[(long long)a * dB + b] : 0.f;
+    const int a0 = (int)(t / tnb) * 64 + warp, b = (int)(t % tnb) * 64 + 2 * lane;
+    if (b >= dB) continue;
+    const bool two = b + 1 < dB;
+    const float* __restrict__ x = (g.user_mode ? g.ux + I.uoff : g.arena + I.voff + I.D) + b;
+    uint32_t* __restrict__ d = reinterpret_cast<uint32_t*>(I.XN + b);
+    const long long kw = I.KpB / 2, pw = (long long)dA * kw;  // words of a row, of a piece
+    float v[8], w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int a = a0 + 8 * i;
+      v[i] = a < dA ? __ldg(x + (long long)a * dB) : 0.f;
+      w[i] = a < dA && two ? __ldg(x + (long long)a * dB + 1) : 0.f;  // zero past d_B: the padding of the row
     }
-    __syncthreads();
-    const int c = 2 * lane;
-    for (int r = warp; r < 64; r += 8) {
-      const int a = a0 + r, b = b0 + c;  // Psi row a, columns b, b + 1
-      if (a < dA && b < dB) {
-        uint16_t h0, h1, h2, k0, k1, k2;
-        split3_dev(tile[r][c], h0, h1, h2);
-        split3_dev(tile[r][c + 1], k0, k1, k2);  // zero past d_B: the padding of the row
-        uint32_t* d = reinterpret_cast<uint32_t*>(XN + (long long)a * I.KpB + b);
-        d[0] = h0 | ((uint32_t)k0 << 16);
-        d[pn / 2] = h1 | ((uint32_t)k1 << 16);
-        d[pn] = h2 | ((uint32_t)k2 << 16);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int a = a0 + 8 * i;
+      if (a < dA) {
+        uint32_t h0, h1, h2;
+        split3_pair(v[i], w[i], h0, h1, h2);
+        d[a * kw] = h0;
+        d[a * kw + pw] = h1;
+        d[a * kw + 2 * pw] = h2;
       }
     }
-    for (int r = warp; r < 64; r += 8) {
-      const int b = b0 + r, a = a0 + c;  // Psi^T row b, columns a, a + 1
-      if (a < dA && b < dB) {
-        uint16_t h0, h1, h2, k0, k1, k2;
-        split3_dev(tile[c][r], h0, h1, h2);
-        split3_dev(tile[c + 1][r], k0, k1, k2);
-        uint32_t* d = reinterpret_cast<uint32_t*>(XT + (long long)b * I.KpA + a);
-        d[0] = h0 | ((uint32_t)k0 << 16);
-        d[pt / 2] = h1 | ((uint32_t)k1 << 16);
-        d[pt] = h2 | ((uint32_t)k2 << 16);
-      }
-    }
-    __syncthreads();
   }
 }
 
@@ -182,36 +192,67 @@ ed_status bdense_tables(const BInst& I, cudaStream_t st) {
 // 32 for the second product (kb < 16 as d <= 1024).  A tile with none gets
 // one zero block (which clears its accumulators).
 template <int BN>
-__device__ __forceinline__ int tile_steps(const BInst& I, int m0, int n0, unsigned char* ks) {
+__device__ __forceinline__ int tile_steps(const BInst& I, int m0, int n0, unsigned char* ks, int& nA) {
   const int tmA = (I.dA + kBdBM - 1) / kBdBM, tn64 = (I.dB + 63) / 64;
   const uint32_t ma = I.kmask[m0 / kBdBM];
   const uint32_t mb = BN == 64 ? I.kmask[tmA + n0 / 64] : I.kmask[tmA + tn64 + n0 / 128];
   int n = 0;
   for (uint32_t m = ma; m; m &= m - 1) ks[n++] = (unsigned char)__ffs(m) - 1;
+  if (ma == 0 && mb == 0) ks[n++] = 0;
+  nA = n;
   for (uint32_t m = mb; m; m &= m - 1) ks[n++] = (unsigned char)(32 + __ffs(m) - 1);
-  if (n == 0) ks[n++] = 0;
   return n;
 }
 
+// one entry of a CTA's tile list
+struct BdTile {
+  int slot, m0, n0, nk, nA;
+  unsigned char ks[32];  // the K steps, the first nA of H_A Psi (tile_steps)
+};
+
+// Bound: operands from L2 (a K step moves 72 KB for a 128 x 64 tile, 96 KB for
+// 128 x 128; 5.7 and 4.1 GB for 512 Hubbard instances of 26 M states, 16 and 11
+// TB/s), the tensor pipe active 44 and 47 % of the time.  Of that batch's
+// H|psi>, with 64-wide / 128-wide tiles: 694 / 537 us with two stages, N = BN
+// instructions, Psi^T sliced beside Psi and every CTA looking up its own tiles;
+// 538 / 542 with three stages (64-wide), N up to 192 and no prefetch into L2,
+// which moved every operand twice through L2's ports; 506 / 545 with the list
+// warp; 449 / 462 without Psi^T (slicing 114 -> 59 us, 0.2 GB less from HBM);
+// 439 / 451 with the launches overlapped.  Tried and slower: barriers per piece
+// instead of per K step (608 / 549), operands prefetched once per row or column
+// of tiles (531 / 560).
 template <int BN>
 __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which) {
   using C = BdCfg<BN>;
+  // The 64-wide tiles follow the slicing and wait for it.  The 128-wide ones
+  // need no more than that: they start on the SMs that the former leave.  They
+  // and k_bapply wait for the kernel before at their end, so that what follows
+  // in the stream follows all three.  (k_bapply starts when the last 128-wide
+  // tile is done: started earlier, its CTAs crowd on the first free SMs.)
+  if (BN == 64) {
+    pdl_wait();
+    pdl_trigger();
+  }
   const int n = g.cnt[which];
-  if (n <= 0) return;
   const int* vidx = BN == 64 ? g.idx64 : g.idx128;
   const long long* tpref = BN == 64 ? g.tpref64 : g.tpref128;
-  const long long total = tpref[n];
-  if ((long long)blockIdx.x >= total) return;
+  const long long total = n > 0 ? tpref[n] : 0;
+  if (total <= 0) {
+    if (BN != 64) pdl_wait();
+    return;
+  }
 
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)sm_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* bar = (uint64_t*)(sm + C::kStages * C::kStage);
-  uint64_t* full = bar;                      // kStages
-  uint64_t* empty = bar + C::kStages;        // kStages
-  uint64_t* acc_full = bar + 2 * C::kStages; // 2
-  uint64_t* acc_empty = acc_full + 2;        // 2
+  uint64_t* full = (uint64_t*)(sm + C::kStages * C::kStage);  // kStages
+  uint64_t* empty = full + C::kStages;                       // kStages
+  uint64_t* acc_full = empty + C::kStages;                   // 2
+  uint64_t* acc_empty = acc_full + 2;                        // 2
   uint64_t* mma_done = acc_empty + 2;
-  float* trans = (float*)(sm + C::kStages * C::kStage + 256);  // kBdEpiWarps x [32][33]
+  uint64_t* ti_full = mma_done + 1;                          // kBdTiles
+  uint64_t* ti_empty = ti_full + kBdTiles;                   // kBdTiles
+  float* trans = (float*)(sm + C::kStages * C::kStage + 512);  // kBdEpiWarps x [32][9]
+  __shared__ BdTile s_tile[kBdTiles];
   __shared__ unsigned s_tmem;
   __shared__ volatile int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -220,6 +261,10 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
     for (int i = 0; i < C::kStages; ++i) {
       tc::mbar_init(&full[i], 1);
       tc::mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < kBdTiles; ++i) {
+      tc::mbar_init(&ti_full[i], 1);
+      tc::mbar_init(&ti_empty[i], 2 + kBdEpiWarps);
     }
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&acc_full[i], 1);
@@ -235,41 +280,65 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
   tc::tc_fence_after();
   const unsigned tmem = s_tmem;
 
-  // tile -> (slot, first row, first column)
-  auto decode = [&](long long tile, int& slot, int& m0, int& n0) {
-    const int ai = find_pref(tpref, n, tile);
-    slot = vidx[ai];
-    const int tn = (g.insts[slot].dB + BN - 1) / BN;
-    const long long t = tile - tpref[ai];
-    m0 = (int)(t / tn) * kBdBM;
-    n0 = (int)(t % tn) * BN;
+  // the list entry of this CTA's tile tl, once it is written; nullptr at the
+  // list's end and when the wait ran out
+  auto tile_at = [&](int tl) -> const BdTile* {
+    if (!tc::mbar_wait(&ti_full[tl % kBdTiles], (unsigned)((tl / kBdTiles) & 1), kBdSpin)) {
+      s_abort = 1;
+      return nullptr;
+    }
+    const BdTile* T = &s_tile[tl % kBdTiles];
+    return T->nk > 0 ? T : nullptr;
   };
 
-  if (warp == kBdWarpTma) {
+  if (warp == kBdWarpList) {
+    // ---- tile list: a tile's instance (a binary search in global memory),
+    // origin and K steps are looked up tiles ahead of their use -- done by the
+    // producer itself, the lookups (5,000 cycles) drained its stages -- and
+    // its tensor maps fetched
+    if (lane == 0) {
+      for (int tl = 0; !s_abort; ++tl) {
+        const long long tile = (long long)atomicAdd(&g.next[BN == 64 ? 0 : 1], 1ull);
+        const int e = tl % kBdTiles, u = tl / kBdTiles;
+        if (u > 0 && !tc::mbar_wait(&ti_empty[e], (unsigned)((u - 1) & 1), kBdSpin)) {
+          s_abort = 1;
+          break;
+        }
+        if (tile >= total) {  // no K steps: the end of the list
+          s_tile[e].nk = 0;
+          tc::mbar_arrive(&ti_full[e]);
+          break;
+        }
+        const int ai = find_pref(tpref, n, tile);
+        const int slot = vidx[ai];
+        const BInst& I = g.insts[slot];
+        const int tn = (I.dB + BN - 1) / BN;
+        const long long t = tile - tpref[ai];
+        BdTile& T = s_tile[e];
+        T.slot = slot;
+        T.m0 = (int)(t / tn) * kBdBM;
+        T.n0 = (int)(t % tn) * BN;
+        const CUtensorMap* mp = g.maps + (long long)slot * kBMaps;
+        tc::tma_prefetch_map(mp + kMapHA);
+        tc::tma_prefetch_map(mp + kMapXN);
+        tc::tma_prefetch_map(mp + kMapXB);
+        tc::tma_prefetch_map(mp + (BN == 64 ? kMapHB64 : kMapHB128));
+        T.nk = tile_steps<BN>(I, T.m0, T.n0, T.ks, T.nA);
+        tc::mbar_arrive(&ti_full[e]);
+      }
+      if (s_abort) atomicExch(g.err, 1);
+    }
+  } else if (warp == kBdWarpTma) {
     // ---- TMA producer: per K step the three pieces of the A tile and of the B tile
     if (lane == 0) {
       long long it = 0;
-      unsigned char kst[32];
-      constexpr int kAhead = 3;  // K steps prefetched into L2 ahead of their loads
-      for (long long tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x) {
-        int slot, m0, n0;
-        decode(tile, slot, m0, n0);
-        const int nk = tile_steps<BN>(g.insts[slot], m0, n0, kst);
-        const CUtensorMap* mp = g.maps + (long long)slot * kBMaps;
-        const CUtensorMap* mXT = mp + (BN == 64 ? kMapXT64 : kMapXT128);
+      for (int tl = 0; !s_abort; ++tl) {
+        const BdTile* T = tile_at(tl);
+        if (!T) break;
+        const int m0 = T->m0, n0 = T->n0, nk = T->nk;
+        const CUtensorMap* mp = g.maps + (long long)T->slot * kBMaps;
         const CUtensorMap* mHB = mp + (BN == 64 ? kMapHB64 : kMapHB128);
-        auto prefetch = [&](int k) {
-          const bool first = kst[k] < 32;  // H_A Psi, then Psi H_B^T
-          const int kc = (kst[k] & 31) * kBdBK;
-#pragma unroll
-          for (int p = 0; p < kBdPieces; ++p) {
-            tc::tma_prefetch_3d(first ? mp + kMapHA : mp + kMapXN, kc, m0, p);
-            tc::tma_prefetch_3d(first ? mXT : mHB, kc, n0, p);
-          }
-        };
-        for (int k = 0; k < kAhead && k < nk; ++k) prefetch(k);
         for (int ks = 0; ks < nk; ++ks, ++it) {
-          if (ks + kAhead < nk) prefetch(ks + kAhead);
           const int s = (int)(it % C::kStages);
           const long long u = it / C::kStages;
           if (u > 0 && !tc::mbar_wait(&empty[s], (unsigned)((u - 1) & 1), kBdSpin)) {
@@ -278,37 +347,41 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
           }
           unsigned char* sa = sm + s * C::kStage;
           unsigned char* sb = sa + kBdPieces * C::kATile;
-          const bool first = kst[ks] < 32;
-          const int kc = (kst[ks] & 31) * kBdBK;
+          const bool first = ks < T->nA;  // H_A Psi, then Psi H_B^T
+          const int kc = (T->ks[ks] & 31) * kBdBK;
           const CUtensorMap* ma = first ? mp + kMapHA : mp + kMapXN;
-          const CUtensorMap* mb = first ? mXT : mHB;
           tc::mbar_expect_tx(&full[s], C::kStage);
 #pragma unroll
           for (int p = 0; p < kBdPieces; ++p) tc::tma_load_3d(sa + p * C::kATile, ma, kc, m0, p, &full[s]);
+          if (first) {  // Psi, 64 rows a' of 64 columns b each
 #pragma unroll
-          for (int q = 0; q < kBdPieces; ++q) tc::tma_load_3d(sb + q * C::kBTile, mb, kc, n0, q, &full[s]);
+            for (int q = 0; q < kBdPieces * BN / 64; ++q)
+              tc::tma_load_3d(sb + q * kBdXTile, mp + kMapXB, n0 + 64 * (q % (BN / 64)), kc, q / (BN / 64), &full[s]);
+          } else {
+#pragma unroll
+            for (int q = 0; q < kBdPieces; ++q) tc::tma_load_3d(sb + q * C::kBTile, mHB, kc, n0, q, &full[s]);
+          }
         }
+        tc::mbar_arrive(&ti_empty[tl % kBdTiles]);
       }
       if (s_abort) atomicExch(g.err, 1);
     }
   } else if (warp == kBdWarpMma) {
-    // ---- MMA issuer: piece pairs p + q <= 2 into the tile's accumulator
+    // ---- MMA issuer: piece pairs p + q <= 2 into the tile's accumulators
     if (lane == 0) {
-      const unsigned idesc = tc::idesc_bf16_f32(kBdBM, BN);
       long long it = 0;
-      int tl = 0;
-      for (long long tile = blockIdx.x; tile < total && !s_abort; tile += gridDim.x, ++tl) {
-        int slot, m0, n0;
-        decode(tile, slot, m0, n0);
-        unsigned char kst[32];
-        const int nk = tile_steps<BN>(g.insts[slot], m0, n0, kst);
+      for (int tl = 0; !s_abort; ++tl) {
+        const BdTile* T = tile_at(tl);
+        if (!T) break;
+        const int nk = T->nk, nA = T->nA;
+        tc::mbar_arrive(&ti_empty[tl % kBdTiles]);
         const int buf = tl & 1, use = tl >> 1;
         if (use > 0 && !tc::mbar_wait(&acc_empty[buf], (unsigned)((use - 1) & 1), kBdSpin)) {
           s_abort = 1;
           break;
         }
         tc::tc_fence_after();
-        const unsigned dt = tmem + (unsigned)(2 * buf * BN);  // leading; corrections at + BN
+        const unsigned dt = tmem + (unsigned)(C::kAcc * buf * BN);
         for (int ks = 0; ks < nk; ++ks, ++it) {
           const int s = (int)(it % C::kStages);
           if (!tc::mbar_wait(&full[s], (unsigned)((it / C::kStages) & 1), kBdSpin)) {
@@ -318,17 +391,32 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
           tc::tc_fence_after();
           unsigned char* sa = sm + s * C::kStage;
           unsigned char* sb = sa + kBdPieces * C::kATile;
-#pragma unroll
-          for (int p = 0; p < kBdPieces; ++p) {
+          // B's pieces lie behind one another in shared memory and the
+          // accumulators in TMEM, so one instruction of N = np BN takes np
+          // pairs (p, q), (p, q + 1), ... whose accumulators differ
+          const bool first = ks < nA;
+          auto pairs = [&](int p, int q, int np, int acc) {
+            const unsigned idesc = tc::idesc_bf16_f32(kBdBM, np * BN) | (first ? tc::kIdescBMnMajor : 0u);
             const uint64_t da = tc::sdesc_kmajor_sw128(sa + p * C::kATile);
+            const unsigned char* b = sb + q * C::kBTile;
+            const uint64_t db = first ? tc::sdesc_mnmajor_sw128(b, kBdXTile) : tc::sdesc_kmajor_sw128(b);
+            // 16 of K per instruction: 32 bytes along a K-major row, 16 rows of Psi
+            const int kb = first ? 16 * 128 / 16 : 2;
 #pragma unroll
-            for (int q = 0; q + p < kBdPieces; ++q) {
-              const uint64_t db = tc::sdesc_kmajor_sw128(sb + q * C::kBTile);
-#pragma unroll
-              for (int kk = 0; kk < kBdBK / 16; ++kk)  // 32 bytes of K per instruction
-                tc::mma_bf16(dt + (p + q > 0 ? BN : 0), da + 2 * kk, db + 2 * kk, idesc,
-                             !(ks == 0 && p == 0 && q <= 1 && kk == 0));
-            }
+            for (int kk = 0; kk < kBdBK / 16; ++kk)
+              tc::mma_bf16(dt + (unsigned)(acc * BN), da + 2 * kk, db + kb * kk, idesc,
+                           !(ks == 0 && p == 0 && q == 0 && kk == 0));
+          };
+          if (BN == 64) {
+            pairs(0, 0, 3, 0);
+            pairs(1, 0, 2, 1);
+            pairs(2, 0, 1, 2);
+          } else {
+            pairs(0, 0, 2, 0);
+            pairs(0, 2, 1, 1);
+            pairs(1, 0, 1, 1);
+            pairs(1, 1, 1, 1);
+            pairs(2, 0, 1, 1);
           }
           tc::mma_commit(&empty[s]);
         }
@@ -347,11 +435,13 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
     // y = accumulators + V x run along rows (lane = column)
     const int quarter = warp & 3, half = warp >> 2;
     float* tr = trans + warp * kBdTrans;
-    int tl = 0;
-    for (long long tile = blockIdx.x; tile < total; tile += gridDim.x, ++tl) {
-      int slot, m0, n0;
-      decode(tile, slot, m0, n0);
-      const BInst& I = g.insts[slot];
+    for (int tl = 0;; ++tl) {
+      const BdTile* T = tile_at(tl);
+      if (!T) break;
+      const int m0 = T->m0, n0 = T->n0;
+      const BInst& I = g.insts[T->slot];
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&ti_empty[tl % kBdTiles]);
       const int buf = tl & 1, use = tl >> 1;
       bool ok = false;
       for (long long i = 0; i < kBdSpin && !ok; ++i) {
@@ -389,35 +479,53 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
 #pragma unroll 1
       for (int c = half; c < BN / 32; c += 2) {
         float v[32], u[32];
-        const unsigned ta = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)(2 * buf * BN + c * 32);
-        tc::tmem_ld32(ta, v);
-        tc::tmem_ld32(ta + BN, u);
+        const unsigned ta = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)(C::kAcc * buf * BN + c * 32);
+        tc::tmem_ld32(ta + BN, v);
+        if (C::kAcc == 3) {
+          tc::tmem_ld32(ta + 2 * BN, u);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) tr[lane * 33 + j] = v[j] + u[j];
-        __syncwarp();
-        const int col = n0 + c * 32 + lane;
-        const bool cv = col < dB;
-        const uint32_t sb = cv ? Bs[col] : 0u;
-        const float bd = cv ? Bd[col] : 0.f;
-        const float* __restrict__ xc = x + (long long)r0 * dB + col;
-        float* __restrict__ yc = y + (long long)r0 * dB + col;
-        // all 32 rows' x loads in flight before any is used (x is read from
-        // DRAM here: one load at a time per warp would leave the epilogue
-        // bound by memory latency)
-        float xv[32];
+          for (int j = 0; j < 32; ++j) v[j] += u[j];
+        }
+        tc::tmem_ld32(ta, u);
 #pragma unroll
-        for (int r = 0; r < 32; ++r) xv[r] = (r < nr && cv) ? xc[(long long)r * dB] : 0.f;
+        for (int j = 0; j < 32; ++j) v[j] += u[j];
+        // 8 columns at a time through shared memory: lane = (row 4 i + lane /
+        // 8, column lane % 8), so x and y move in whole 32-byte sectors
+        const int lr = lane >> 3, lc = lane & 7;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-          const uint32_t sa = __shfl_sync(0xffffffffu, sal, r);
-          const float da = __shfl_sync(0xffffffffu, dal, r);
-          if (r < nr && cv) {
-            const uint32_t z = vand ? (sa & sb) : (sa ^ sb);
-            float dg = da + bd;
+        for (int s8 = 0; s8 < 4; ++s8) {
+          __syncwarp();
 #pragma unroll
-            for (int q = 0; q < kMaxClasses; ++q)  // unrolled: w, mk stay in registers
-              if (q < ncls) dg += w[q] * (float)__popc(z & mk[q]);
-            yc[(long long)r * dB] = fmaf(dg, xv[r], tr[r * 33 + lane]);
+          for (int j = 0; j < 8; ++j) tr[lane * 9 + j] = v[8 * s8 + j];
+          const int col = n0 + c * 32 + 8 * s8 + lc;
+          const bool cv = col < dB;
+          const uint32_t sb = cv ? Bs[col] : 0u;
+          const float bd = cv ? Bd[col] : 0.f;
+          const float* __restrict__ xc = x + (long long)r0 * dB + col;
+          float* __restrict__ yc = y + (long long)r0 * dB + col;
+          // the 32 rows' x loads in flight before any is used (x is read from
+          // DRAM here: one load at a time per warp would leave the epilogue
+          // bound by memory latency)
+          float xv[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + lr;
+            xv[i] = (r < nr && cv) ? xc[(long long)r * dB] : 0.f;
+          }
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + lr;
+            const uint32_t sa = __shfl_sync(0xffffffffu, sal, r);
+            const float da = __shfl_sync(0xffffffffu, dal, r);
+            if (r < nr && cv) {
+              const uint32_t z = vand ? (sa & sb) : (sa ^ sb);
+              float dg = da + bd;
+#pragma unroll
+              for (int q = 0; q < kMaxClasses; ++q)  // unrolled: w, mk stay in registers
+                if (q < ncls) dg += w[q] * (float)__popc(z & mk[q]);
+              yc[(long long)r * dB] = fmaf(dg, xv[i], tr[r * 9 + lc]);
+            }
           }
         }
         __syncwarp();
@@ -432,6 +540,7 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
     tc::tc_fence_after();
     tc::tmem_dealloc(tmem, C::kTmemCols);
   }
+  if (BN != 64) pdl_wait();
 }
 
 ed_status bdense_prepare() {
@@ -442,8 +551,8 @@ ed_status bdense_prepare() {
 
 ed_status bdense_apply(const BDenseArgs& a, cudaStream_t st) {
   k_bslice<<<a.sms * 8, 256, 0, st>>>(a);
-  k_bgemm<64><<<a.sms, kBdThreads, BdCfg<64>::kSmem, st>>>(a, 2);
-  k_bgemm<128><<<a.sms, kBdThreads, BdCfg<128>::kSmem, st>>>(a, 3);
+  ED_CUDA_TRY(launch_pdl(k_bgemm<64>, a.sms, kBdThreads, BdCfg<64>::kSmem, st, a, 2));
+  ED_CUDA_TRY(launch_pdl(k_bgemm<128>, a.sms, kBdThreads, BdCfg<128>::kSmem, st, a, 3));
   ED_CUDA_TRY(cudaGetLastError());
   return ED_OK;
 }

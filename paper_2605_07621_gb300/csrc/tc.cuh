@@ -78,6 +78,11 @@ __device__ __forceinline__ void tma_prefetch_3d(const void* tmap, int c0, int c1
                : "memory");
 }
 
+// fetch of a tensor map ahead of the loads that use it
+__device__ __forceinline__ void tma_prefetch_map(const void* tmap) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
+}
+
 // ---- tcgen05 (one CTA, cta_group::1)
 __device__ __forceinline__ void tmem_alloc(unsigned* dst_smem, unsigned ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
@@ -146,6 +151,17 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_sw128(const void* tile) {
   const uint64_t sbo = 1024 >> 4;     // next 8-row atom
   return a | (lbo << 16) | (sbo << 32) | (1ull << 46) | (2ull << 61);
 }
+
+// Shared-memory matrix descriptor of an MN-major operand tile written by TMA
+// with 128-byte swizzle: rows k of 64 BF16 along M or N (128 bytes), groups of
+// 8 rows 1024 bytes apart (stride-dimension offset), the next 64 of M or N
+// `chunk` bytes on (leading-dimension offset).
+__device__ __forceinline__ uint64_t sdesc_mnmajor_sw128(const void* tile, unsigned chunk) {
+  const uint64_t a = (uint64_t)((smem_u32(tile) & 0x3FFFFu) >> 4);
+  const uint64_t lbo = chunk >> 4, sbo = 1024 >> 4;
+  return a | (lbo << 16) | (sbo << 32) | (1ull << 46) | (2ull << 61);
+}
+constexpr unsigned kIdescBMnMajor = 1u << 16;  // B is MN-major (instruction descriptor)
 
 // Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), A and
 // B BF16 (bits 7-9, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 in
