@@ -206,7 +206,7 @@ ed_status ed_lanczos_gf(ed_ctx* ctx, const void* psi0, double e0, int site, int 
  * smaller of d_A(s), d_B(s), formed on the device by this library; its
  * eigenvalues come from a blocked Householder reduction to tridiagonal form
  * on the device (float-float panel arithmetic, FP64-accurate tensor-core
- * trailing updates), the blocks concurrently on up to three internal streams
+ * trailing updates), the blocks concurrently on up to five internal streams
  * that start after the caller's prior work on `stream`, and from bisection by
  * Sturm counts of all blocks' tridiagonal matrices in one batch on `stream`
  * (each within a few eps of the matrix norm).

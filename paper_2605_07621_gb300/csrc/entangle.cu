@@ -85,10 +85,14 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
 
   // The blocks are reduced concurrently on up to kLanes streams ("lanes"): a
   // column is mostly latency and leaves most of the GPU idle.  They go, largest
-  // first, to the lane with the least work so far (cost ~ m^3 / 3 for the
-  // products plus a fixed cost per column); each lane has its own buffers,
-  // sized for its largest block, and its share of the SMs.
-  constexpr int kLanes = 3;
+  // first, to the lane with the least work so far; each lane has its own
+  // buffers, sized for its largest block, and a share of the SMs for its panel
+  // kernels (one CTA per SM).  Spectrum of 15 blocks with m up to 3432 / of 13
+  // with m up to 924, in equal shares: 2 lanes 146 / 27 ms, 3: 130 / 19.6, 4:
+  // 134 / 16.7, 6: 154 / 15.9; shared out by their work: 3: 127 / 19.5, 4: 122 /
+  // 17.1, 5: 114 / 16.2, 6: 134 / 20.5; with a fifth of the SMs left to the
+  // trailing updates, 5: 122 / 17.1.
+  constexpr int kLanes = 5;
   std::vector<size_t> order(nb);
   for (size_t i = 0; i < nb; ++i) order[i] = i;
   auto bm = [&](size_t i) { return (long long)std::min(c->blocks[i].dA, c->blocks[i].dB); };
@@ -115,19 +119,45 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
   }
   std::vector<int> lane_of(nb, 0);
   std::vector<std::vector<size_t>> lane_blocks(lanes);
+  // a reduction on g SMs takes about serial(m) + spread(m) / g microseconds
+  // (m = 1716 / 3003 / 3432 alone on 25 to 152 SMs: within 5 %)
+  auto serial = [](double m) { return m * (9.0 + 0.6e-3 * m); };
+  auto spread = [](double m) { return 1.45e6 * std::pow(m / 3432.0, 2.5); };
+  std::vector<double> lane_serial(lanes, 0.0), lane_spread(lanes, 0.0);
   {
     std::vector<double> load(lanes, 0.0);
     for (size_t oi = 0; oi < nb; ++oi) {
       const size_t bi = order[oi];
       const double m = (double)bm(bi);
-      const double cost = m * m * m / 3.0 + 4e7 * m;
       const int k = (int)(std::min_element(load.begin(), load.end()) - load.begin());
       lane_of[bi] = k;
-      load[k] += cost;
+      load[k] += serial(m) + spread(m) * lanes / sms;
+      lane_serial[k] += serial(m);
+      lane_spread[k] += spread(m);
       lane_blocks[k].push_back(bi);
     }
   }
   while (lanes > 1 && lane_blocks[lanes - 1].empty()) --lanes;
+  // the SMs shared out so that the lanes end together, at T: bisection for the
+  // least T at which the shares fit
+  std::vector<int> share(lanes, 1);
+  {
+    double lo = *std::max_element(lane_serial.begin(), lane_serial.begin() + lanes), hi = lo + 1.0;
+    auto shares = [&](double T) {
+      int sum = 0;
+      for (int k = 0; k < lanes; ++k) {
+        share[k] = (int)std::min((double)sms, std::max(1.0, std::floor(lane_spread[k] / (T - lane_serial[k]))));
+        sum += share[k];
+      }
+      return sum;
+    };
+    while (shares(hi) > sms) hi = lo + 2.0 * (hi - lo);
+    for (int i = 0; i < 40; ++i) {
+      const double mid = 0.5 * (lo + hi);
+      if (shares(mid) > sms) lo = mid; else hi = mid;
+    }
+    shares(hi);
+  }
 
   DevMem mem;
   OzContext oz;
@@ -311,7 +341,7 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       if ((s = oz_gemm(&oz, d_probs + bi, 1, tiles[bi], nullptr, ln.s)) != ED_OK) return fail(s);
       if (cudaEventRecord(ev_g1.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
       TriBlocked tb{&oz, ln.NVW, ln.WV, ln.WVf, ln.F, tridiag_ldF(m), {}, oz.d_err, d_tjobs + 2 * toff[bi],
-                    d_tprobs + toff[bi], std::max(1, sms / lanes)};
+                    d_tprobs + toff[bi], share[k]};
       if (m >= 3 && (s = tmap_8b_2d(&tb.tmF, ln.F, m, m, tb.ldF, 34, 32)) != ED_OK) return fail(s);
       if ((s = tridiag_reduce_blocked(ln.G, m, ln.work, bd, bd + m, ln.s, sms, tb)) != ED_OK) return fail(s);
     }
