@@ -274,6 +274,10 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
       return dot_dev<T>(c, w, w, n, slot(c, 1), st, 1);
     }
   };
+  // small sectors without orthogonalisation: the step after H|psi> is one
+  // launch (in tail), except for the last step, which has no next vector
+  const bool small = !reorth && !pro && lz_step_fits(c, n);
+  auto one_launch = [&](int j) { return small && j + 1 < max_iter; };
   // one step up to its history entry (apply, alpha, beta, orthogonalisation)
   auto head = [&](int j, bool& ortho_now) -> ed_status {
     ortho_now = false;
@@ -285,6 +289,7 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     } else {
       ED_TRY(apply_H_impl(c, v, w, dtype_of<T>(), st));
     }
+    if (one_launch(j)) return ED_OK;
     launch_lz_a<T>(c, w, v, vprev, j > 0 ? 1 : 0, n, st);
     // lz_b writes the history entry itself unless an orthogonalisation follows
     const bool full = reorth && basis && basis->kind == BASIS_SAME && basis->complete && basis->count <= kMaxBasis;
@@ -314,11 +319,15 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
   // its rows are 16-byte aligned, as H|psi> wants its input), else to the
   // caller's buffer that does not hold v
   const bool in_place = basis && basis->kind == BASIS_SAME && (n * (long long)sizeof(T)) % 16 == 0;
-  auto tail = [&](bool ortho_now) {
+  auto tail = [&](int j, bool ortho_now) -> ed_status {
     T* out = in_place ? (T*)basis_next(basis) : nullptr;
     const bool stored = out != nullptr;
     if (!out) out = v == bufs[0] ? bufs[1] : bufs[0];
-    if constexpr (std::is_same<T, double>::value) {
+    if (one_launch(j)) {
+      const bool fix = fuse && c->d_fixed;
+      ED_TRY(launch_lz_step<T>(c, w, v, vprev, out, j > 0 ? 1 : 0, n, fix, hist, hcount, st));
+      prepared = fix;
+    } else if constexpr (std::is_same<T, double>::value) {
       // (after an orthogonalisation the exponent lz_b recorded may be stale)
       if (fuse && c->d_fixed && !ortho_now) {
         launch_lz_c_fixed(c, w, out, c->d_fixed, ew, c->d_exp, n, st);
@@ -334,13 +343,21 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     v = out;
     if (stored) basis_plane<T>(c, basis, v, n, st);
     else if (!in_place) basis_store<T>(c, basis, v, n, st);
+    return ED_OK;
   };
   // read the scalars of the steps since the last read and examine them in order
   auto examine = [&](int m) -> ed_status {
     hbuf.resize((size_t)(m - read) * 2);
     ED_CUDA_TRY(cudaMemcpyAsync(hbuf.data(), hist + 2 * read, hbuf.size() * sizeof(double), cudaMemcpyDeviceToHost,
                                 st));
+    int late = 0;
+    if (small) ED_CUDA_TRY(cudaMemcpyAsync(&late, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     ED_CUDA_TRY(cudaStreamSynchronize(st));
+    if (late) {
+      ED_CUDA_TRY(cudaMemsetAsync(c->d_err, 0, 8 * sizeof(int), st));
+      set_error("a Lanczos step's wait for its CTAs ran out");
+      return ED_ETIMEOUT;
+    }
     for (int k = read; k < m && !done; ++k) {
       const double a = hbuf[2 * (k - read)], b = hbuf[2 * (k - read) + 1];
       out.alpha.push_back(a);
@@ -415,7 +432,7 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
           for (int q = 0; q < 2 && es == ED_OK; ++q) {
             bool on = false;
             es = head(j + q, on);
-            if (es == ED_OK) tail(on);
+            if (es == ED_OK) es = tail(j + q, on);
           }
           ok = cudaStreamEndCapture(ps, &graph) == cudaSuccess && es == ED_OK &&
                cudaGraphInstantiate(&gexec, graph, 0) == cudaSuccess;
@@ -442,8 +459,8 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     } else {
       bool on = false;
       ED_TRY(head(j, on));
+      if (j + 1 < max_iter) ED_TRY(tail(j, on));
       ++j;
-      if (j < max_iter) tail(on);
     }
     if (j - read >= every || j == max_iter) ED_TRY(examine(j));
   }

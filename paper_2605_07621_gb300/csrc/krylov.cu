@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 
 #include <chrono>
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -168,6 +170,184 @@ __global__ void k_lz_c(const T* __restrict__ w, T* __restrict__ out, const doubl
   const T inv = (T)(b > 0.0 ? 1.0 / b : 0.0);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = w[i] * inv;
+}
+
+// The three updates of a step in one launch, for vectors that the grid holds in
+// registers (E elements per thread): w - beta vprev and alpha, then w - alpha v
+// and the next beta, then out = w / beta (FIX: and the fixed-point copy, as
+// k_lz_c_fixed); w itself is not written.  The CTAs meet at each of the two sums:
+//  * CL: one cluster of 8 or 16 CTAs, which read one another's partial sums
+//    from shared memory;
+//  * else a cooperative grid of at most one CTA per SM: the last CTA to arrive
+//    sums the partial results, clears the ticket bar[0] and lets the others go
+//    by a new generation bar[1].
+// Bound: latency.  150 steps against k_lz_a, k_lz_b and k_lz_c as three
+// dependent launches, one cluster: 400 states 3.05 -> 2.61 ms, 12,870 (J1-J2)
+// 3.90 -> 3.58, 15,876 3.33 -> 3.07, 30,240 3.31 -> 3.24 (beyond, FP64
+// arithmetic on 16 SMs takes longer than the launches: 44,100 states no gain,
+// 63,504 at 16 elements per thread 3.76 -> 4.58); cooperative: 184,756 6.15 ->
+// 5.74, 213,444 5.53 -> 4.71, 853,776 8.70 -> 7.46 (a cooperative launch does
+// not overlap the one before: 12,870 3.47 -> 4.01, 63,504 3.76 -> 3.99).
+constexpr int kStepThreads = 512, kStepMaxE = 16, kStepCl = 16, kStepClE = 4;
+constexpr long long kStepGridMin = 1 << 17;
+constexpr long long kStepSpin = 1ll << 22;  // polls of a barrier (seconds) before the kernel gives up
+
+template <typename T, int E, bool FIX, bool CL>
+__global__ void __launch_bounds__(kStepThreads, 1)
+    k_lz_step(const T* __restrict__ w, const T* __restrict__ v, const T* __restrict__ vprev, T* __restrict__ out,
+              int use_beta, long long n, double* part, double* alpha, double* beta, double* hist, int* hcount,
+              int* epart, int* ex, long long* __restrict__ X, int P, unsigned* bar, int* err) {
+  __shared__ double s_val;
+  __shared__ int s_em, s_ok;
+  __shared__ unsigned s_last;
+  __shared__ double s_part[2];  // CL: this CTA's share of either sum, read by the others
+  __shared__ int s_epart;
+  if constexpr (CL) pdl_wait();
+  const int tid = threadIdx.x;
+  const long long step = (long long)gridDim.x * kStepThreads;
+  const T bt = use_beta ? (T)beta[0] : (T)0;
+  unsigned gen = 0;
+  if (!CL && tid == 0) gen = *(volatile unsigned*)(bar + 1);  // it moves only after this CTA has arrived
+  int phase = 0;
+  // the grid's sum of s (thread 0's) and largest em; publish: thread 0 of the last CTA
+  auto grid_sum = [&](double s, int em, auto publish) -> bool {
+    if constexpr (CL) {
+      auto cl = cooperative_groups::this_cluster();
+      if (tid == 0) {
+        s_part[phase] = s;
+        s_epart = em;
+      }
+      cl.sync();
+      if (tid == 0) {
+        double t = 0.0;
+        int m = 0;
+#pragma unroll 8
+        for (int r = 0; r < (int)gridDim.x; ++r) {
+          t += *cl.map_shared_rank(&s_part[phase], r);
+          if constexpr (FIX) m = max(m, *cl.map_shared_rank(&s_epart, r));
+        }
+        publish(t, m);
+      }
+      ++phase;
+      __syncthreads();
+      return true;
+    }
+    if (tid == 0) {
+      part[blockIdx.x] = s;
+      if constexpr (FIX) epart[blockIdx.x] = em;
+      __threadfence();
+      s_last = atomicAdd(bar, 1u) == gridDim.x - 1 ? 1u : 0u;
+      s_ok = 1;
+      s_em = 0;
+    }
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      if constexpr (FIX) {
+        int m = 0;
+        for (int i = tid; i < (int)gridDim.x; i += kStepThreads) m = max(m, __ldcg(epart + i));
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((tid & 31) == 0) atomicMax(&s_em, m);
+      }
+      const double t = sum_parts(part);  // (synchronises the CTA)
+      if (tid == 0) {
+        publish(t, s_em);
+        bar[0] = 0u;
+        __threadfence();
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(bar + 1), "r"(gen + 1u) : "memory");
+      }
+    } else if (tid == 0) {
+      unsigned g = gen;
+      for (long long i = 0; i < kStepSpin && g == gen; ++i)
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(bar + 1) : "memory");
+      if (g == gen) {
+        atomicExch(err, 1);
+        s_ok = 0;
+      }
+    }
+    ++gen;
+    __syncthreads();
+    return s_ok != 0;
+  };
+  T wr[E], vr[E];
+  DotAcc<T> acc;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const long long i = (long long)blockIdx.x * kStepThreads + tid + e * step;
+    wr[e] = i < n ? w[i] : (T)0;
+    vr[e] = i < n ? v[i] : (T)0;
+    if (use_beta && i < n) wr[e] -= bt * vprev[i];
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e) acc.add_prod(vr[e], wr[e]);
+  // (CL: thread 0 of every CTA has the sum; the first CTA's stores it)
+  if (!grid_sum(block_sum(acc.value()), 0, [&](double t, int) {
+        if (!CL || blockIdx.x == 0) alpha[0] = t;
+        s_val = t;
+      }))
+    return;
+  if constexpr (!CL) {
+    if (tid == 0) s_val = __ldcg(alpha);
+    __syncthreads();
+  }
+  const double s_alpha = s_val;
+  const T al = (T)s_alpha;
+  DotAcc<T> nrm;
+  int em = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    wr[e] = wr[e] - al * vr[e];
+    nrm.add_prod(wr[e], wr[e]);
+    if constexpr (FIX) em = max(em, (int)(((unsigned long long)__double_as_longlong(wr[e]) >> 52) & 0x7ffull));
+  }
+  if constexpr (FIX) {
+    if (tid == 0) s_em = 0;
+    __syncthreads();
+    em = __reduce_max_sync(0xffffffffu, em);
+    if ((tid & 31) == 0) atomicMax(&s_em, em);
+    __syncthreads();
+    em = s_em;
+  }
+  const bool ok = grid_sum(block_sum(nrm.value()), em, [&](double t, int m) {
+    const double b = sqrt(t > 0.0 ? t : 0.0);
+    // |out| < 2^E, see k_lz_c_fixed
+    const int eb = (int)(((unsigned long long)__double_as_longlong(b) >> 52) & 0x7ffull);
+    const int xe = (m - 1022) - (eb - 1022) + 1 + 1022;
+    if (!CL || blockIdx.x == 0) {
+      beta[0] = b;
+      if (hist) {
+        const int j = *hcount;
+        hist[2 * j] = CL ? (double)s_alpha : alpha[0];
+        hist[2 * j + 1] = b;
+        *hcount = j + 1;
+      }
+      if constexpr (FIX) ex[0] = xe;
+    }
+    s_val = b;
+    s_em = xe;
+  });
+  if (!ok) return;
+  if constexpr (CL) {
+    cooperative_groups::this_cluster().sync();  // no CTA leaves while another reads its sums
+  } else {
+    if (tid == 0) {
+      s_val = __ldcg(beta);
+      if constexpr (FIX) s_em = __ldcg(ex);
+    }
+    __syncthreads();
+  }
+  const double b = s_val;
+  const T inv = (T)(b > 0.0 ? 1.0 / b : 0.0);
+  const int sh = FIX ? P - (s_em - 1022) : 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const long long i = (long long)blockIdx.x * kStepThreads + tid + e * step;
+    if (i < n) {
+      const T o = wr[e] * inv;
+      out[i] = o;
+      if constexpr (FIX) X[i] = to_fixed(o, sh);
+    }
+  }
 }
 
 // y[i] = s * x[i] (types may differ); s from host
@@ -378,12 +558,16 @@ __global__ void k_basis_update(const T* __restrict__ V, long long ldv, int m, co
 
 // ---------------------------------------------------------------- host helpers
 
-int grid_for(const ed_ctx* c, long long n) {
+static int sm_count(const ed_ctx* c) {
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
     cudaGetLastError();
     sms = 148;
   }
+  return sms;
+}
+int grid_for(const ed_ctx* c, long long n) {
+  const int sms = sm_count(c);
   long long g = (n + kRedThreads - 1) / kRedThreads;
   long long cap = (long long)sms * 8;
   if (g > cap) g = cap;
@@ -541,6 +725,53 @@ void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, int* ew, double* hist
   launch_pdl(k_lz_b<T, false>, g, kRedThreads, 0, st, w, v, alpha, n, c->d_partials, beta, ctr, hist, hcount,
              (int*)nullptr, (int*)nullptr);
 }
+static bool step_cluster(long long n) { return n <= (long long)kStepCl * kStepThreads * kStepClE; }
+bool lz_step_fits(const ed_ctx* c, long long n) {
+  return step_cluster(n) || (n >= kStepGridMin && n <= (long long)sm_count(c) * kStepThreads * kStepMaxE);
+}
+template <typename T, bool FIX>
+static ed_status go_lz_step(ed_ctx* c, const T* w, const T* v, const T* vprev, T* out, int use_beta, long long n,
+                            double* hist, int* hcount, cudaStream_t st) {
+  const bool cl = step_cluster(n);
+  // a cluster of eight while two elements per thread are enough
+  const int g = cl ? (n <= kStepThreads * kStepCl ? kStepCl / 2 : kStepCl) : (int)std::min<long long>(sm_count(c), (n + kStepThreads - 1) / kStepThreads);
+  const long long e = (n + (long long)g * kStepThreads - 1) / ((long long)g * kStepThreads);
+  auto kern = cl ? (e <= 1   ? k_lz_step<T, 1, FIX, true>
+                    : e <= 2 ? k_lz_step<T, 2, FIX, true>
+                             : k_lz_step<T, kStepClE, FIX, true>)
+                 : (e <= 4 ? k_lz_step<T, 4, FIX, false> : k_lz_step<T, kStepMaxE, FIX, false>);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)g);
+  cfg.blockDim = dim3(kStepThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  if (cl) {
+    // (16 CTAs in a cluster: an opt-in, the same on every call)
+    ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)g;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;  // the CTAs wait for one another
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = cl ? 2 : 1;
+  ED_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, w, v, vprev, out, use_beta, n, c->d_partials, slot(c, 0), slot(c, 1), hist,
+                                 hcount, FIX ? c->d_exp + 16 : (int*)nullptr, FIX ? c->d_exp : (int*)nullptr,
+                                 FIX ? c->d_fixed : (long long*)nullptr, FIX ? c->t3.P : 0, (unsigned*)c->d_err + 4,
+                                 c->d_err));
+  return ED_OK;
+}
+template <typename T>
+ed_status launch_lz_step(ed_ctx* c, const T* w, const T* v, const T* vprev, T* out, int use_beta, long long n,
+                         bool fix, double* hist, int* hcount, cudaStream_t st) {
+  if constexpr (std::is_same<T, double>::value)
+    if (fix) return go_lz_step<double, true>(c, w, v, vprev, out, use_beta, n, hist, hcount, st);
+  return go_lz_step<T, false>(c, w, v, vprev, out, use_beta, n, hist, hcount, st);
+}
 template <typename T>
 void launch_lz_c(ed_ctx* c, const T* w, T* out, long long n, cudaStream_t st) {
   launch_pdl(k_lz_c<T>, grid_for(c, n), kRedThreads, 0, st, w, out, slot(c, 1), n);
@@ -622,6 +853,7 @@ void launch_fermion_remap(ed_ctx* c, const double* psi, long long dA_src, long l
   template void launch_lz_a<T>(ed_ctx*, T*, const T*, const T*, int, long long, cudaStream_t);          \
   template void launch_lz_b<T>(ed_ctx*, T*, const T*, long long, int*, double*, int*, cudaStream_t);    \
   template void launch_lz_c<T>(ed_ctx*, const T*, T*, long long, cudaStream_t);                        \
+  template ed_status launch_lz_step<T>(ed_ctx*, const T*, const T*, const T*, T*, int, long long, bool, double*, int*, cudaStream_t); \
   template void launch_lz_rerun<T>(ed_ctx*, const T*, const T*, const T*, double, double, double, T*,   \
                                    long long, cudaStream_t);                                            \
   template void launch_axpy_dev<T>(ed_ctx*, const T*, T*, const double*, double, long long, cudaStream_t);

@@ -33,6 +33,12 @@ template <typename T>
 void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, int* ew, double* hist, int* hcount, cudaStream_t st);
 template <typename T>
 void launch_lz_c(ed_ctx* c, const T* w, T* out, long long n, cudaStream_t st);
+// lz_a, lz_b and lz_c (fix: lz_c_fixed) in one launch, where the vectors fit the
+// registers of one grid; w is only read
+bool lz_step_fits(const ed_ctx* c, long long n);
+template <typename T>
+ed_status launch_lz_step(ed_ctx* c, const T* w, const T* v, const T* vprev, T* out, int use_beta, long long n,
+                         bool fix, double* hist, int* hcount, cudaStream_t st);
 // FP64 Lanczos steps that hand the next H|psi> its fixed-point input:
 // lz_b (ew not NULL) also records the largest exponent of w; lz_c also writes the
 // fixed-point copy X of w / beta and its scale (biased exponent) to *ex
