@@ -218,7 +218,8 @@ struct BdTile {
 // 538 / 542 with three stages (64-wide), N up to 192 and no prefetch into L2,
 // which moved every operand twice through L2's ports; 506 / 545 with the list
 // warp; 449 / 462 without Psi^T (slicing 114 -> 59 us, 0.2 GB less from HBM);
-// 439 / 451 with the launches overlapped.  Tried and slower: barriers per piece
+// 439 / 451 with the launches overlapped; 432 / 448 without 64-bit divisions and
+// with ready descriptors in the issuing thread.  Tried and slower: barriers per piece
 // instead of per K step (608 / 549), operands prefetched once per row or column
 // of tiles (531 / 560).
 template <int BN>
@@ -331,17 +332,17 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
   } else if (warp == kBdWarpTma) {
     // ---- TMA producer: per K step the three pieces of the A tile and of the B tile
     if (lane == 0) {
-      long long it = 0;
+      int s = 0;  // the stage, and the parity of its phase
+      unsigned ph = 0;
       for (int tl = 0; !s_abort; ++tl) {
         const BdTile* T = tile_at(tl);
         if (!T) break;
         const int m0 = T->m0, n0 = T->n0, nk = T->nk;
         const CUtensorMap* mp = g.maps + (long long)T->slot * kBMaps;
         const CUtensorMap* mHB = mp + (BN == 64 ? kMapHB64 : kMapHB128);
-        for (int ks = 0; ks < nk; ++ks, ++it) {
-          const int s = (int)(it % C::kStages);
-          const long long u = it / C::kStages;
-          if (u > 0 && !tc::mbar_wait(&empty[s], (unsigned)((u - 1) & 1), kBdSpin)) {
+        for (int ks = 0; ks < nk; ++ks) {
+          // (a fresh barrier passes the wait for the phase before its first)
+          if (!tc::mbar_wait(&empty[s], ph ^ 1u, kBdSpin)) {
             s_abort = 1;
             break;
           }
@@ -361,6 +362,10 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
 #pragma unroll
             for (int q = 0; q < kBdPieces; ++q) tc::tma_load_3d(sb + q * C::kBTile, mHB, kc, n0, q, &full[s]);
           }
+          if (++s == C::kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
         tc::mbar_arrive(&ti_empty[tl % kBdTiles]);
       }
@@ -369,7 +374,12 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
   } else if (warp == kBdWarpMma) {
     // ---- MMA issuer: piece pairs p + q <= 2 into the tile's accumulators
     if (lane == 0) {
-      long long it = 0;
+      // descriptors of the first stage: A, and B as rows of Psi or of H_B
+      const uint64_t dA = tc::sdesc_kmajor_sw128(sm);
+      const uint64_t dX = tc::sdesc_mnmajor_sw128(sm + kBdPieces * C::kATile, kBdXTile);
+      const uint64_t dH = tc::sdesc_kmajor_sw128(sm + kBdPieces * C::kATile);
+      int s = 0;  // the stage, and the parity of its phase
+      unsigned ph = 0;
       for (int tl = 0; !s_abort; ++tl) {
         const BdTile* T = tile_at(tl);
         if (!T) break;
@@ -382,24 +392,20 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
         }
         tc::tc_fence_after();
         const unsigned dt = tmem + (unsigned)(C::kAcc * buf * BN);
-        for (int ks = 0; ks < nk; ++ks, ++it) {
-          const int s = (int)(it % C::kStages);
-          if (!tc::mbar_wait(&full[s], (unsigned)((it / C::kStages) & 1), kBdSpin)) {
+        for (int ks = 0; ks < nk; ++ks) {
+          if (!tc::mbar_wait(&full[s], ph, kBdSpin)) {
             s_abort = 1;
             break;
           }
           tc::tc_fence_after();
-          unsigned char* sa = sm + s * C::kStage;
-          unsigned char* sb = sa + kBdPieces * C::kATile;
           // B's pieces lie behind one another in shared memory and the
           // accumulators in TMEM, so one instruction of N = np BN takes np
           // pairs (p, q), (p, q + 1), ... whose accumulators differ
           const bool first = ks < nA;
           auto pairs = [&](int p, int q, int np, int acc) {
             const unsigned idesc = tc::idesc_bf16_f32(kBdBM, np * BN) | (first ? tc::kIdescBMnMajor : 0u);
-            const uint64_t da = tc::sdesc_kmajor_sw128(sa + p * C::kATile);
-            const unsigned char* b = sb + q * C::kBTile;
-            const uint64_t db = first ? tc::sdesc_mnmajor_sw128(b, kBdXTile) : tc::sdesc_kmajor_sw128(b);
+            const uint64_t da = dA + (unsigned)((s * C::kStage + p * C::kATile) / 16);
+            const uint64_t db = (first ? dX : dH) + (unsigned)((s * C::kStage + q * C::kBTile) / 16);
             // 16 of K per instruction: 32 bytes along a K-major row, 16 rows of Psi
             const int kb = first ? 16 * 128 / 16 : 2;
 #pragma unroll
@@ -419,6 +425,10 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
             pairs(2, 0, 1, 1);
           }
           tc::mma_commit(&empty[s]);
+          if (++s == C::kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
         if (s_abort) break;
         tc::mma_commit(&acc_full[buf]);

@@ -399,14 +399,16 @@ __device__ inline int find_prob(const OzProblem* probs, int n, long long tile) {
   return lo;
 }
 
-// One output tile per CTA.  Bound: the tensor pipe waits for its operands and
-// for the drain of the accumulators (active 50 % of the time on the 572 tiles
-// of the dense-block Y stage, 54 % on its 1,644 T tiles; one K step moves 192 KB
-// from L2 for 38 MFLOP).  Dense-block H|psi> (alpha = 0.95, 4,003 states of bond
-// dimension): 5.28 ms with N = 64 instructions and three A stages, 3.72 with N
-// = 256 and six, 2.67 with chains (one launch for all blocks of Y, C written
-// once), eight epilogue warps and column slicing split over rows; the digit
-// products alone would take 1.43 ms at the burst BF16 rate.
+// One output tile per CTA.  Bound: the tensor pipe waits for the issuing thread,
+// its operands and the drain of the accumulators (one K step moves 192 KB from
+// L2 for 38 MFLOP; with the TMA writes shared memory could feed it 88 % of the
+// time).  Dense-block H|psi> (alpha = 0.95, 4,003 states of bond dimension): 5.28
+// ms with N = 64 instructions and three A stages, 3.72 with N = 256 and six,
+// 2.67 with chains (one launch for all blocks of Y, C written once), eight
+// epilogue warps and column slicing split over rows, 2.30 with the issuing
+// thread's arithmetic reduced; the digit products alone would take 1.43 ms at
+// the burst BF16 rate.  No gain: B's planes loaded by a thread of their own (2.30),
+// A's planes awaited in pairs (2.26, but 2.93 against 2.91 at alpha = 1.11).
 __global__ void __launch_bounds__(kOzThreads, 1)
     k_oz_gemm(const OzProblem* __restrict__ probs, int nprob, const CUtensorMap* __restrict__ maps, double* y,
               int* err) {
@@ -470,7 +472,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   if (warp == kOzEpi) {
     // ---- TMA producer: per K step the 8 digit planes of B^T, then A's planes one by one
     if (lane == 0) {
-      long long na = 0, kg = 0;  // A planes, K steps over all parts
+      long long kg = 0;  // K steps over all parts
+      int s = 0;         // A's stage, and the parity of its phase
+      unsigned ph = 1;
       for (int pt = 0; pt < nparts; ++pt) {
         const CUtensorMap* ma = maps + parts[pt].mapA;
         const CUtensorMap* mb = maps + parts[pt].mapB;
@@ -482,12 +486,15 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           tc::mbar_expect_tx(&b_full[b], kOzBBuf);
           for (int q = 0; q < kOzDigits; ++q)
             tc::tma_load_3d(sB + b * kOzBBuf + q * kOzBTile, mb, kb * kOzBK, n0, q, &b_full[b]);
-          for (int p = 0; p < kOzDigits; ++p, ++na) {
-            const int s = (int)(na % kOzAStages);
-            const long long ua = na / kOzAStages;
-            if (ua > 0 && !tc::mbar_wait(&a_empty[s], (unsigned)((ua - 1) & 1), kOzSpin)) { s_abort = 1; break; }
+          for (int p = 0; p < kOzDigits; ++p) {
+            // (a fresh barrier passes the wait for the phase before its first)
+            if (!tc::mbar_wait(&a_empty[s], ph, kOzSpin)) { s_abort = 1; break; }
             tc::mbar_expect_tx(&a_full[s], kOzATile);
             tc::tma_load_3d(sA + s * kOzATile, ma, kb * kOzBK, m0, p, &a_full[s]);
+            if (++s == kOzAStages) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
         }
       }
@@ -496,8 +503,15 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   } else if (warp == kOzEpi + 1) {
     // ---- MMA issuer: accumulator g (TMEM columns 64 g) sums the digit pairs p + q = g
     if (lane == 0) {
-      long long na = 0, kg = 0;
+      long long kg = 0;
       int cg = 0;  // chunks over all parts
+      int s = 0;   // A's stage, and the parity of its phase
+      unsigned ph = 0;
+      // (one thread issues 48 instructions per K step, so its own arithmetic
+      // counts: with the stage and phase from 64-bit divisions, the planes' loop
+      // not unrolled and every descriptor made anew the dense-block H|psi> took
+      // 2.67 instead of 2.30 ms)
+      const uint64_t dA = tc::sdesc_kmajor_sw128(sA), dB = tc::sdesc_kmajor_sw128(sB);
       for (int pt = 0; pt < nparts; ++pt) {
         const int nkb = (parts[pt].K + kOzBK - 1) / kOzBK;
         const int nchunk = (nkb + kb_per_chunk - 1) / kb_per_chunk;
@@ -510,26 +524,31 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             if (!tc::mbar_wait(&b_full[b], (unsigned)((kg >> 1) & 1), kOzSpin)) { s_abort = 1; break; }
             tc::tc_fence_after();
             const bool first_kb = kb == c * kb_per_chunk;
-            for (int p = 0; p < kOzDigits; ++p, ++na) {
-              const int s = (int)(na % kOzAStages);
-              if (!tc::mbar_wait(&a_full[s], (unsigned)((na / kOzAStages) & 1), kOzSpin)) { s_abort = 1; break; }
+#pragma unroll
+            for (int p = 0; p < kOzDigits; ++p) {
+              if (!tc::mbar_wait(&a_full[s], ph, kOzSpin)) { s_abort = 1; break; }
               tc::tc_fence_after();
-              const uint64_t da = tc::sdesc_kmajor_sw128(sA + s * kOzATile);
+              const uint64_t da = dA + (unsigned)(s * (kOzATile / 16));
               // the B planes q, q + 1, ... lie behind one another in shared
               // memory and their accumulators p + q, ... in TMEM, so one
               // instruction takes up to four of them (N = 256): the A plane is
               // read once per four products.  At N = 64 the operands' shared-
               // memory reads (192 bytes a cycle) bound the tensor cores to half
+#pragma unroll
               for (int q = 0; q + p < kOzDigits; q += 4) {
                 const int np = min(4, kOzDigits - p - q);
                 const unsigned idesc = tc::idesc_bf16_f32(kOzBM, kOzBN * np);
-                const uint64_t db = tc::sdesc_kmajor_sw128(sB + b * kOzBBuf + q * kOzBTile);
+                const uint64_t db = dB + (unsigned)(b * (kOzBBuf / 16) + q * (kOzBTile / 16));
                 const unsigned dt = tmem + (unsigned)((p + q) * kOzBN);
-  #pragma unroll
+#pragma unroll
                 for (int kk = 0; kk < kOzBK / 16; ++kk)  // 32 bytes of K per instruction
                   tc::mma_bf16(dt, da + 2 * kk, db + 2 * kk, idesc, !(first_kb && p == 0 && kk == 0));
               }
               tc::mma_commit(&a_empty[s]);
+              if (++s == kOzAStages) {
+                s = 0;
+                ph ^= 1u;
+              }
             }
             tc::mma_commit(&b_empty[b]);
           }
