@@ -145,10 +145,10 @@ def entanglement_section(ed, ctx):
     xi_low = [float(-np.log(l[0] / tot)) if len(l) and l[0] > 0 else None for l in es.lam]
     peak, src = bf16_peak()
     achieved = tflops / (gram_ms * 1e-3) / 1e12 if gram_ms > 0 else None
-    # the reduction's dominant traffic: every column's product reads the
-    # float-float trailing triangle (8 bytes an entry) once; over the whole
-    # stage (every kernel of it in the time) this is a lower bound of the
-    # product kernel's rate
+    # the reduction's least traffic: every column's product reads the
+    # float-float trailing triangle (8 bytes an entry) once (panels of up to
+    # 6,144 rows read the whole square, mostly from L2); over the whole stage
+    # (every kernel of it in the time) a lower bound of the product's rate
     f_bytes = 0.0
     for mb in m:
         n = np.arange(int(mb) - 3, -1, -1, dtype=np.float64) + 2.0 if mb >= 3 else np.zeros(0)  # n = m - c - 1
@@ -157,8 +157,9 @@ def entanglement_section(ed, ctx):
     stream_gbs = f_bytes / (eig_ms * 1e-3) / 1e9 if eig_ms > 0 else None
     eig_stream = {"bytes": f_bytes, "achieved": stream_gbs, "unit": "GB/s", "peak": peaks["hbm_gbs"],
                   "frac": stream_gbs / peaks["hbm_gbs"] if stream_gbs else None, "peak_source": psrc,
-                  "note": "float-float triangle bytes the per-column products read, over the whole eigenvalue "
-                          "stage's device time (panel kernels and trailing updates included)"}
+                  "note": "float-float triangle bytes the per-column products need, over the whole eigenvalue "
+                          "stage's device time (panel kernels, trailing updates and Sturm counts included; "
+                          "panels of up to 6,144 rows read twice as much, mostly from L2)"}
     return {"ground_state_s": t_gs, "e0": r.e0, "seconds": t_es, "gram_ms": gram_ms, "eigensolver_ms": eig_ms,
             "gram_fp64_equiv_tflops": 2 * macs / (gram_ms * 1e-3) / 1e12 if gram_ms > 0 else None,
             "gram_roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",

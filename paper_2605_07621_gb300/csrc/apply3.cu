@@ -134,7 +134,7 @@ __device__ __forceinline__ float ldg_if(const float* p, bool on) { return on ? _
 // Hubbard torus, 64 % with cross terms), then issue (60 %).  A 16-byte access
 // takes four wavefronts at best; the lists are ordered so that it takes 4.06
 // (order_lists).  Measured, FP64 fixed point / FP32: J1-J2 4x8 (601 M states)
-// 22.9 -> 15.6 / 14.3 -> 9.2 ms, Hubbard 4x4 (166 M states) 2.75 -> 1.63 /
+// 22.9 -> 16.4 / 14.3 -> 9.2 ms, Hubbard 4x4 (166 M states) 2.75 -> 1.63 /
 // 1.48 -> 0.92 ms, against lists of 8-byte groups per column, scattered over the
 // lanes and padded to 16 entries.  The digit-split dense products on the
 // tensor cores that could take the terms inside a group of sites would cost
