@@ -194,7 +194,7 @@ constexpr long long kStepSpin = 1ll << 22;  // polls of a barrier (seconds) befo
 
 template <typename T, int E, bool FIX, bool CL>
 __global__ void __launch_bounds__(kStepThreads, 1)
-    k_lz_step(const T* __restrict__ w, const T* __restrict__ v, const T* __restrict__ vprev, T* __restrict__ out,
+    k_lz_step(const T* __restrict__ w, const T* __restrict__ v, const T* vprev, T* out,  // (out may be vprev's buffer)
               int use_beta, long long n, double* part, double* alpha, double* beta, double* hist, int* hcount,
               int* epart, int* ex, long long* __restrict__ X, int P, unsigned* bar, int* err) {
   __shared__ double s_val;
@@ -726,15 +726,40 @@ void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, int* ew, double* hist
              (int*)nullptr, (int*)nullptr);
 }
 static bool step_cluster(long long n) { return n <= (long long)kStepCl * kStepThreads * kStepClE; }
+// the device has room for a cluster of 16 (a GPU with fewer SMs enabled may not)
+static bool cluster_runs() {
+  auto kern = k_lz_step<double, kStepClE, true, true>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kStepCl);
+  cfg.blockDim = dim3(kStepThreads);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kStepCl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int k = 0;
+  if (cudaOccupancyMaxActiveClusters(&k, kern, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return k >= 1;
+}
 bool lz_step_fits(const ed_ctx* c, long long n) {
-  return step_cluster(n) || (n >= kStepGridMin && n <= (long long)sm_count(c) * kStepThreads * kStepMaxE);
+  if (step_cluster(n)) return cluster_runs();
+  return n >= kStepGridMin && n <= (long long)sm_count(c) * kStepThreads * kStepMaxE;
 }
 template <typename T, bool FIX>
 static ed_status go_lz_step(ed_ctx* c, const T* w, const T* v, const T* vprev, T* out, int use_beta, long long n,
                             double* hist, int* hcount, cudaStream_t st) {
   const bool cl = step_cluster(n);
   // a cluster of eight while two elements per thread are enough
-  const int g = cl ? (n <= kStepThreads * kStepCl ? kStepCl / 2 : kStepCl) : (int)std::min<long long>(sm_count(c), (n + kStepThreads - 1) / kStepThreads);
+  const int g = cl ? (n <= kStepThreads * kStepCl ? kStepCl / 2 : kStepCl)
+                   : (int)std::min<long long>(sm_count(c), (n + kStepThreads - 1) / kStepThreads);
   const long long e = (n + (long long)g * kStepThreads - 1) / ((long long)g * kStepThreads);
   auto kern = cl ? (e <= 1   ? k_lz_step<T, 1, FIX, true>
                     : e <= 2 ? k_lz_step<T, 2, FIX, true>
