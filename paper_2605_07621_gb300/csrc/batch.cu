@@ -305,7 +305,7 @@ ed_status host_tables(const ed_model_desc& m, HostTables& h) {
 bool dense_capable(const HostTables& h) { return h.dA <= kBDenseMax && h.dB <= kBDenseMax; }
 
 // bytes of the CSR tables (uploaded), then of the dense form: the pieces of
-// H_A, H_B (uploaded) and of Psi, Psi^T (written by every apply)
+// H_A, H_B (built once) and of Psi (written by every apply)
 size_t csr_bytes(const HostTables& h) {
   size_t b = 0;
   b += align256(h.A_rp.size() * 4) + align256(h.A_col.size() * 4) + align256(h.A_val.size() * 4);

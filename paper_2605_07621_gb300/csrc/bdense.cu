@@ -11,9 +11,10 @@
 // piece products h_p(H) h_q(Psi) with p + q <= 2 are accumulated in FP32,
 // the dropped ones (p + q >= 3) being below 2^-24 of the leading product.
 // The leading products (p = q = 0) and the corrections (p + q = 1, 2) go into
-// two accumulators, so the rounding of the many small correction sums does
-// not fall on the large leading sum; both products of an output tile (they
-// add) share them, and the epilogue adds the two and the diagonal.
+// separate accumulators (64-wide tiles: one per order), so the rounding of the
+// many small correction sums does not fall on the large leading sum; both
+// products of an output tile (they add) share them, and the epilogue adds them
+// and the diagonal.
 //
 // Per output tile (128 rows a x BN columns b): the K steps of H_A Psi
 // (A operand: H_A's pieces, rows a, K = a' contiguous; B operand: Psi's pieces,
@@ -440,9 +441,9 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
     }
   } else {
     // ---- epilogue: warp w drains TMEM lanes 32 (w % 4) .. + 31 (tile rows)
-    // for every other 32-column chunk; each 32 x 32 chunk is transposed
-    // through shared memory so the loads of x and the stores of
-    // y = accumulators + V x run along rows (lane = column)
+    // for every other 32-column chunk; each 32 x 8 part of it goes through
+    // shared memory so the loads of x and the stores of y = accumulators + V x
+    // move whole 32-byte sectors along rows
     const int quarter = warp & 3, half = warp >> 2;
     float* tr = trans + warp * kBdTrans;
     for (int tl = 0;; ++tl) {

@@ -71,13 +71,6 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
   return pol;
 }
 
-// L2 prefetch of the box a tma_load_3d with the same map and coordinates reads
-__device__ __forceinline__ void tma_prefetch_3d(const void* tmap, int c0, int c1, int c2) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tmap), "r"(c0), "r"(c1),
-               "r"(c2)
-               : "memory");
-}
-
 // fetch of a tensor map ahead of the loads that use it
 __device__ __forceinline__ void tma_prefetch_map(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
