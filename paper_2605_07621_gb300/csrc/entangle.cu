@@ -151,7 +151,7 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       }
       return sum;
     };
-    while (shares(hi) > sms) hi = lo + 2.0 * (hi - lo);
+    for (int i = 0; i < 60 && shares(hi) > sms; ++i) hi = lo + 2.0 * (hi - lo);
     for (int i = 0; i < 40; ++i) {
       const double mid = 0.5 * (lo + hi);
       if (shares(mid) > sms) lo = mid; else hi = mid;
