@@ -381,8 +381,8 @@ ed_status oz_slice(OzContext* o, const OzSliceJob* d_jobs, int njobs, long long 
 // ---------------------------------------------------------------- the GEMM
 
 constexpr int kOzEpi = 8;                  // epilogue warps: two per 32 TMEM lanes, 32 columns each
-constexpr int kOzThreads = 32 * (kOzEpi + 2);  // then the TMA producer and the MMA issuer
-constexpr int kOzAStages = 6;
+constexpr int kOzThreads = 32 * (kOzEpi + 3);  // then the TMA producer of A, the MMA issuer, the producer of B
+constexpr int kOzAStages = 6;              // even: planes are awaited in pairs
 constexpr int kOzATile = kOzBM * kOzBK * 2;   // 16 KB
 constexpr int kOzBTile = kOzBN * kOzBK * 2;   // 8 KB
 constexpr int kOzBBuf = kOzDigits * kOzBTile; // the 8 digit planes of one K step: 64 KB
@@ -406,9 +406,10 @@ __device__ inline int find_prob(const OzProblem* probs, int n, long long tile) {
 // ms with N = 64 instructions and three A stages, 3.72 with N = 256 and six,
 // 2.67 with chains (one launch for all blocks of Y, C written once), eight
 // epilogue warps and column slicing split over rows, 2.30 with the issuing
-// thread's arithmetic reduced; the digit products alone would take 1.43 ms at
-// the burst BF16 rate.  No gain: B's planes loaded by a thread of their own (2.30),
-// A's planes awaited in pairs (2.26, but 2.93 against 2.91 at alpha = 1.11).
+// thread's arithmetic reduced, 2.26 with A's planes awaited in pairs and B loaded
+// by a thread of its own (freed in pairs as well: 2.25, but 2.92 against 2.87 at
+// alpha = 1.11); the digit products alone would take 1.43 ms at the burst BF16
+// rate.
 __global__ void __launch_bounds__(kOzThreads, 1)
     k_oz_gemm(const OzProblem* __restrict__ probs, int nprob, const CUtensorMap* __restrict__ maps, double* y,
               int* err) {
@@ -470,13 +471,33 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   const unsigned tmem = s_tmem;
 
   if (warp == kOzEpi) {
-    // ---- TMA producer: per K step the 8 digit planes of B^T, then A's planes one by one
+    // ---- TMA producer of A: the planes one by one, awaited by the issuer in pairs
     if (lane == 0) {
-      long long kg = 0;  // K steps over all parts
-      int s = 0;         // A's stage, and the parity of its phase
+      int s = 0;  // A's stage, and the parity of its phase
       unsigned ph = 1;
       for (int pt = 0; pt < nparts; ++pt) {
         const CUtensorMap* ma = maps + parts[pt].mapA;
+        const int nkb = (parts[pt].K + kOzBK - 1) / kOzBK;
+        for (int kb = 0; kb < nkb && !s_abort; ++kb) {
+          for (int p = 0; p < kOzDigits; ++p) {
+            // (a fresh barrier passes the wait for the phase before its first)
+            if (!tc::mbar_wait(&a_empty[s], ph, kOzSpin)) { s_abort = 1; break; }
+            if (!(s & 1)) tc::mbar_expect_tx(&a_full[s], 2 * kOzATile);
+            tc::tma_load_3d(sA + s * kOzATile, ma, kb * kOzBK, m0, p, &a_full[s & ~1]);
+            if (++s == kOzAStages) {
+              s = 0;
+              ph ^= 1u;
+            }
+          }
+        }
+      }
+      if (s_abort) atomicExch(err, 1);
+    }
+  } else if (warp == kOzEpi + 2) {
+    // ---- TMA producer of B: the 8 digit planes of B^T of a K step
+    if (lane == 0) {
+      long long kg = 0;  // K steps over all parts
+      for (int pt = 0; pt < nparts; ++pt) {
         const CUtensorMap* mb = maps + parts[pt].mapB;
         const int nkb = (parts[pt].K + kOzBK - 1) / kOzBK;
         for (int kb = 0; kb < nkb && !s_abort; ++kb, ++kg) {
@@ -486,16 +507,6 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           tc::mbar_expect_tx(&b_full[b], kOzBBuf);
           for (int q = 0; q < kOzDigits; ++q)
             tc::tma_load_3d(sB + b * kOzBBuf + q * kOzBTile, mb, kb * kOzBK, n0, q, &b_full[b]);
-          for (int p = 0; p < kOzDigits; ++p) {
-            // (a fresh barrier passes the wait for the phase before its first)
-            if (!tc::mbar_wait(&a_empty[s], ph, kOzSpin)) { s_abort = 1; break; }
-            tc::mbar_expect_tx(&a_full[s], kOzATile);
-            tc::tma_load_3d(sA + s * kOzATile, ma, kb * kOzBK, m0, p, &a_full[s]);
-            if (++s == kOzAStages) {
-              s = 0;
-              ph ^= 1u;
-            }
-          }
         }
       }
       if (s_abort) atomicExch(err, 1);
@@ -526,7 +537,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             const bool first_kb = kb == c * kb_per_chunk;
 #pragma unroll
             for (int p = 0; p < kOzDigits; ++p) {
-              if (!tc::mbar_wait(&a_full[s], ph, kOzSpin)) { s_abort = 1; break; }
+              if (!(p & 1) && !tc::mbar_wait(&a_full[s], ph, kOzSpin)) { s_abort = 1; break; }
               tc::tc_fence_after();
               const uint64_t da = dA + (unsigned)(s * (kOzATile / 16));
               // the B planes q, q + 1, ... lie behind one another in shared
