@@ -125,7 +125,7 @@ class BatchEngine {
   // apply over them, cache the choice per shape
   ed_status tune(const std::vector<int>& slots);
   // the cached choice for the instance's shape, else the dense form with
-  // 64-wide tiles when d_B <= 64, 128-wide otherwise
+  // 64-wide tiles
   int default_mode(const BSlot& S) const;
   // device time (ms) of one H psi over all active instances (Lanczos vectors)
   ed_status time_apply(int reps, float* ms);

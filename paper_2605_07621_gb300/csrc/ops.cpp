@@ -506,12 +506,19 @@ static ed_status build_v3(ed_ctx* c, const HostSideOps& ha, const HostSideOps& h
   for (size_t i = 0; i < mb.size(); ++i) mb[i] = hb.maps[i] < 0 ? 0xFFFF : (uint16_t)hb.maps[i];
   ED_TRY(upload(c, &mA, ma));
   ED_TRY(upload(c, &mB, mb));
-  uint2* Bsl;
   unsigned* Bpr;
-  ED_TRY(upload(c, &Bsl, b3.slab));
   ED_TRY(upload(c, &Bpr, b3.pair));
-  t.B_slab = Bsl;
   t.B_pair = Bpr;
+  // the small tables of the row pass in one allocation (16-byte aligned parts)
+  std::vector<uint4> pk;
+  auto part = [&](const void* src, size_t bytes) {
+    const size_t at = pk.size();
+    pk.resize(at + (bytes + 15) / 16, uint4{0, 0, 0, 0});
+    if (bytes) std::memcpy(pk.data() + at, src, bytes);
+    return at;
+  };
+  const size_t at_slab = part(b3.slab.data(), b3.slab.size() * sizeof(uint2));
+  size_t at_ax = 0, at_bx = 0, at_xm = 0;
   if (t.xs_ok && t.n_oct > 0) {
     const int64_t tA = c->A.total(), tB = c->B.total();
     std::vector<unsigned> ax(t.n_oct * tA, 0u), bx(t.n_oct * tB, 0u);
@@ -525,16 +532,19 @@ static ed_status build_v3(ed_ctx* c, const HostSideOps& ha, const HostSideOps& h
     }
     for (size_t v = 0; v < xs_site.size(); ++v)
       for (int64_t g = 0; g < tB; ++g) xm[((v / 8) * tB + g) * 8 + v % 8] = mb[(size_t)xs_site[v] * tB + g];
-    std::vector<uint4> xm4(xm.size() / 8);
-    std::memcpy(xm4.data(), xm.data(), xm.size() * sizeof(uint16_t));
-    unsigned *axd, *bxd;
-    uint4* xmd;
-    ED_TRY(upload(c, &axd, ax));
-    ED_TRY(upload(c, &bxd, bx));
-    ED_TRY(upload(c, &xmd, xm4));
-    t.A_xs = axd;
-    t.B_xs = bxd;
-    t.B_xmap = xmd;
+    at_ax = part(ax.data(), ax.size() * sizeof(unsigned));
+    at_bx = part(bx.data(), bx.size() * sizeof(unsigned));
+    at_xm = part(xm.data(), xm.size() * sizeof(uint16_t));
+  }
+  {
+    uint4* d;
+    ED_TRY(upload(c, &d, pk));
+    t.B_slab = reinterpret_cast<const uint2*>(d + at_slab);
+    if (t.xs_ok && t.n_oct > 0) {
+      t.A_xs = reinterpret_cast<const unsigned*>(d + at_ax);
+      t.B_xs = reinterpret_cast<const unsigned*>(d + at_bx);
+      t.B_xmap = d + at_xm;
+    }
   }
   t.A_meta = Am; t.A_col = Ac; t.A_pack = Ap; t.B_pack = Bp;
   t.A_dI = AdI; t.B_dI = BdI; t.A_dW = AdWd; t.B_dW = BdWd; t.mapA = mA; t.mapB = mB;
