@@ -209,7 +209,8 @@ ed_status ed_lanczos_gf(ed_ctx* ctx, const void* psi0, double e0, int site, int 
  * trailing updates), the blocks concurrently on up to five internal streams
  * that start after the caller's prior work on `stream`, and from bisection by
  * Sturm counts of all blocks' tridiagonal matrices in one batch on `stream`
- * (each within a few eps of the matrix norm).
+ * (each within a few eps of the norm of the unreduced part of the tridiagonal
+ * matrix that it belongs to; a block of zeros gives exact zeros).
  *   psi      device FP64 vector of ctx (not normalised by the call)
  *   lambda   host, capacity cap: for every block in ed_blocks order, its
  *            min(d_A, d_B) eigenvalues in descending order (rounding can

@@ -54,12 +54,16 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, 
                                  int sms, const TriBlocked& tb);
 // all eigenvalues of a batch of tridiagonal matrices on the device (sturm.cu):
 // block b's diagonal (n) and off-diagonal (n - 1) from de + 2 off, its
-// eigenvalues in descending order into lam + off; nrm[b] receives the
-// matrix's norm, NaN where an entry is not finite (lam is then undefined)
+// eigenvalues into lam + off, in descending order within each unreduced part of
+// the matrix; nrm[b] receives the matrix's norm, NaN where an entry is not
+// finite (lam is then undefined)
 struct SturmBlk {
   int n;
   long long off;
   int w0, w1;  // first warp of each stage (sturm_plan)
+};
+struct SturmRow {
+  int first, end, ex;  // the unreduced part of a row: rows first .. end - 1, norm in [2^(ex-1), 2^ex)
 };
 struct SturmBatch {
   const SturmBlk* d_blk;  // device, nb entries, n >= 1
@@ -70,7 +74,7 @@ struct SturmBatch {
   double* nrm;                 // device [nb]
   float4* tf;                  // device scratch [sum n] each
   double2 *td, *br;
-  int* shp;  // device scratch [nb]
+  SturmRow* row;
 };
 void sturm_plan(std::vector<SturmBlk>& blk, int sms, SturmBatch* B);
 ed_status sturm_eigenvalues(const SturmBatch& B, cudaStream_t st);

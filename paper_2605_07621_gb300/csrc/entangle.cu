@@ -266,7 +266,7 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
     ED_TRY(mem.get((void**)&sb.tf, n1 * sizeof(float4)));
     ED_TRY(mem.get((void**)&sb.td, n1 * sizeof(double2)));
     ED_TRY(mem.get((void**)&sb.br, n1 * sizeof(double2)));
-    ED_TRY(mem.get((void**)&sb.shp, b1 * sizeof(int)));
+    ED_TRY(mem.get((void**)&sb.row, n1 * sizeof(SturmRow)));
     ED_TRY(mem.get((void**)&d_sblk, b1 * sizeof(SturmBlk)));
     sb.nrm = sb.lam + need;
     sb.de = d_de;
@@ -396,7 +396,8 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       }
       std::copy(dd.begin(), dd.end(), w);
     }
-    // descending (neighbours within the brackets' width may be swapped)
+    // descending (the parts of a matrix follow one another, and neighbours within
+    // the brackets' width may be swapped)
     if (!std::is_sorted(w, w + n, std::greater<double>())) std::sort(w, w + n, std::greater<double>());
   }
   std::copy(lam.begin(), lam.begin() + need, lambda);

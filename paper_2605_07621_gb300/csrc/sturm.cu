@@ -5,7 +5,8 @@
 // of a symmetric tridiagonal matrix by the method of bisection", Numer. Math.
 // 9, 1967; Kahan 1966 for its backward stability).  Every eigenvalue is
 // bracketed on its own, so the whole batch is one launch per stage:
-//   k_sturm_df   brackets of 2^-49 of the norm.  The recurrence runs in
+//   k_sturm_df   brackets of 2^-49 of the norm (of the unreduced part, see
+//                k_sturm_prep).  The recurrence runs in
 //                float-float on the FP32 pipe: a step is about 30 FP32
 //                instructions and a chain of about 60 cycles.
 //   k_sturm_f64  from there to 2^-53 of the norm in FP64, whose pipe takes 64
@@ -35,39 +36,101 @@ namespace edk {
 namespace {
 
 constexpr int kStThreads = 128;
+constexpr int kStPrep = 1024;   // threads of k_sturm_prep
 constexpr int kStPasses = 200;  // most passes of a bracket (S = 1 needs about 60)
 
-// scale T by 2^sh so that its norm max(|d_i| + |e_{i-1}| + |e_i|) lies in [1/2,
-// 1); d and e^2 as float-float (tf) and FP64 (td).  nrm: the norm, NaN if an
-// entry is not finite.  e2 of row i couples it to row i - 1.
-__global__ void __launch_bounds__(1024) k_sturm_prep(const SturmBlk* __restrict__ blk, const double* __restrict__ de,
-                                                     float4* __restrict__ tf, double2* __restrict__ td, int* shp,
-                                                     double* nrm) {
+// The matrix falls apart where an off-diagonal entry is no larger than eps times
+// its two neighbours on the diagonal, or than eps times the norm of the whole
+// matrix (the rule of the QL iteration in eigsym.cu).  Every part is scaled and
+// counted by itself: a part of one row is its own eigenvalue, so a block without
+// weight has exact zeros and a diagonal one keeps levels far below its norm
+// (counted as one matrix they all came out at 2^-53 of the norm, or of 1 for a
+// zero matrix), and the others' brackets are as narrow as their own norm asks.
+//
+// Per block: its parts (row: first row, end, exponent of the part's norm
+// max(|d_i| + |e_{i-1}| + |e_i|)), and the matrix with each part's norm scaled
+// into [1/2, 1): d and e^2 as float-float (tf) and FP64 (td), e2 of row i
+// coupling it to row i - 1, zero in a part's first row.  nrm: the norm, NaN if
+// an entry is not finite.  A thread takes a run of consecutive rows; the first
+// row of each row's part is a prefix maximum over the threads, the end a suffix
+// minimum, the norms are the maxima of the bits (pn, one word per row).
+__global__ void __launch_bounds__(kStPrep) k_sturm_prep(const SturmBlk* __restrict__ blk, const double* __restrict__ de,
+                                                        float4* __restrict__ tf, double2* __restrict__ td,
+                                                        SturmRow* __restrict__ row, unsigned long long* __restrict__ pn,
+                                                        double* nrm) {
   const SturmBlk B = blk[blockIdx.x];
   const double *d = de + 2 * B.off, *e = d + B.n;
-  __shared__ double s_m[32];
-  __shared__ int s_bad;
-  if (threadIdx.x == 0) s_bad = 0;
+  row += B.off;
+  pn += B.off;
+  const int tid = threadIdx.x, n = B.n;
+  __shared__ double s_m[kStPrep / 32];
+  __shared__ int s_bad, s_first[kStPrep], s_end[kStPrep];
+  if (tid == 0) s_bad = 0;
   __syncthreads();
   double mx = 0.0;
-  for (int i = threadIdx.x; i < B.n; i += blockDim.x) {
-    const double t = fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < B.n - 1 ? fabs(e[i]) : 0.0);
+  for (int i = tid; i < n; i += kStPrep) {
+    const double t = fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < n - 1 ? fabs(e[i]) : 0.0);
     if (!isfinite(t)) s_bad = 1;
     mx = fmax(mx, t);
+    pn[i] = 0;
   }
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = mx;
+  if ((tid & 31) == 0) s_m[tid >> 5] = mx;
   __syncthreads();
   mx = s_m[0];
-  for (int w = 1; w < 32; ++w) mx = fmax(mx, s_m[w]);
-  int ex = 0;
-  if (!s_bad && mx > 0.0) frexp(mx, &ex);
-  if (threadIdx.x == 0) {
-    shp[blockIdx.x] = -ex;
-    nrm[blockIdx.x] = s_bad ? __longlong_as_double(0x7ff8000000000000ll) : mx;
+  for (int w = 1; w < kStPrep / 32; ++w) mx = fmax(mx, s_m[w]);
+  if (tid == 0) nrm[blockIdx.x] = s_bad ? __longlong_as_double(0x7ff8000000000000ll) : mx;
+  // a part starts at row i
+  auto starts = [&](int i) {
+    if (i == 0) return true;
+    const double a = fabs(e[i - 1]);
+    return a <= 0x1p-53 * (fabs(d[i - 1]) + fabs(d[i])) || a <= 0x1p-53 * mx;
+  };
+  const int per = (n + kStPrep - 1) / kStPrep, i0 = min(n, tid * per), i1 = min(n, i0 + per);
+  int first = -1, end = n;  // the last start in this thread's rows, and the first
+  for (int i = i0; i < i1; ++i)
+    if (starts(i)) {
+      if (first < 0) end = i;
+      first = i;
+    }
+  s_first[tid] = first;
+  s_end[tid] = end;
+  __syncthreads();
+  for (int o = 1; o < kStPrep; o *= 2) {
+    const int f = tid >= o ? s_first[tid - o] : -1, z = tid + o < kStPrep ? s_end[tid + o] : n;
+    __syncthreads();
+    s_first[tid] = max(s_first[tid], f);
+    s_end[tid] = min(s_end[tid], z);
+    __syncthreads();
   }
-  for (int i = threadIdx.x; i < B.n; i += blockDim.x) {
-    const double ds = ldexp(d[i], -ex), es = i > 0 ? ldexp(e[i - 1], -ex) : 0.0, e2 = es * es;
+  int at = tid > 0 ? s_first[tid - 1] : 0;  // the part of the row before this thread's
+  double pm = 0.0;
+  auto put = [&] {
+    if (pm > 0.0) atomicMax(pn + at, (unsigned long long)__double_as_longlong(pm));
+    pm = 0.0;
+  };
+  for (int i = i0; i < i1; ++i) {
+    if (starts(i)) {
+      put();
+      at = i;
+    }
+    row[i].first = at;
+    const double t = fabs(d[i]) + (i > at ? fabs(e[i - 1]) : 0.0) + (i < n - 1 && !starts(i + 1) ? fabs(e[i]) : 0.0);
+    if (isfinite(t)) pm = fmax(pm, t);
+  }
+  put();
+  int z = tid + 1 < kStPrep ? s_end[tid + 1] : n;  // the end of the part of this thread's last row
+  for (int i = i1 - 1; i >= i0; --i) {
+    row[i].end = z;
+    if (row[i].first == i) z = i;
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += kStPrep) {
+    const int r0 = row[i].first;
+    int ex = 0;
+    if (pn[r0]) frexp(__longlong_as_double((long long)pn[r0]), &ex);
+    row[i].ex = ex;
+    const double ds = ldexp(d[i], -ex), es = i > r0 ? ldexp(e[i - 1], -ex) : 0.0, e2 = es * es;
     td[B.off + i] = make_double2(ds, e2);
     const float2 a = split_scaled(ds, 0), b = split_scaled(e2, 0);
     tf[B.off + i] = make_float4(a.x, a.y, b.x, b.y);
@@ -128,8 +191,9 @@ __device__ __forceinline__ int count_f64(const double2* __restrict__ t, int n, d
   return c;
 }
 
-// the block and eigenvalue of this group of S lanes; warp w of the launch
-// belongs to the block b with first[b] <= w
+// the block and row of this group of S lanes, whose eigenvalue is the one that
+// stands as many places up in the row's part; warp w of the launch belongs to
+// the block b with first[b] <= w
 template <int STAGE>
 __device__ __forceinline__ bool group_of(const SturmBlk* __restrict__ blk, int nb, int S, int& b, int& k) {
   const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -164,39 +228,46 @@ __device__ __forceinline__ void narrow(double& lo, double& hi, int cnt, int k, i
 }
 
 __global__ void __launch_bounds__(kStThreads) k_sturm_df(const SturmBlk* __restrict__ blk, int nb, int S, int warps,
-                                                         const float4* __restrict__ tf, double2* __restrict__ br) {
+                                                         const float4* __restrict__ tf,
+                                                         const SturmRow* __restrict__ row, double2* __restrict__ br) {
   if ((int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) >= warps) return;
   int b, k;
   const bool mine = group_of<0>(blk, nb, S, b, k);
-  const int n = blk[b].n, sub = threadIdx.x & (S - 1);
+  const SturmRow R = row[blk[b].off + k];
+  const int n = R.end - R.first, sub = threadIdx.x & (S - 1);
+  const float4* t = tf + blk[b].off + R.first;
   const double inv = 1.0 / (S + 1);
-  double lo = -1.0, hi = 1.0;
+  double lo = -1.0, hi = n > 1 ? 1.0 : -1.0;  // (a part of one row needs no bracket)
   for (int p = 0; p < kStPasses && __any_sync(0xffffffffu, hi - lo > 0x1p-49); ++p)
-    narrow(lo, hi, count_df(tf + blk[b].off, n, cut(lo, hi, sub, inv)), k, S, inv);
+    narrow(lo, hi, n > 1 ? count_df(t, n, cut(lo, hi, sub, inv)) : 0, k - R.first, S, inv);
   if (mine && sub == 0) br[blk[b].off + k] = make_double2(lo, hi);
 }
 
 __global__ void __launch_bounds__(kStThreads) k_sturm_f64(const SturmBlk* __restrict__ blk, int nb, int S, int warps,
                                                           const double2* __restrict__ td,
-                                                          const double2* __restrict__ br, const int* __restrict__ shp,
+                                                          const double2* __restrict__ br,
+                                                          const SturmRow* __restrict__ row,
                                                           const double* __restrict__ de, double* __restrict__ lam) {
   if ((int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) >= warps) return;
   int b, k;
   const bool mine = group_of<1>(blk, nb, S, b, k);
-  const int n = blk[b].n, sub = threadIdx.x & (S - 1);
+  const SturmRow R = row[blk[b].off + k];
+  const int n = R.end - R.first, sub = threadIdx.x & (S - 1);
+  const double2* t = td + blk[b].off + R.first;
   const double inv = 1.0 / (S + 1);
   const double2 v = br[blk[b].off + k];
   double lo = v.x - 0x1p-49, hi = v.y + 0x1p-49, grow = 0x1p-45;
   // whether the FP64 counts put the eigenvalue above lo, below hi
   bool lok = false, hok = false, stuck = false;  // stuck: no FP64 value in between
+  const int nth = k - R.first;                   // the eigenvalue's number in its part
   for (int p = 0; p < kStPasses; ++p) {
-    const bool wide = hi - lo > 0x1p-53 && !stuck, ends = !wide && !(lok && hok);
+    const bool wide = n > 1 && hi - lo > 0x1p-53 && !stuck, ends = n > 1 && !wide && !(lok && hok);
     if (!__any_sync(0xffffffffu, wide || ends)) break;
     const double x = wide ? cut(lo, hi, sub, inv) : !lok ? lo : hi;
-    const int cnt = count_f64(td + blk[b].off, n, x);
+    const int cnt = wide || ends ? count_f64(t, n, x) : 0;
     const double lo0 = lo, hi0 = hi;
     double a = lo, c = hi;
-    narrow(a, c, cnt, k, S, inv);
+    narrow(a, c, cnt, nth, S, inv);
     if (wide) {
       lo = a;
       hi = c;
@@ -204,7 +275,7 @@ __global__ void __launch_bounds__(kStThreads) k_sturm_f64(const SturmBlk* __rest
       hok |= hi != hi0;
       stuck = lo == lo0 && hi == hi0;
     } else if (ends) {
-      const bool in = !lok ? cnt <= k : cnt > k;
+      const bool in = !lok ? cnt <= nth : cnt > nth;
       if (in) {
         (!lok ? lok : hok) = true;
       } else if (!lok) {  // below lo: that is an upper end
@@ -223,7 +294,7 @@ __global__ void __launch_bounds__(kStThreads) k_sturm_f64(const SturmBlk* __rest
     }
   }
   if (mine && sub == 0)
-    lam[blk[b].off + n - 1 - k] = n == 1 ? de[2 * blk[b].off] : ldexp(0.5 * (lo + hi), -shp[b]);
+    lam[blk[b].off + blk[b].n - 1 - k] = n == 1 ? de[2 * blk[b].off + k] : ldexp(0.5 * (lo + hi), R.ex);
 }
 
 }  // namespace
@@ -231,10 +302,11 @@ __global__ void __launch_bounds__(kStThreads) k_sturm_f64(const SturmBlk* __rest
 ed_status sturm_eigenvalues(const SturmBatch& B, cudaStream_t st) {
   const int nb = (int)B.nb;
   if (nb == 0) return ED_OK;
-  k_sturm_prep<<<nb, 1024, 0, st>>>(B.d_blk, B.de, B.tf, B.td, B.shp, B.nrm);
+  k_sturm_prep<<<nb, kStPrep, 0, st>>>(B.d_blk, B.de, B.tf, B.td, B.row, (unsigned long long*)B.br, B.nrm);
   const int per = kStThreads / 32;
-  k_sturm_df<<<(B.warps0 + per - 1) / per, kStThreads, 0, st>>>(B.d_blk, nb, B.S0, B.warps0, B.tf, B.br);
-  k_sturm_f64<<<(B.warps1 + per - 1) / per, kStThreads, 0, st>>>(B.d_blk, nb, B.S1, B.warps1, B.td, B.br, B.shp, B.de,
+  k_sturm_df<<<(B.warps0 + per - 1) / per, kStThreads, 0, st>>>(B.d_blk, nb, B.S0, B.warps0, B.tf, B.row,
+                                                               B.br);
+  k_sturm_f64<<<(B.warps1 + per - 1) / per, kStThreads, 0, st>>>(B.d_blk, nb, B.S1, B.warps1, B.td, B.br, B.row, B.de,
                                                                 B.lam);
   ED_CUDA_TRY(cudaGetLastError());
   return ED_OK;
