@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(256) k_bapply(const BInst* __restrict__ insts,
                                                 int user_mode) {
   __shared__ float stage[kBW][kBStage];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
   const int n = cnt[0];
   const long long total = n > 0 ? rowpref[n] : 0;
   for (long long row = (long long)blockIdx.x * kBW + warp; row < total; row += (long long)gridDim.x * kBW) {
@@ -81,7 +82,6 @@ __global__ void __launch_bounds__(256) k_bapply(const BInst* __restrict__ insts,
     }
     __syncwarp();
   }
-  pdl_wait();  // after the dense products, which may still run (launch_apply)
 }
 
 // chunk c of the active set -> (instance, element range)
@@ -707,8 +707,8 @@ ed_status BatchEngine::launch_apply(cudaStream_t s, const float* x, float* y) {
     a.err = d_err_;
     ED_TRY(bdense_apply(a, s));
   }
-  // beside the last dense tiles (its instances are others); without dense
-  // products it follows whatever the stream holds
+  // set up while the last dense tiles run; without dense products it follows
+  // whatever the stream holds
   if (dense_)
     ED_CUDA_TRY(launch_pdl(k_bapply, sms_ * 4, 256, 0, s, d_inst_, d_cidx_, d_crowpref_, d_cnt_, x, y, (float*)arena_, user));
   else

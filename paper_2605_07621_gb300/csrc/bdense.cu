@@ -226,23 +226,17 @@ struct BdTile {
 template <int BN>
 __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which) {
   using C = BdCfg<BN>;
-  // The 64-wide tiles follow the slicing and wait for it.  The 128-wide ones
-  // need no more than that: they start on the SMs that the former leave.  They
-  // and k_bapply wait for the kernel before at their end, so that what follows
-  // in the stream follows all three.  (k_bapply starts when the last 128-wide
-  // tile is done: started earlier, its CTAs crowd on the first free SMs.)
-  if (BN == 64) {
-    pdl_wait();
-    pdl_trigger();
-  }
+  // Both widths wait for the kernel before them in the stream, and so does
+  // k_bapply: a grid that was released early sees what earlier grids wrote only
+  // after its own wait.  The early release still lets the 128-wide launch be set
+  // up while the last 64-wide tiles run.
+  pdl_wait();
+  if (BN == 64) pdl_trigger();
   const int n = g.cnt[which];
   const int* vidx = BN == 64 ? g.idx64 : g.idx128;
   const long long* tpref = BN == 64 ? g.tpref64 : g.tpref128;
   const long long total = n > 0 ? tpref[n] : 0;
-  if (total <= 0) {
-    if (BN != 64) pdl_wait();
-    return;
-  }
+  if (total <= 0) return;
 
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)sm_raw + 1023) & ~(uintptr_t)1023);
@@ -551,7 +545,6 @@ __global__ void __launch_bounds__(kBdThreads, 1) k_bgemm(BDenseArgs g, int which
     tc::tc_fence_after();
     tc::tmem_dealloc(tmem, C::kTmemCols);
   }
-  if (BN != 64) pdl_wait();
 }
 
 ed_status bdense_prepare() {
