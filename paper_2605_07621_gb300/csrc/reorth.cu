@@ -4,12 +4,17 @@
 // about 183 us for 150 vectors of 731,808 elements), which the update's
 // products would occupy as long again.  So the update runs in FP32 on an FP32
 // copy of the basis (a plane of rows of fp32_ld(n) elements, written with each
-// vector) while every |h_j| is at most 2^-36 |w|: after a Lanczos step they
-// are at rounding level (2^-50), and the FP32 products then add less than 2^-56
-// of |w| to an element, below the rounding of w itself.  Otherwise, and
-// without the plane, it takes the FP64 basis.
+// vector) where that costs no digit of w: the rounding of the m coefficients,
+// of the plane and of the m FP32 additions of an element is at most (m + 3)
+// 2^-24 sum_j |h_j| |V_j|, over all elements in norm (m + 3) 2^-24 sum_j |h_j|
+// for unit vectors V_j, and the update takes the plane while that is at most
+// 2^-54 |w|, below the rounding of w itself (kRoSmall).  |w| is the norm before
+// this very pass, so the second pass after a large first one is judged by what
+// the first one left.  After a Lanczos step the coefficients are at rounding
+// level, 300 of them at about 2^-52: 2^-59.  Otherwise, and without the plane,
+// the FP64 basis.
 // 300-step Green's function of the 12-site Hubbard ring (two sectors of
-// 731,808 states): 554 -> 391 ms (dots 210 us at 0.54 T products/s, update 75
+// 731,808 states): 554 -> 394 ms (dots 210 us at 0.54 T products/s, update 75
 // us).  Not kept: float-float dots on two FP32 planes (325 ms, but G of the
 // reference test scattered about 20 % more) and exact integer dots on
 // fixed-point planes (416 ms: bound by the 32 x 32 + 64-bit multiply-adds).
@@ -22,7 +27,7 @@
 namespace edk {
 
 constexpr int kRoBatch = 8;  // basis vectors per CTA of the dots
-constexpr double kRoSmall = 0x1p-36;
+constexpr double kRoSmall = 0x1p-30;  // (m + 3) sum |h_j| / |w| up to which the update takes the FP32 plane
 
 // part[j * gridDim.x + blockIdx.x] = the share of <V_j, w> of the CTA's column
 // range, for the kRoBatch vectors of blockIdx.y: w is read once for eight
@@ -82,10 +87,11 @@ __global__ void __launch_bounds__(256) k_reorth_sum(const double* __restrict__ p
   if (lane == 0) h[j] = s;
 }
 
-// w -= sum_j h_j V_j, four elements per thread and U vectors in flight; NORM:
-// then beta = ||w|| by the last CTA.  *beta holds the norm of w before the
-// orthogonalisation.  F: the FP32 plane (row stride ldf), or null.
-template <bool NORM>
+// w -= sum_j h_j V_j, four elements per thread and U vectors in flight; LAST, or
+// where the coefficients are large: then beta = ||w|| by the last CTA (small ones
+// leave the norm as it was, to 2^-60).  *beta holds the norm of w before.  F: the
+// FP32 plane (row stride ldf), or null.
+template <bool LAST>
 __global__ void __launch_bounds__(128) k_reorth_update(const double* __restrict__ V, long long ldv,
                                                        const float* __restrict__ F, long long ldf, int m,
                                                        double* __restrict__ w, long long n,
@@ -98,14 +104,15 @@ __global__ void __launch_bounds__(128) k_reorth_update(const double* __restrict_
   constexpr int U = 8;
   const double b0 = beta[0];
   const int sh = min(900, max(-900, 1022 - biased_exp(b0)));  // the norm near 1
-  bool big = F == nullptr;
+  double hsum = 0.0;
   for (int j = threadIdx.x; j < m; j += 128) {
     const double v = h[j];
     hs[j] = v;
     hf[j] = (float)ldexp(v, sh);
-    big = big || !(fabs(v) <= kRoSmall * b0);
+    hsum += fabs(v);
   }
-  big = __syncthreads_or(big);
+  hsum = block_sum(hsum);
+  const bool big = __syncthreads_or(threadIdx.x == 0 && !(F && (m + 3) * hsum <= kRoSmall * b0));
   double nacc = 0.0;
   for (long long i = 4 * (blockIdx.x * 128ll + threadIdx.x); i < n; i += 4 * gridDim.x * 128ll) {
     double s[4];
@@ -144,28 +151,27 @@ __global__ void __launch_bounds__(128) k_reorth_update(const double* __restrict_
       if (i + q < n) {
         const double v = w[i + q] - s[q];
         w[i + q] = v;
-        if constexpr (NORM) nacc = fma(v, v, nacc);
+        if (LAST || big) nacc = fma(v, v, nacc);
       }
   }
-  if constexpr (NORM) {
-    const double s = block_sum(nacc);
-    __shared__ unsigned s_last;
-    if (threadIdx.x == 0) {
-      npart[blockIdx.x] = s;
+  if (!LAST && !big) return;
+  const double s = block_sum(nacc);
+  __shared__ unsigned s_last;
+  if (threadIdx.x == 0) {
+    npart[blockIdx.x] = s;
+    __threadfence();
+    s_last = atomicAdd(ctr, 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (s_last) {
+      *ctr = 0u;
       __threadfence();
-      s_last = atomicAdd(ctr, 1u) == gridDim.x - 1 ? 1u : 0u;
-      if (s_last) {
-        *ctr = 0u;
-        __threadfence();
-      }
     }
-    __syncthreads();
-    if (!s_last) return;
-    double v = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += 128) v += __ldcg(npart + i);
-    const double t = block_sum(v);
-    if (threadIdx.x == 0) beta[0] = sqrt(t > 0.0 ? t : 0.0);
   }
+  __syncthreads();
+  if (!s_last) return;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 128) v += __ldcg(npart + i);
+  const double t = block_sum(v);
+  if (threadIdx.x == 0) beta[0] = sqrt(t > 0.0 ? t : 0.0);
 }
 
 long long fp32_ld(long long n) { return (n + 3) / 4 * 4; }
