@@ -76,7 +76,9 @@ constexpr int kPsT = 16;           // threads per row of k_psum2
 // one reduction, m = 924 / 1716 / 3432 / 5005: three kernels per column 28.4 /
 // 56.9 / 124.7 / 216.5 ms, one launch per panel 10.1 / 19.6 / 48.0 / 122.8 ms;
 // m = 6435 / 11440 with the line at 64: 331 / 1037 ms, at 6144: 250 / 957, at
-// 8192: 254 / 986.
+// 8192: 254 / 986.  It also needs as many CTAs as hold the rows in shared memory
+// (tridiag_panel_ctas: 39 at 6,144 rows, 6 at 1,001): a lane of the spectrum with
+// fewer SMs takes the three kernels per column (see entangle_shares).
 constexpr int kPtMax = 6144;
 constexpr int kPtSmem = 216 * 1024;  // its dynamic shared memory at most
 constexpr int kPtRows = 24;        // rows per CTA it aims at (two warps per four rows, 12 warps)
@@ -1127,6 +1129,20 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), unsigned grid, unsigned block
   return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// shared memory of k_panel_tri: `chunk` rows per CTA, `cols` columns of the
+// trailing matrix's copy
+static size_t panel_smem(int chunk, long long cols) {
+  return ((size_t)chunk * (kKw + 7) + (size_t)cols + 4) * sizeof(float2);
+}
+
+int tridiag_panel_ctas(int m) {
+  const int rows = std::min(m, kPtMax);
+  if (rows <= 64) return 1;
+  int g = 1;
+  while (panel_smem((rows + g - 1) / g, rows + 1) > kPtSmem) ++g;
+  return g;
+}
+
 ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, double* e_out, cudaStream_t st,
                                  int sms, const TriBlocked& tb) {
   if (m <= 0) return ED_OK;
@@ -1165,10 +1181,11 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, 
     k_amax<<<ga, 256, 0, st>>>(A, m, P.k0, amx);
     // one launch for the panel: at least kPtRows rows per CTA (a matrix of up
     // to 64 rows in one), while a CTA's rows and the column fit shared memory
+    // (with tridiag_panel_ctas(m) CTAs or more they do)
     const int rows = m - P.k0;
     const int g = rows <= 64 ? 1 : (int)std::min((long long)std::min(tb.ctas, kPtCtas), cdiv(rows, kPtRows));
     const int chunk = (int)cdiv(rows, g);
-    const size_t smem = ((size_t)chunk * (kKw + 7) + (size_t)(tb.ldF - P.k0) + 4) * sizeof(float2);
+    const size_t smem = panel_smem(chunk, tb.ldF - P.k0);
     if (rows <= kPtMax && smem <= kPtSmem) {
       const long long T = cdiv(rows, 32);
       const int gc = (int)std::max(1LL, std::min((long long)sms * 8, T * (T + 1) / 2));

@@ -23,6 +23,11 @@ std::vector<TriPanel> tridiag_panels(int m);
 // and, per panel, two slicing jobs and one product (built by
 // tridiag_blocked_setup, on device)
 inline long long tridiag_ldF(int m) { return m + (m & 1); }
+// fewest CTAs with which an m x m reduction takes one launch for every panel of
+// up to kPtMax rows (eigsym.cu)
+int tridiag_panel_ctas(int m);
+// entangle.cu
+void entangle_shares(const long long* m, int nb, int lanes, int sms, int* lane_of, int* share);
 struct TriBlocked {
   OzContext* oz;
   double* NVW;

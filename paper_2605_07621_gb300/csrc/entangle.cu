@@ -42,6 +42,57 @@ struct DevMem {
 };
 
 }  // namespace
+
+// The lane of each of nb blocks (of m[i] rows) and the share of the SMs of each
+// lane: the blocks, largest first, to the lane with the least work so far, and
+// the SMs so that the lanes end together.  A reduction on g SMs takes about
+// serial(m) + spread(m) / g microseconds (m = 1716 / 3003 / 3432 alone on 25 to
+// 152 SMs: within 5 %).  No lane gets fewer SMs than the panels of up to
+// kShareRows rows of its blocks need to run as one launch each
+// (tridiag_panel_ctas): by their work alone the lanes of a few hundred to two
+// thousand rows beside larger ones got so few that their panels went back to
+// three kernels per column.  28 sites with 11 / 9 up spins (m up to 2,002 / 1,001):
+// 42.0 -> 33.0 / 17.2 -> 15.1 ms, 30 sites with 12 (5,005): 204 -> 183.  Larger
+// panels on few SMs are better off with those kernels, which use the whole GPU:
+// with the line at 4,096 rows, or for all, 32 sites with 12 up spins (8,008) 514
+// -> 573 / 591, 30 with 15 623 -> 632 / 690, 32 with 16 3,174 -> 3,232 / 3,459; at
+// 2,048: 520, 620, 3,178.  On a GPU with fewer SMs than the needs add up to, a
+// lane's launches wait for another's.
+constexpr long long kShareRows = 2048;
+void entangle_shares(const long long* m, int nb, int lanes, int sms, int* lane_of, int* share) {
+  std::vector<int> order(nb), need(lanes, 0);
+  for (int i = 0; i < nb; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return m[u] > m[v]; });
+  auto serial = [](double x) { return x * (9.0 + 0.6e-3 * x); };
+  auto spread = [](double x) { return 1.45e6 * std::pow(x / 3432.0, 2.5); };
+  std::vector<double> lane_serial(lanes, 0.0), lane_spread(lanes, 0.0), load(lanes, 0.0);
+  for (int i : order) {
+    const double x = (double)m[i];
+    const int k = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    lane_of[i] = k;
+    load[k] += serial(x) + spread(x) * lanes / sms;
+    lane_serial[k] += serial(x);
+    lane_spread[k] += spread(x);
+    need[k] = std::max(need[k], std::min(sms, tridiag_panel_ctas((int)std::min(m[i], kShareRows))));
+  }
+  // the lanes end together, at T: bisection for the least T at which the shares fit
+  double lo = *std::max_element(lane_serial.begin(), lane_serial.end()), hi = lo + 1.0;
+  auto shares = [&](double T) {
+    int sum = 0;
+    for (int k = 0; k < lanes; ++k) {
+      share[k] = (int)std::min((double)sms, std::max((double)need[k], std::floor(lane_spread[k] / (T - lane_serial[k]))));
+      sum += share[k];
+    }
+    return sum;
+  };
+  for (int i = 0; i < 60 && shares(hi) > sms; ++i) hi = lo + 2.0 * (hi - lo);
+  for (int i = 0; i < 40; ++i) {
+    const double mid = 0.5 * (lo + hi);
+    if (shares(mid) > sms) lo = mid; else hi = mid;
+  }
+  shares(hi);
+}
+
 }  // namespace edk
 
 using namespace edk;
@@ -117,47 +168,13 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
     const double one = lane_bytes(m0, x0);
     while (lanes > 1 && one * lanes > 0.8 * (double)fr) --lanes;
   }
-  std::vector<int> lane_of(nb, 0);
+  std::vector<long long> mb(nb);
+  for (size_t bi = 0; bi < nb; ++bi) mb[bi] = bm(bi);
+  std::vector<int> lane_of(nb, 0), share(lanes, 1);
+  entangle_shares(mb.data(), (int)nb, lanes, sms, lane_of.data(), share.data());
   std::vector<std::vector<size_t>> lane_blocks(lanes);
-  // a reduction on g SMs takes about serial(m) + spread(m) / g microseconds
-  // (m = 1716 / 3003 / 3432 alone on 25 to 152 SMs: within 5 %)
-  auto serial = [](double m) { return m * (9.0 + 0.6e-3 * m); };
-  auto spread = [](double m) { return 1.45e6 * std::pow(m / 3432.0, 2.5); };
-  std::vector<double> lane_serial(lanes, 0.0), lane_spread(lanes, 0.0);
-  {
-    std::vector<double> load(lanes, 0.0);
-    for (size_t oi = 0; oi < nb; ++oi) {
-      const size_t bi = order[oi];
-      const double m = (double)bm(bi);
-      const int k = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-      lane_of[bi] = k;
-      load[k] += serial(m) + spread(m) * lanes / sms;
-      lane_serial[k] += serial(m);
-      lane_spread[k] += spread(m);
-      lane_blocks[k].push_back(bi);
-    }
-  }
+  for (size_t bi : order) lane_blocks[lane_of[bi]].push_back(bi);
   while (lanes > 1 && lane_blocks[lanes - 1].empty()) --lanes;
-  // the SMs shared out so that the lanes end together, at T: bisection for the
-  // least T at which the shares fit
-  std::vector<int> share(lanes, 1);
-  {
-    double lo = *std::max_element(lane_serial.begin(), lane_serial.begin() + lanes), hi = lo + 1.0;
-    auto shares = [&](double T) {
-      int sum = 0;
-      for (int k = 0; k < lanes; ++k) {
-        share[k] = (int)std::min((double)sms, std::max(1.0, std::floor(lane_spread[k] / (T - lane_serial[k]))));
-        sum += share[k];
-      }
-      return sum;
-    };
-    for (int i = 0; i < 60 && shares(hi) > sms; ++i) hi = lo + 2.0 * (hi - lo);
-    for (int i = 0; i < 40; ++i) {
-      const double mid = 0.5 * (lo + hi);
-      if (shares(mid) > sms) lo = mid; else hi = mid;
-    }
-    shares(hi);
-  }
 
   DevMem mem;
   OzContext oz;
