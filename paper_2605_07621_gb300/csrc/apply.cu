@@ -398,9 +398,12 @@ static ed_status launch_apply_rows(const ed_ctx* c, const T* x, T* y, cudaStream
   const long long stage_elems = ((mdb + 16 / (long long)sizeof(T) + 15) / 16) * 16;
   const size_t smem2 = 128 + 2 * (size_t)stage_elems * sizeof(T);
   const bool aligned = ((uintptr_t)x % 16) == 0;
-  if (aligned && smem2 <= 220 * 1024) {
+  // (the attributes below are the functions': the same value for every context,
+  // so that another thread's cannot come between them and the launch)
+  constexpr size_t most2 = 220 * 1024, most = 200 * 1024;
+  if (aligned && smem2 <= most2) {
     auto kern = k_rowpass<T>;
-    ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
+    ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most2));
     const long long grid = std::min<long long>(p.n_rows, (long long)sms);
     kern<<<(unsigned)grid, 256, smem2, st>>>(p, x, y, stage_elems, c->d_err);
     ED_CUDA_TRY(cudaGetLastError());
@@ -417,9 +420,9 @@ static ed_status launch_apply_rows(const ed_ctx* c, const T* x, T* y, cudaStream
   int threads = (int)std::min<int64_t>(256, ((mdb + 31) / 32) * 32);
   threads = std::max(threads, 64);
   const long long grid = std::min<long long>(p.n_rows, (long long)sms * 16);
-  if (smem <= 200 * 1024) {
+  if (smem <= most) {
     auto kern = k_apply_rows<T, true>;
-    ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     kern<<<(unsigned)grid, threads, smem, st>>>(p, x, y);
   } else {
     k_apply_rows<T, false><<<(unsigned)grid, threads, 0, st>>>(p, x, y);

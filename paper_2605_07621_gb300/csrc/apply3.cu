@@ -526,11 +526,13 @@ static size_t v3_smem(const ed_ctx* c) {
   return (size_t)(mdb + 8) * 16;
 }
 
-constexpr size_t kRowHalf = 106 * 1024;  // most row bytes for two CTAs of the row pass per SM
+constexpr size_t kRowMax = 220 * 1024;      // most row bytes of the row pass
+constexpr size_t kRowHalf = 106 * 1024;     // for two CTAs of it per SM
+constexpr size_t kRowQuarter = 50 * 1024;   // for four
 
 bool v3_usable(const ed_ctx* c, ed_dtype dt, const void* x) {
   (void)dt;
-  return c->v3_ok && ((uintptr_t)x % 16) == 0 && v3_smem(c) <= 220 * 1024;
+  return c->v3_ok && ((uintptr_t)x % 16) == 0 && v3_smem(c) <= kRowMax;
 }
 
 // events bracketing the stages of one apply when profiling is on
@@ -569,16 +571,18 @@ static ed_status run_v3(ed_ctx* c, const std::conditional_t<CVT, double, typenam
     const long long ng = R == 4 ? c->n_grp4 : c->n_grp2;
     // 1024 threads per SM: in one CTA while its rows need more than half of
     // the shared memory, else in two or four CTAs, so that one stages its
-    // rows while another sums
-    auto go = [&](auto kern, int nt) -> ed_status {
-      ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // rows while another sums.  (The attribute is the function's: the same value
+    // for every context, so that another thread's cannot come between it and
+    // the launch.)
+    auto go = [&](auto kern, int nt, size_t most) -> ed_status {
+      ED_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
       const long long grid = std::min<long long>(ng, (long long)sms * (1024 / nt));
       ED_CUDA_TRY(launch_pdl(kern, grid, nt, smem, st, p, gs, ng, x, y, emax, xw, part, npart));
       return ED_OK;
     };
-    if (smem > kRowHalf) ED_TRY(go(k_row5<Pol, R, 1024, CVT>, 1024));
-    else if (smem > 50 * 1024) ED_TRY(go(k_row5<Pol, R, 512, CVT>, 512));
-    else ED_TRY(go(k_row5<Pol, R, 256, CVT>, 256));
+    if (smem > kRowHalf) ED_TRY(go(k_row5<Pol, R, 1024, CVT>, 1024, kRowMax));
+    else if (smem > kRowQuarter) ED_TRY(go(k_row5<Pol, R, 512, CVT>, 512, kRowHalf));
+    else ED_TRY(go(k_row5<Pol, R, 256, CVT>, 256, kRowQuarter));
   }
   pm.mark(3, st);
   constexpr int q = sizeof(typename Pol::S) == 4 ? 1 : 0;
