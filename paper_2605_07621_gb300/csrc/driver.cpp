@@ -276,7 +276,8 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
   };
   // small sectors without orthogonalisation: the step after H|psi> is one
   // launch (in tail), except for the last step, which has no next vector
-  const bool small = !reorth && !pro && lz_step_fits(c, n);
+  // (a refused launch, found at the first step, leaves it to the three kernels)
+  bool small = !reorth && !pro && lz_step_fits(c, n);
   auto one_launch = [&](int j) { return small && j + 1 < max_iter; };
   // one step up to its history entry (apply, alpha, beta, orthogonalisation)
   auto head = [&](int j, bool& ortho_now) -> ed_status {
@@ -323,13 +324,23 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
     T* out = in_place ? (T*)basis_next(basis) : nullptr;
     const bool stored = out != nullptr;
     if (!out) out = v == bufs[0] ? bufs[1] : bufs[0];
+    const bool fix = fuse && c->d_fixed;
+    ed_status one = ED_EUNSUPPORTED;
     if (one_launch(j)) {
-      const bool fix = fuse && c->d_fixed;
-      ED_TRY(launch_lz_step<T>(c, w, v, vprev, out, j > 0 ? 1 : 0, n, fix, hist, hcount, st));
+      one = launch_lz_step<T>(c, w, v, vprev, out, j > 0 ? 1 : 0, n, fix, hist, hcount, st);
+      if (one == ED_EUNSUPPORTED) {
+        small = false;
+        launch_lz_a<T>(c, w, v, vprev, j > 0 ? 1 : 0, n, st);
+        launch_lz_b<T>(c, w, v, n, fuse ? ew : nullptr, hist, hcount, st);
+      } else {
+        ED_TRY(one);
+      }
+    }
+    if (one == ED_OK) {
       prepared = fix;
     } else if constexpr (std::is_same<T, double>::value) {
       // (after an orthogonalisation the exponent lz_b recorded may be stale)
-      if (fuse && c->d_fixed && !ortho_now) {
+      if (fix && !ortho_now) {
         launch_lz_c_fixed(c, w, out, c->d_fixed, ew, c->d_exp, n, st);
         prepared = true;
       } else {

@@ -33,6 +33,16 @@ void set_error(const char* fmt, ...);
     if (s_ != ED_OK) return s_;      \
   } while (0)
 
+// A launch whose CTAs wait for one another was refused because they cannot all be
+// resident (part of the GPU given to others): the error is cleared, and the
+// caller takes the kernels that need no such thing.
+inline bool grid_refused(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources && e != cudaErrorInvalidClusterSize)
+    return false;
+  cudaGetLastError();
+  return true;
+}
+
 // Makes `dev` the current device for the scope of one entry point and puts
 // the caller's current device back on exit, so no call changes the calling
 // thread's current device.

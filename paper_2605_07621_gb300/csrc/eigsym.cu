@@ -1173,6 +1173,7 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, 
   pb.ctr = reinterpret_cast<unsigned*>(pb.cp + (long long)kPtCtas * kPtCp);
   ED_CUDA_TRY(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned), st));
   const std::vector<TriPanel> pan = tridiag_panels(m);  // none for m < 3: k_tail alone
+  bool refused = false;  // k_panel_tri's CTAs cannot all be resident: the kernels per column instead
   for (size_t q = 0; q < pan.size(); ++q) {
     const TriPanel& P = pan[q];
     ED_CUDA_TRY(cudaMemsetAsync(tb.WV + (long long)P.k0 * kKw, 0, (size_t)(m - P.k0) * kKw * sizeof(double), st));
@@ -1186,7 +1187,8 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, 
     const int g = rows <= 64 ? 1 : (int)std::min((long long)std::min(tb.ctas, kPtCtas), cdiv(rows, kPtRows));
     const int chunk = (int)cdiv(rows, g);
     const size_t smem = panel_smem(chunk, tb.ldF - P.k0);
-    if (rows <= kPtMax && smem <= kPtSmem) {
+    bool one = rows <= kPtMax && smem <= kPtSmem && !refused;
+    if (one) {
       const long long T = cdiv(rows, 32);
       const int gc = (int)std::max(1LL, std::min((long long)sms * 8, T * (T + 1) / 2));
       ED_CUDA_TRY(launch_pdl(k_pconv_full, gc, 256, st, A, tb.F, tb.ldF, m, P.k0, amx, ga, shp));
@@ -1203,9 +1205,13 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, 
       at[0].val.cooperative = 1;
       cfg.attrs = at;
       cfg.numAttrs = 1;
-      ED_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_tri, (const float2*)tb.F, tb.ldF, m, P.k0, P.jb, chunk,
-                                     (const int*)shp, tb.WVf, d, e, pb, tb.err));
-    } else {
+      const cudaError_t le = cudaLaunchKernelEx(&cfg, k_panel_tri, (const float2*)tb.F, tb.ldF, m, P.k0, P.jb, chunk,
+                                                (const int*)shp, tb.WVf, d, e, pb, tb.err);
+      refused = grid_refused(le);
+      if (!refused) ED_CUDA_TRY(le);
+      one = !refused;
+    }
+    if (!one) {
       // float-float copy of the panel's trailing triangle (rows and columns >= k0)
       {
         const int gc = (int)std::max(1LL, std::min((long long)sms * 8, cdiv(m - P.k0, 8)));

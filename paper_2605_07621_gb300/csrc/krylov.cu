@@ -784,10 +784,12 @@ static ed_status go_lz_step(ed_ctx* c, const T* w, const T* v, const T* vprev, T
   }
   cfg.attrs = at;
   cfg.numAttrs = cl ? 2 : 1;
-  ED_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, w, v, vprev, out, use_beta, n, c->d_partials, slot(c, 0), slot(c, 1), hist,
-                                 hcount, FIX ? c->d_exp + 16 : (int*)nullptr, FIX ? c->d_exp : (int*)nullptr,
-                                 FIX ? c->d_fixed : (long long*)nullptr, FIX ? c->t3.P : 0, (unsigned*)c->d_err + 4,
-                                 c->d_err));
+  const cudaError_t le = cudaLaunchKernelEx(
+      &cfg, kern, w, v, vprev, out, use_beta, n, c->d_partials, slot(c, 0), slot(c, 1), hist, hcount,
+      FIX ? c->d_exp + 16 : (int*)nullptr, FIX ? c->d_exp : (int*)nullptr, FIX ? c->d_fixed : (long long*)nullptr,
+      FIX ? c->t3.P : 0, (unsigned*)c->d_err + 4, c->d_err);
+  if (grid_refused(le)) return ED_EUNSUPPORTED;
+  ED_CUDA_TRY(le);
   return ED_OK;
 }
 template <typename T>

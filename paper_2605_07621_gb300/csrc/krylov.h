@@ -34,7 +34,8 @@ void launch_lz_b(ed_ctx* c, T* w, const T* v, long long n, int* ew, double* hist
 template <typename T>
 void launch_lz_c(ed_ctx* c, const T* w, T* out, long long n, cudaStream_t st);
 // lz_a, lz_b and lz_c (fix: lz_c_fixed) in one launch, where the vectors fit the
-// registers of one grid; w is only read
+// registers of one grid; w is only read.  ED_EUNSUPPORTED (no message): the
+// launch was refused, nothing has run
 bool lz_step_fits(const ed_ctx* c, long long n);
 template <typename T>
 ed_status launch_lz_step(ed_ctx* c, const T* w, const T* v, const T* vprev, T* out, int use_beta, long long n,
