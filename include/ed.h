@@ -166,7 +166,13 @@ void ed_lanczos_default_opts(ed_lanczos_opts* o);
  * changes by at most tol (relative) over check_every steps; when psi0 is
  * requested the Ritz residual estimate beta_m |s_m| must also be at most
  * 1e-10 max(1, |E0|).  Synchronises the stream.  Returns ED_ENOCONV (with
- * *e0 and the report filled) when this was not met within max_iter. */
+ * *e0 and the report filled) when this was not met within max_iter.
+ * Between 131,072 and about 1.2 M states a step is a cooperative launch, whose
+ * CTAs wait for one another and so need all SMs now and then.  Where they do not
+ * get them (part of the GPU is given to others: the launch is refused; other work
+ * holds SMs for some seconds: a wait runs out) the run takes, or starts again
+ * with, kernels that do not wait; the same holds for ed_lanczos_gf without
+ * re-orthogonalisation and, for its reductions, ed_entanglement_spectrum. */
 ed_status ed_lanczos_ground(ed_ctx* ctx, const ed_lanczos_opts* opts, double* e0, void* psi0, ed_report* rep);
 
 /* Zero-temperature Green's function of a Hubbard context:

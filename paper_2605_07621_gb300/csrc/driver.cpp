@@ -226,9 +226,10 @@ struct OmegaPRO {
   }
 };
 
+// one_form: small sectors may take a step in one launch.
 template <typename T>
-ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_iter, double tol, int check_every,
-                 bool fixed, bool reorth, Basis* basis, RunOut& out, double resid_tol = 0.0, bool partial = false) {
+ed_status lz_steps(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_iter, double tol, int check_every,
+                   bool fixed, bool reorth, Basis* basis, RunOut& out, double resid_tol, bool partial, bool one_form) {
   const long long n = c->D;
   T* vprev = bufs[0];
   T* v = bufs[1];
@@ -277,7 +278,7 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
   // small sectors without orthogonalisation: the step after H|psi> is one
   // launch (in tail), except for the last step, which has no next vector
   // (a refused launch, found at the first step, leaves it to the three kernels)
-  bool small = !reorth && !pro && lz_step_fits(c, n);
+  bool small = one_form && !reorth && !pro && lz_step_fits(c, n);
   auto one_launch = [&](int j) { return small && j + 1 < max_iter; };
   // one step up to its history entry (apply, alpha, beta, orthogonalisation)
   auto head = [&](int j, bool& ortho_now) -> ed_status {
@@ -482,6 +483,22 @@ ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_it
   out.orthogonalised = pro ? om.count : (reorth ? steps : 0);
   if (basis && basis->count > steps) basis->count = steps;
   return ED_OK;
+}
+
+// The recurrence; where a one-launch step's wait for its CTAs ran out (other work
+// held SMs for seconds) once more from v0 with kernels that do not wait.
+template <typename T>
+ed_status lz_run(ed_ctx* c, cudaStream_t st, T* bufs[3], const T* v0, int max_iter, double tol, int check_every,
+                 bool fixed, bool reorth, Basis* basis, RunOut& out, double resid_tol = 0.0, bool partial = false) {
+  const bool kept = basis && basis->complete;
+  const ed_status s = lz_steps<T>(c, st, bufs, v0, max_iter, tol, check_every, fixed, reorth, basis, out, resid_tol,
+                                  partial, true);
+  if (s != ED_ETIMEOUT) return s;
+  if (basis) {
+    basis->count = 0;
+    basis->complete = kept;
+  }
+  return lz_steps<T>(c, st, bufs, v0, max_iter, tol, check_every, fixed, reorth, basis, out, resid_tol, partial, false);
 }
 
 // Ritz vector x = sum_j s_j v_j (FP64, normalised) from a stored basis or,

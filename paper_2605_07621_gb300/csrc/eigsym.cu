@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
       __threadfence();
       atomicAdd(B.ctr, 1u);
       if (!pt_poll(B.ctr, bars * (unsigned)G)) {
-        atomicExch(err, 4);
+        atomicExch(err, kPanelLate);
         s_abort = 1;
       }
     }
@@ -883,7 +883,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
           atomicAdd(B.ctr + 1, done);
         }
         if (!pt_poll(B.ctr + 1, (unsigned)kPtSlots * (unsigned)(j + 1))) {
-          atomicExch(err, 4);
+          atomicExch(err, kPanelLate);
           s_abort = 1;
         }
       }
@@ -1173,7 +1173,7 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, 
   pb.ctr = reinterpret_cast<unsigned*>(pb.cp + (long long)kPtCtas * kPtCp);
   ED_CUDA_TRY(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned), st));
   const std::vector<TriPanel> pan = tridiag_panels(m);  // none for m < 3: k_tail alone
-  bool refused = false;  // k_panel_tri's CTAs cannot all be resident: the kernels per column instead
+  bool refused = tb.ctas < 1;  // k_panel_tri's CTAs cannot all be resident: the kernels per column instead
   for (size_t q = 0; q < pan.size(); ++q) {
     const TriPanel& P = pan[q];
     ED_CUDA_TRY(cudaMemsetAsync(tb.WV + (long long)P.k0 * kKw, 0, (size_t)(m - P.k0) * kKw * sizeof(double), st));
@@ -1184,7 +1184,7 @@ ed_status tridiag_reduce_blocked(double* A, int m, double* work, double* d_out, 
     // to 64 rows in one), while a CTA's rows and the column fit shared memory
     // (with tridiag_panel_ctas(m) CTAs or more they do)
     const int rows = m - P.k0;
-    const int g = rows <= 64 ? 1 : (int)std::min((long long)std::min(tb.ctas, kPtCtas), cdiv(rows, kPtRows));
+    const int g = rows <= 64 ? 1 : (int)std::min((long long)std::max(1, std::min(tb.ctas, kPtCtas)), cdiv(rows, kPtRows));
     const int chunk = (int)cdiv(rows, g);
     const size_t smem = panel_smem(chunk, tb.ldF - P.k0);
     bool one = rows <= kPtMax && smem <= kPtSmem && !refused;

@@ -26,6 +26,7 @@ inline long long tridiag_ldF(int m) { return m + (m & 1); }
 // fewest CTAs with which an m x m reduction takes one launch for every panel of
 // up to kPtMax rows (eigsym.cu)
 int tridiag_panel_ctas(int m);
+constexpr int kPanelLate = 4;  // TriBlocked::err: a wait of the panel kernel ran out
 // entangle.cu
 void entangle_shares(const long long* m, int nb, int lanes, int sms, int* lane_of, int* share);
 struct TriBlocked {
@@ -39,7 +40,7 @@ struct TriBlocked {
   int* err;
   const OzSliceJob* d_jobs;
   const OzProblem* d_probs;
-  int ctas;  // most CTAs of the panel kernel (they wait for one another: all must be resident)
+  int ctas;  // most CTAs of the panel kernel (they wait for one another: all must be resident); 0: none
 };
 // appends the jobs and products of an m x m reduction of A (tensor maps in oz;
 // opA / opB: digit-plane buffers for m x 2 kTriNb operands)

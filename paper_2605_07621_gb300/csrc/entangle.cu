@@ -97,9 +97,10 @@ void entangle_shares(const long long* m, int nb, int lanes, int sms, int* lane_o
 
 using namespace edk;
 
-extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, double* lambda, int64_t cap,
-                                              int64_t* n_lambda, double* weight, double* entropy, double* stage_ms,
-                                              void* stream) {
+// panels: the reductions may take one cooperative launch per panel.  late: a wait
+// of those launches ran out (the status is then not ED_OK).
+static ed_status spectrum(ed_ctx* c, const double* psi, double* lambda, int64_t cap, int64_t* n_lambda, double* weight,
+                          double* entropy, double* stage_ms, void* stream, bool panels, bool* late) {
   if (!c || !n_lambda) {
     set_error("ctx or n_lambda is NULL");
     return ED_EINVAL;
@@ -358,7 +359,7 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
       if ((s = oz_gemm(&oz, d_probs + bi, 1, tiles[bi], nullptr, ln.s)) != ED_OK) return fail(s);
       if (cudaEventRecord(ev_g1.e[bi], ln.s) != cudaSuccess) return fail(ED_ECUDA);
       TriBlocked tb{&oz, ln.NVW, ln.WV, ln.WVf, ln.F, tridiag_ldF(m), {}, oz.d_err, d_tjobs + 2 * toff[bi],
-                    d_tprobs + toff[bi], share[k]};
+                    d_tprobs + toff[bi], panels ? share[k] : 0};
       if (m >= 3 && (s = tmap_8b_2d(&tb.tmF, ln.F, m, m, tb.ldF, 34, 32)) != ED_OK) return fail(s);
       if ((s = tridiag_reduce_blocked(ln.G, m, ln.work, bd, bd + m, ln.s, sms, tb)) != ED_OK) return fail(s);
     }
@@ -390,7 +391,10 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
     ED_TRY(dot_dev<double>(c, psi + b.off, psi + b.off, b.dA * b.dB, slot(c, 3), st, 0));
     ED_TRY(read_scalars(c, 3, 1, &wt[bi], st));  // synchronises the stream
   }
-  ED_TRY(oz_status(&oz, st));  // no bounded wait of the reduction's kernels ran out
+  int code = 0;
+  const ed_status waits = oz_status(&oz, st, &code);  // no bounded wait of the reduction's kernels ran out
+  *late = code == kPanelLate;
+  ED_TRY(waits);
   double t_gram = 0.0;
   float t_all = 0.f;
   for (size_t bi = 0; bi < nb; ++bi) {
@@ -441,4 +445,13 @@ extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, doub
     *entropy = s;
   }
   return ED_OK;
+}
+
+extern "C" ed_status ed_entanglement_spectrum(ed_ctx* c, const double* psi, double* lambda, int64_t cap,
+                                              int64_t* n_lambda, double* weight, double* entropy, double* stage_ms,
+                                              void* stream) {
+  bool late = false;
+  const ed_status s = spectrum(c, psi, lambda, cap, n_lambda, weight, entropy, stage_ms, stream, true, &late);
+  // other work held SMs for seconds: once more, with kernels that do not wait
+  return late ? spectrum(c, psi, lambda, cap, n_lambda, weight, entropy, stage_ms, stream, false, &late) : s;
 }

@@ -207,7 +207,11 @@ __global__ void __launch_bounds__(kStepThreads, 1)
   const long long step = (long long)gridDim.x * kStepThreads;
   const T bt = use_beta ? (T)beta[0] : (T)0;
   unsigned gen = 0;
-  if (!CL && tid == 0) gen = *(volatile unsigned*)(bar + 1);  // it moves only after this CTA has arrived
+  bool late = false;  // a wait of an earlier step ran out: its barrier's state is not to be relied on
+  if (!CL && tid == 0) {
+    gen = *(volatile unsigned*)(bar + 1);  // it moves only after this CTA has arrived
+    late = *(volatile int*)err != 0;
+  }
   int phase = 0;
   // the grid's sum of s (thread 0's) and largest em; publish: thread 0 of the last CTA
   auto grid_sum = [&](double s, int em, auto publish) -> bool {
@@ -236,8 +240,8 @@ __global__ void __launch_bounds__(kStepThreads, 1)
       part[blockIdx.x] = s;
       if constexpr (FIX) epart[blockIdx.x] = em;
       __threadfence();
-      s_last = atomicAdd(bar, 1u) == gridDim.x - 1 ? 1u : 0u;
-      s_ok = 1;
+      s_last = !late && atomicAdd(bar, 1u) == gridDim.x - 1 ? 1u : 0u;
+      s_ok = late ? 0 : 1;
       s_em = 0;
     }
     __syncthreads();
@@ -256,7 +260,7 @@ __global__ void __launch_bounds__(kStepThreads, 1)
         __threadfence();
         asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(bar + 1), "r"(gen + 1u) : "memory");
       }
-    } else if (tid == 0) {
+    } else if (tid == 0 && !late) {
       unsigned g = gen;
       for (long long i = 0; i < kStepSpin && g == gen; ++i)
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(bar + 1) : "memory");

@@ -129,12 +129,14 @@ ed_status tmap_8b_2d(CUtensorMap* m, const void* base, long long cols, long long
   return ED_OK;
 }
 
-ed_status oz_status(OzContext* o, cudaStream_t st) {
+ed_status oz_status(OzContext* o, cudaStream_t st, int* code) {
+  if (code) *code = 0;
   if (!o->d_err) return ED_OK;
   int h = 0;
   ED_CUDA_TRY(cudaMemcpyAsync(&h, o->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   ED_CUDA_TRY(cudaStreamSynchronize(st));
   if (h != 0) {
+    if (code) *code = h;
     ED_CUDA_TRY(cudaMemsetAsync(o->d_err, 0, sizeof(int), st));
     set_error("a tensor-core kernel's wait for its operands ran out (code %d)", h);
     return ED_ECUDA;

@@ -77,7 +77,7 @@ ed_status tmap_8b_2d(CUtensorMap* m, const void* base, long long cols, long long
                      int box_rows);
 // reads and clears the flag that the tensor-core kernels set when one of
 // their bounded waits ran out (synchronises the stream); ED_ECUDA if set
-ed_status oz_status(OzContext* o, cudaStream_t st);
+ed_status oz_status(OzContext* o, cudaStream_t st, int* code = nullptr);
 // operand from a host FP64 row-major matrix (digits formed on the host)
 ed_status oz_operand_host(OzContext* o, const double* h, int R, int K, bool a_role, OzOperand* out);
 // operand buffers filled on the device by oz_slice_* (no data yet)

@@ -4,7 +4,8 @@ of a kernel is an attribute of the function, not of a launch: contexts of differ
 width must set the same value, or one thread's value comes between another's and
 its launch.  A launch whose CTAs must all be resident may be refused (part of the
 GPU given to others): Lanczos steps and entanglement spectra then take the kernels
-that need no such thing."""
+that need no such thing, and so they do when such a launch's wait for its CTAs ran
+out (the shim sets the flag that the kernel sets then, and launches nothing)."""
 import os
 import subprocess
 import sys
@@ -110,15 +111,28 @@ print("OUT", json.dumps(out))
 """
 
 
-def test_refused_cooperative_launch(tmp_path):
+LATE = REFUSE.replace("""      fprintf(stderr, "REFUSED\\n");
+      return cudaErrorCooperativeLaunchTooLarge;
+""", """      /* the error flag is the last parameter: of the step (no dynamic shared memory) the 17th, of the panel the 12th */
+      static int seen[2];
+      const int panel = cfg->dynamicSmemBytes > 0;
+      if (seen[panel]++ != 3) continue;
+      fprintf(stderr, "LATE %d\\n", panel);
+      return cudaMemsetAsync(*(void**)args[panel ? 11 : 16], 4, 1, cfg->stream);
+""")
+
+
+@pytest.mark.parametrize("what", ["REFUSED", "LATE"])
+def test_cooperative_launch(tmp_path, what):
     import json
 
     import numpy as np
 
     inc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
-    shims = (REFUSE, REFUSE.replace(" && cfg->attrs[i].val", " && 0 && cfg->attrs[i].val"))  # the second refuses none
-    rs = [_child(tmp_path, shim, RUN, inc) for shim in shims]
-    assert rs[0].stderr.count("REFUSED") >= 4 and "REFUSED" not in rs[1].stderr
+    shim = REFUSE if what == "REFUSED" else LATE
+    shims = (shim, shim.replace(" && cfg->attrs[i].val", " && 0 && cfg->attrs[i].val"))  # the second passes all on
+    rs = [_child(tmp_path, x, RUN, inc) for x in shims]
+    assert rs[0].stderr.count(what) >= (4 if what == "REFUSED" else 2) and what not in rs[1].stderr
     runs = [json.loads(r.stdout.split("OUT", 1)[1]) for r in rs]
     for mode, tol in (("f64", 1e-11), ("f32", 2e-5)):  # as in test_gpu_lanczos_step
         (a, b), (a0, b0) = (np.array(r[mode]) for r in runs)
