@@ -511,7 +511,6 @@ static P3 make_p3(const ed_ctx* c) {
   P3 p;
   p.t = c->t3;
   p.blocks = c->d_blocks;
-  p.cross = c->d_cross;
   p.nblk = (int)c->blocks.size();
   p.ncross = c->kind == ED_SPIN ? (int)c->cross.size() : 0;
   p.xd = nullptr;

@@ -14,7 +14,6 @@ namespace edk {
 struct P3 {
   Dev3 t;
   const DevBlock* blocks;
-  const DevCross* cross;
   int nblk;
   int ncross;
   const double* xd;  // FP64 input of a split diagonal (PI64S)

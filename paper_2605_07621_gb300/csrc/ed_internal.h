@@ -198,7 +198,6 @@ struct Dev3 {
   float dc0_32;
   double dc0_64;
   long long dc0_I;
-  unsigned cross_cls_mask[kMaxCls];  // cross bonds (bit k) with off-diagonal class c
   int q_shift;              // values * 2^q_shift are integers (fixed-point path)
   int P;                    // fraction bits of the fixed-point vector
   // side-B lists of the row pass, in slabs of 32 columns: per slab the first
@@ -207,8 +206,6 @@ struct Dev3 {
   // indices of the slab's column l (past its end the zero slots d_B .. d_B + 7)
   const uint2* B_slab;      // x: first pair row, y: per-class pair rows (8 bits each)
   const unsigned* B_pair;
-  int n_ib;
-  int n_ia;
   // cross terms of the row pass (xs_ok: the cross bonds take at most two
   // value classes).  The bonds are dealt to "sites", each one B cross site
   // with at most two bonds of the first class (slots 0, 1) and two of the
@@ -222,8 +219,6 @@ struct Dev3 {
   const unsigned* A_xs;     // [n_oct][A_total] A-side bit of each slot's bond
   const unsigned* B_xs;     // [n_oct][B_total] B-side bit of each slot's bond
   const uint4* B_xmap;      // [n_oct][B_total] eight 16-bit column maps
-  unsigned ib_mask[32];
-  unsigned ia_mask[32];     // bonds (bits) whose A site is ia
   unsigned char bond_ib[32];
   unsigned char bond_ia[32];
   float bond_w32[32];

@@ -368,14 +368,6 @@ __global__ void k_axpy(const TI* __restrict__ x, TO* __restrict__ y, double s, l
     y[i] = (TO)((double)y[i] + s * (double)x[i]);
 }
 
-// y[i] += s[0] * x[i], s read on the device (reorthogonalisation)
-template <typename TI, typename TO>
-__global__ void k_axpy_dev(const TI* __restrict__ x, TO* __restrict__ y, const double* s, double sign, long long n) {
-  const double c = sign * s[0];
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = (TO)((double)y[i] + c * (double)x[i]);
-}
-
 __device__ __forceinline__ double to_d(double v) { return v; }
 __device__ __forceinline__ double to_d(float v) { return (double)v; }
 __device__ __forceinline__ double to_d(__nv_bfloat16 v) { return (double)__bfloat162float(v); }
@@ -853,10 +845,6 @@ void launch_cvt(ed_ctx* c, const TI* x, TO* y, long long n, cudaStream_t st) {
   k_cvt<TI, TO><<<grid_for(c, n), kRedThreads, 0, st>>>(x, y, n);
 }
 template <typename T>
-void launch_axpy_dev(ed_ctx* c, const T* x, T* y, const double* s, double sign, long long n, cudaStream_t st) {
-  k_axpy_dev<T, T><<<grid_for(c, n), kRedThreads, 0, st>>>(x, y, s, sign, n);
-}
-template <typename T>
 void launch_reorth(ed_ctx* c, const T* V, long long ldv, int m, T* w, long long n, double* h, cudaStream_t st) {
   if (m <= 0) return;
   int chunks = std::max(1, std::min(kMaxPartials / m, (int)((n + kRedThreads - 1) / kRedThreads)));
@@ -886,8 +874,7 @@ void launch_fermion_remap(ed_ctx* c, const double* psi, long long dA_src, long l
   template void launch_lz_c<T>(ed_ctx*, const T*, T*, long long, cudaStream_t);                        \
   template ed_status launch_lz_step<T>(ed_ctx*, const T*, const T*, const T*, T*, int, long long, bool, double*, int*, cudaStream_t); \
   template void launch_lz_rerun<T>(ed_ctx*, const T*, const T*, const T*, double, double, double, T*,   \
-                                   long long, cudaStream_t);                                            \
-  template void launch_axpy_dev<T>(ed_ctx*, const T*, T*, const double*, double, long long, cudaStream_t);
+                                   long long, cudaStream_t);
 ED_INST(double)
 ED_INST(float)
 template void launch_scale_cvt<double, double>(ed_ctx*, const double*, double*, double, long long, cudaStream_t);

@@ -68,8 +68,6 @@ constexpr int kMaxChunks = 64;
 ed_status launch_combine_f32(ed_ctx* c, void* const* chunks, int nchunks, int per, long long n, const double* s, int m,
                              double* x, cudaStream_t st);
 template <typename T>
-void launch_axpy_dev(ed_ctx* c, const T* x, T* y, const double* s, double sign, long long n, cudaStream_t st);
-template <typename T>
 void launch_reorth(ed_ctx* c, const T* V, long long ldv, int m, T* w, long long n, double* h, cudaStream_t st);
 // FP64, twice over (reorth.cu), and the norm of the result to slot 1 (which
 // holds the norm of w before).  F: FP32 copy of the basis, rows of fp32_ld(n)

@@ -284,16 +284,11 @@ static ed_status build_v3(ed_ctx* c, const HostSideOps& ha, const HostSideOps& h
   for (size_t k = 0; k < c->cross.size(); ++k) {
     int ci = (int)(std::find(cls.begin(), cls.end(), c->cross[k].coef) - cls.begin());
     c->cross_cls[k] = ci;
-    t.cross_cls_mask[ci] |= 1u << k;
-    t.ib_mask[c->cross[k].ib] |= 1u << k;
-    t.ia_mask[c->cross[k].ia] |= 1u << k;
     t.bond_ia[k] = (unsigned char)c->cross[k].ia;
     t.bond_ib[k] = (unsigned char)c->cross[k].ib;
     t.bond_w64[k] = c->cross[k].coef;
     t.bond_w32[k] = (float)c->cross[k].coef;
   }
-  t.n_ib = (int)c->crossB_bits.size();
-  t.n_ia = (int)c->crossA_bits.size();
   // slots of the row pass's cross terms: each B cross site's bonds by value
   // class, two per class and site entry, as many entries as it needs
   std::vector<int> xs_site;  // B cross site of each entry
@@ -305,7 +300,7 @@ static ed_status build_v3(ed_ctx* c, const HostSideOps& ha, const HostSideOps& h
     t.xl_c[0] = cc.empty() ? 0 : cc[0];
     t.xl_c[1] = cc.size() > 1 ? cc[1] : t.xl_c[0];
     for (unsigned char& k : t.xs_k) k = 255;
-    for (int ib = 0; t.xs_ok && ib < t.n_ib; ++ib) {
+    for (int ib = 0; t.xs_ok && ib < (int)c->crossB_bits.size(); ++ib) {
       std::vector<int> b[2];
       for (int k = 0; k < (int)c->cross.size(); ++k)
         if (c->cross[k].ib == ib) b[c->cross_cls[k] == t.xl_c[0] ? 0 : 1].push_back(k);
