@@ -322,11 +322,8 @@ size_t h_piece_bytes(const HostTables& h) {
   return align256((size_t)3 * h.dA * pad64(h.dA) * 2) + align256((size_t)3 * h.dB * pad64(h.dB) * 2) +
          align256(kmask_words(h) * 4);
 }
-// the pieces of Psi, and as much again for a transposed copy, which the
-// products no longer need: the sizes by which an engine admits instances stay
-size_t x_piece_bytes(const HostTables& h) {
-  return align256((size_t)3 * h.dA * pad64(h.dB) * 2) + align256((size_t)3 * h.dB * pad64(h.dA) * 2);
-}
+// the pieces of Psi
+size_t x_piece_bytes(const HostTables& h) { return align256((size_t)3 * h.dA * pad64(h.dB) * 2); }
 size_t tables_bytes(const HostTables& h, bool dense) {
   size_t b = align256((size_t)3 * h.dA * h.dB * 4) + csr_bytes(h);
   if (dense && dense_capable(h)) b += h_piece_bytes(h) + x_piece_bytes(h);
