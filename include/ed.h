@@ -269,7 +269,10 @@ ed_status ed_tridiag_eigenvalues(const double* d, const double* e, int64_t n, do
  *   delta    per cross term, nonzero
  *   Lm, Rm   host pointers [m * nq + q]: chi_{q+delta} x chi_q row-major for
  *            the source blocks q with q + delta inside 0..nq-1, NULL otherwise
- * The matrices are copied to the device; the caller keeps its own.
+ * The matrices are copied to the device; the caller keeps its own.  Device
+ * memory: 16 bytes per element of every H_L, H_R, L_m, R_m and product
+ * L_m Psi, 32 per state and 8 more per element of every L_m Psi (the products
+ * of all cross terms are held at once).
  * ed_dense_apply: x, y device FP64 vectors of ed_dense_dim elements, not
  * overlapping; asynchronous on the stream.  One operator holds one scratch
  * buffer for its partial products: applies of the same operator must not

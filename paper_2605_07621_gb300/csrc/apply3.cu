@@ -130,8 +130,8 @@ __device__ __forceinline__ float ldg_if(const float* p, bool on) { return on ? _
 //    gathers of a site before their sums, one weight per value class and
 //    column;
 //  * the diagonal from per-row constants and popcounts of packed words.
-// Bound: the L1 / shared-memory data path (74 % of its wavefronts on the 4x4
-// Hubbard torus, 64 % with cross terms), then issue (60 %).  A 16-byte access
+// Bound: the L1 / shared-memory data path (69 % of its wavefronts on J1-J2 4x7),
+// then issue (63 %).  A 16-byte access
 // takes four wavefronts at best; the lists are ordered so that it takes 4.06
 // (order_lists).  Measured, FP64 fixed point / FP32: J1-J2 4x8 (601 M states)
 // 22.9 -> 16.4 / 14.3 -> 9.2 ms, Hubbard 4x4 (166 M states) 2.75 -> 1.63 /
@@ -392,7 +392,7 @@ constexpr int kPanelCtas = 3;  // resident CTAs of the panel pass per SM
 // per item, started in item order, keeps every SM on the same one or two
 // panels; a persistent grid drifts apart over many panels and loses the L2
 // residency (J1-J2 4x8: 17 ms).
-// Bound: latency of L2 (52 % of its throughput) and issue (57 %).  Measured,
+// Bound: latency of L2 (56 % of its throughput) and issue (53 %).  Measured,
 // FP64 fixed point / FP32: J1-J2 4x8 (601 M states) 9.8 -> 7.8 / 5.4 -> 4.1 ms,
 // Hubbard 4x4 (166 M states) 2.04 -> 1.65 / 1.16 -> 0.84 ms against one row and
 // 256 columns per warp with per-entry index loads and 64-bit offsets.  Runs of
